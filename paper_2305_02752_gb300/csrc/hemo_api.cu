@@ -111,8 +111,6 @@ int coprime_stride(int n) {
 void hemo::set_last_error(const char *msg) { g_err = msg; }
 
 // device buffers of the reverse sweep (grown on demand, kept for reuse)
-constexpr size_t TILE_NODES3 = (size_t)(BLK + 3) * (BLK + 3) * (BLK + 3);  // nodes of a bin's spreading tile
-
 struct AdjBuffers {
     void *lamf_in = nullptr, *lamf_out = nullptr, *lamu = nullptr, *lamF = nullptr, *amom = nullptr;
     void *lamX = nullptr, *lamFv = nullptr, *grad = nullptr;
@@ -432,7 +430,7 @@ void enqueue_step(hemo_sim *s, const View<R> &v, int parity, int force, cudaStre
     View<R> vc = v;  // the spreading tiles are dead once F is gathered
     if (s->ncell) {
         vc.dead = s->tiles;
-        vc.dead_lines = (long long)(rsize(s) * 3 * (size_t)TILE_NODES3 * s->nbins / 128);
+        vc.dead_lines = (long long)(rsize(s) * 3 * (size_t)SPREAD_NODES * s->nbins / 128);
     }
     launch_collide<R>(vc, s->precision, parity, st);  // BGK + Guo force + AA streaming
     mark(HEMO_PHASE_MOMENTS);
@@ -467,7 +465,7 @@ int finalize_impl(hemo_sim *s) {
     s->counts = (int *)dalloc(s, sizeof(int) * (s->nbins + 1));
     s->cursor = (int *)dalloc(s, sizeof(int) * (s->nbins + 1));
     s->start = (int *)dalloc(s, sizeof(int) * (s->nbins + 2));
-    s->tiles = dalloc(s, rs * 3 * TILE_NODES3 * s->nbins);
+    s->tiles = dalloc(s, rs * 3 * (size_t)SPREAD_NODES * s->nbins);
     s->Uprev = dalloc(s, rs * 3 * std::max(nv, 1));
     s->csp = dalloc(s, rs * 6 * std::max(nc, 1));
     if (!s->tiles || !s->Uprev || !s->csp || !s->ctr || !s->off || !s->Fv || !s->vcell_d || !s->cell_first_d || !s->cell_type_d || !s->meshes_d ||

@@ -13,6 +13,9 @@ namespace hemo {
 constexpr int Q = 19;
 constexpr int BLK = 8;              // lattice block edge used for vertex bins
 constexpr int MAX_TYPES = 8;        // membrane mesh types per simulation
+// A bin's (BLK + 3)^3 spreading tile, [component][z][y][x]: rows padded to 12
+// nodes and planes to 136 (8 mod 32: see spread_tile_f32_kernel)
+constexpr int SPREAD_PITCH = 12, SPREAD_PLANE = 136, SPREAD_NODES = SPREAD_PLANE * (BLK + 3);
 
 // status bits raised on the device
 constexpr unsigned ST_NUMERIC = 1u;
@@ -159,7 +162,7 @@ template <typename R> struct View {
     int *perm;                 // nv, stable (key, vertex id)
     int *anc_i;                // nv*3 stencil base floor(X) (wrapped on periodic axes)
     R *anc_t;                  // nv*3 fractions X - floor(X)
-    R *tiles;                  // nbins*3*11^3 per-bin spreading tiles
+    R *tiles;                  // nbins*3*SPREAD_NODES per-bin spreading tiles
     // vertex integrator (Sec. 2.6): 0 Euler X += U; 1 Euler and U kept in
     // Uprev; 2 Adams-Bashforth X += 3/2 U - 1/2 Uprev and U kept in Uprev
     int integ;

@@ -41,6 +41,10 @@ __device__ __forceinline__ double sqrt_r(double a) { return sqrt(a); }
 
 constexpr int TILE = BLK + 3;           // stencil reach: one node below, two above
 constexpr int TILE3 = TILE * TILE * TILE;
+// strides of a bin's spreading tile, in memory as in the FP32 kernel's shared
+// memory
+constexpr int TP_Y = SPREAD_PITCH, TP_Z = SPREAD_PLANE, TP_N = SPREAD_NODES;
+__device__ __forceinline__ int tile_index(int x, int y, int z) { return x + TP_Y * y + TP_Z * z; }
 // Padded shared-memory strides of an 11^3 tile: the 16 lanes (b, c) of a
 // half-warp address rows TS_Y*b + TS_Z*c, which fall in 16 distinct banks
 // (TS_Y = 12, TS_Z = 161 = 1 mod 32).
@@ -319,20 +323,19 @@ __device__ __forceinline__ void stage_chunk(const View<R> &v, int p0, int n, con
     }
 }
 
-// Phase 1 of spreading: one CTA per non-empty bin; a warp takes two
-// vertices, each half-warp's 16 lanes own one (y, z) row of the 4x4x4
-// stencil and add four x-neighbours into the bin's 11^3 shared tile.  The
-// tile is written out whole (compact [3][11^3]) for the owners to gather.
+// Phase 1 of spreading: one CTA per non-empty bin adds the 4x4x4 stencils of
+// the bin's vertices into an 11^3 shared tile, which is written out whole for
+// the owners to gather.
 //
-// The tile accumulates in fixed point with integer shared atomics (native,
-// unaffected by address collisions, and exact: the sums do not depend on the
-// order of the vertices, so every run gives the same bits).  FP32: 32-bit
-// integers; per bin and component the scale is the power of two 2^e with
-// e = 30 - ceil(log2(max|F| * n / 8)): a node's sum is at most max|F| times
-// the sum of its n weights, each at most 1/8, so |sum| * 2^e <= 2^30, and
-// the quantum, max|F| * n * 2^-33 per contribution, is below the FP32
-// rounding of sums of that size.  FP64: 64-bit integers with 2^62 in place
-// of 2^30 (quantum max|F| n 2^-65, below FP64 rounding).
+// The tile accumulates in fixed point with integer shared atomics (native and
+// exact: the sums do not depend on the order of the vertices, so every run
+// gives the same bits).  FP32: 32-bit integers; per bin and component the
+// scale is the power of two 2^e with e = 30 - ceil(log2(max|F| * n / 8)): a
+// node's sum is at most max|F| times the sum of its n weights, each at most
+// 1/8, so |sum| * 2^e <= 2^30, and the quantum, max|F| * n * 2^-33 per
+// contribution, is below the FP32 rounding of sums of that size.  FP64:
+// 64-bit integers with 2^62 in place of 2^30 (quantum max|F| n 2^-65, below
+// FP64 rounding).
 template <typename R> struct TileAcc {
     using T = long long;
     static constexpr int E = 61;  // log2 of the bound minus one
@@ -341,11 +344,258 @@ template <> struct TileAcc<float> {
     using T = int;
     static constexpr int E = 29;
 };
-__device__ __forceinline__ int fixed_of(float x) { return __float2int_rn(x); }
 __device__ __forceinline__ long long fixed_of(double x) { return __double2ll_rn(x); }
 
+// the scale of a component from its largest force; 0 (and the numeric
+// status) for forces that are not finite
 template <typename R>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 6 : 1) spread_tile_kernel(View<R> v) {
+__device__ __forceinline__ R tile_scale(R fmax_abs, int n, unsigned *status) {
+    const R bound = fmax_abs * R(n) * R(0.125);
+    if (!(bound <= R(3.0e38))) {
+        atomicOr(status, ST_NUMERIC);
+        return R(0);
+    }
+    return bound > R(0) ? ldexp(R(1), min(TileAcc<R>::E - ilogb(bound), 120)) : R(0);
+}
+
+// FP32.  Two lanes per vertex, lane h adding the stencil's x nodes 2h and
+// 2h + 1 (96 contributions each).  The shared atomics run at one warp
+// instruction per cycle when the 32 lanes fall in 32 distinct banks, and cost
+// a cycle more per collision.  The tile's z stride is 8 (mod 32) banks, so a
+// lane that walks its four z layers starting from layer s instead of 0 sits 8 s
+// banks further in every instruction (8 * 4 = 32: the walk wraps around with
+// the banks).  An item (vertex, h) whose first position is in bank class c =
+// (row + 2h) mod 8 can therefore take any of the four lanes of its class (bank c +
+// 8m in lane 4c + m).  The bin's
+// vertices are sorted by row mod 8 in shared memory, and each row of 32 lanes
+// takes four items of each class: conflict-free, with as many rows as the
+// fullest class needs (22 % more than a perfect balance on the pipe: 7.3
+// atomic cycles per vertex instead of 6; the FP64 kernel's half-warp per
+// vertex has two vertices collide, 11.8).  Integer sums do not depend on
+// the order, so the walk and the sort leave the bits alone.
+//
+// Rounding to the fixed-point grid: half of the contributions by a conversion
+// (F2I runs at 16 lanes per cycle, and all of them would take twice as long as
+// the atomics), half without one: a magnitude c <= 2^24 quanta times 2^-149,
+// the smallest denormal, is rounded to the nearest quantum by that
+// multiplication, and the bits of the product are the integer (the bits of
+// denormals and of the first normal binade count in quanta), the same integer
+// as the conversion's.  A contribution is at most 2^30 / n quanta, so bins of at
+// least 64 vertices qualify; smaller bins convert, and so does a row of lanes
+// with a weight below zero (one that vanishes, rounded), whose contributions
+// do not have the forces' signs.
+//
+// Bound by the shared-memory pipe (75 % busy) and by issue (78 %).  128 x 128 x
+// 512 vessel (2.9 M vertices in 14.7 k bins): 242 -> 193 us; the spreading
+// phase of the 1000 x 208 x 208 pipe (12.6 M vertices in 54 k bins) 1429 -> 1236
+// us (all converted: 1347 with the gather's six CTAs per SM, where half takes
+// 1287 and none 1303).  Six CTAs per SM: seven spill.
+constexpr int SP_Y = TP_Y, SP_Z = TP_Z, SP_N = TP_N;  // the shared tile
+static_assert(SP_Z % 32 == 8 && SP_Y % 8 == 4, "bank classes of the spreading tile");
+constexpr int NO_SCALE = -1000;
+constexpr int SP_CHUNK = 256;      // vertices sorted at a time, one per thread
+constexpr int SP_GRID_MIN = 64;    // fewest vertices of a bin on the denormal grid
+constexpr int SP_CONVERT = 12;     // of 24 contributions per layer, those converted there
+struct SpreadStage {
+    float4 a[SP_CHUNK];  // tx, qx, ty, qy: fraction and sqrt(1 + 4t - 4t^2) per axis
+    float4 b[SP_CHUNK];  // tz, qz, F_x, F_y (forces scaled)
+    float2 c[SP_CHUNK];  // F_z, tile row (as int)
+};
+
+// i = -i for four values if c != 0, as predicated instructions
+__device__ __forceinline__ void negate_if(int c, int &i, int &j, int &k, int &l) {
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %4, 0;\n\t"
+        "@p neg.s32 %0, %0;\n\t@p neg.s32 %1, %1;\n\t@p neg.s32 %2, %2;\n\t@p neg.s32 %3, %3;\n\t}"
+        : "+r"(i), "+r"(j), "+r"(k), "+r"(l)
+        : "r"(c));
+}
+
+// the contributions of an item: forces F, weights (2 w per axis), its first
+// position in the tile and its walk's first z layer s; GRID: SP_CONVERT of the
+// 24 contributions per layer are converted, the others land on the denormal
+// grid; otherwise all are converted
+template <bool GRID>
+__device__ __forceinline__ void spread_item(int *first, int s, const float (&F)[3], const float (&wx)[2],
+                                            const float (&wy)[4], const float (&wz)[4]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        int *const pj = first + SP_Z * ((j + s) & 3);
+        float wyz[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) wyz[b] = wy[b] * wz[j];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+#pragma unroll
+            for (int b = 0; b < 4; b += 2) {
+                const bool conv = !GRID || 8 * d + 2 * b < SP_CONVERT;
+                const float Fd = conv ? F[d] : fabsf(F[d]), f0 = Fd * wyz[b], f1 = Fd * wyz[b + 1];
+                const float c[4] = {f0 * wx[0], f0 * wx[1], f1 * wx[0], f1 * wx[1]};
+                int i[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) i[q] = conv ? __float2int_rn(c[q]) : __float_as_int(c[q] * 0x1p-149f);
+                if (!conv) negate_if(F[d] < 0.f, i[0], i[1], i[2], i[3]);
+                int *const p = pj + d * SP_N + SP_Y * b;
+                atomicAdd(p, i[0]);
+                atomicAdd(p + 1, i[1]);
+                atomicAdd(p + SP_Y, i[2]);
+                atomicAdd(p + SP_Y + 1, i[3]);
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(SP_CHUNK, 6) spread_tile_f32_kernel(View<float> v) {
+    const int k = blockIdx.x;
+    const int s = v.start[k], e = v.start[k + 1], n = e - s;
+    if (n == 0) return;
+    __shared__ __align__(16) int tile[3 * SP_N];
+    __shared__ SpreadStage st;
+    __shared__ float smax[24];  // [component][warp]
+    __shared__ __align__(16) int count[8];  // vertices of the chunk per row mod 8
+    constexpr int NW = SP_CHUNK / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int q = tid; q < 3 * SP_N / 4; q += SP_CHUNK) reinterpret_cast<int4 *>(tile)[q] = make_int4(0, 0, 0, 0);
+    if (tid < 8) count[tid] = 0;
+    int org[3];
+    bin_origin(v, k, org);
+    // chunks of equal size
+    const int nch = (n + SP_CHUNK - 1) / SP_CHUNK, csz = (n + nch - 1) / nch;
+    // a vertex's record; row -1 outside the bin (domain status already raised)
+    auto load = [&](int j, float t[3], float F[3]) -> int {
+        const int i = v.perm[j];
+        if (!index_ok(i >= 0 && i < v.nv, v.status)) return -1;
+        int row = 0;
+        bool ok = true;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int b = v.anc_i[3 * (size_t)i + d] - org[d];
+            ok &= b >= 0 && b < BLK;
+            row += b * (d == 0 ? 1 : (d == 1 ? SP_Y : SP_Z));
+            t[d] = v.anc_t[3 * (size_t)i + d];
+            F[d] = v.Fv[3 * (size_t)i + d];
+        }
+        return ok ? row : -1;
+    };
+    // the first chunk's records, and one scale per component for the whole bin
+    float t[3] = {0.f, 0.f, 0.f}, F[3] = {0.f, 0.f, 0.f};
+    int row = tid < csz ? load(s + tid, t, F) : -1;
+    unsigned m[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) m[d] = __float_as_uint(fabsf(F[d]));  // (order as the floats, NaN above all)
+    for (int j = s + csz + tid; j < e; j += SP_CHUNK) {
+        const int i = v.perm[j];
+        if (!index_ok(i >= 0 && i < v.nv, v.status)) continue;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) m[d] = max(m[d], __float_as_uint(fabsf(v.Fv[3 * (size_t)i + d])));
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        m[d] = __reduce_max_sync(0xffffffffu, m[d]);
+        if (lane == 0) smax[d * NW + warp] = __uint_as_float(m[d]);
+    }
+    __syncthreads();
+    int ex[3];  // the scales' exponents; NO_SCALE: no force, or one that is not finite
+    {
+        unsigned mm = lane < 3 * NW ? __float_as_uint(smax[lane]) : 0u;
+#pragma unroll
+        for (int o = 1; o < NW; o <<= 1) mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+        const float bound = __uint_as_float(mm) * (float)n * 0.125f;
+        int x = min(TileAcc<float>::E + 127 - (int)(__float_as_uint(bound) >> 23), 120);
+        if (!(bound <= 3.0e38f)) {
+            if (tid < 3 * NW) atomicOr(v.status, ST_NUMERIC);
+            x = NO_SCALE;
+        }
+        if (bound == 0.f) x = NO_SCALE;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) ex[d] = __shfl_sync(0xffffffffu, x, NW * d);
+    }
+    auto pow2 = [](int x) { return x == NO_SCALE ? 0.f : __int_as_float((x + 127) << 23); };
+    const bool grid = n >= SP_GRID_MIN;
+    const float scale[3] = {pow2(ex[0]) * 0.125f, pow2(ex[1]) * 0.125f, pow2(ex[2]) * 0.125f};  // (2 w per axis)
+    for (int p = s; p < e; p += csz) {
+        if (p != s) {
+            __syncthreads();  // the previous chunk is done with the stage
+            if (tid < 8) count[tid] = 0;
+            row = tid < csz && p + tid < e ? load(p + tid, t, F) : -1;
+            __syncthreads();
+        }
+        // sort by row mod 8: the lanes of a class count together
+        unsigned peers = __ballot_sync(0xffffffffu, row >= 0);
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+            const unsigned bal = __ballot_sync(0xffffffffu, row & o);
+            peers &= row & o ? bal : ~bal;
+        }
+        const int leader = __ffs(peers) - 1;
+        int rank = 0;
+        if (row >= 0 && lane == leader) rank = atomicAdd(count + (row & 7), __popc(peers));
+        rank = __shfl_sync(0xffffffffu, rank, leader & 31) + __popc(peers & ((1u << lane) - 1u));
+        __syncthreads();
+        // lanes 4c .. 4c + 3 serve class c: its count and first position
+        const int n0 = count[lane >> 2];
+        int f0 = n0;
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, f0, o);
+            if (lane >= o) f0 += x;
+        }
+        f0 -= n0;
+        const int n1 = __shfl_sync(0xffffffffu, n0, lane + 24), f1 = __shfl_sync(0xffffffffu, f0, lane + 24);  // class c - 2
+        const int rows = (__reduce_max_sync(0xffffffffu, n0 + n1) + 3) >> 2;
+        const int at = __shfl_sync(0xffffffffu, f0, 4 * (row & 7)) + rank;
+        if (row >= 0) {
+            float r[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) r[d] = sqrtf(1.f + 4.f * t[d] - 4.f * t[d] * t[d]);
+            st.a[at] = make_float4(t[0], r[0], t[1], r[1]);
+            st.b[at] = make_float4(t[2], r[2], F[0] * scale[0], F[1] * scale[1]);
+            st.c[at] = make_float2(F[2] * scale[2], __int_as_float(row));
+        }
+        __syncthreads();
+        // the items of this lane's class c: half 0 of the vertices of class c,
+        // then half 1 of those of class c - 2
+        for (int i = warp; i < rows; i += NW) {
+            const int it = 4 * i + (lane & 3);
+            const bool on = it < n0 + n1;
+            const int h = on && it >= n0, q = on ? (h ? f1 + it - n0 : f0 + it) : 0;
+            const float4 A = st.a[q], B = st.b[q];
+            const float2 C = st.c[q];
+            const int pos = __float_as_int(C.y) + 2 * h;  // position of the item's first node
+            const int z0 = (lane - (pos >> 3)) & 3;
+            // 2 w = (3 - 2t - q, 3 - 2t + q, 1 + 2t + q, 1 + 2t - q) / 4 per axis
+            const float ux = h ? fmaf(.5f, A.x, .25f) : fmaf(-.5f, A.x, .75f), gx = h ? -.25f : .25f;
+            const float wx[2] = {fmaf(-gx, A.y, ux), fmaf(gx, A.y, ux)};
+            const float y0 = fmaf(-.5f, A.z, .75f), y1 = fmaf(.5f, A.z, .25f);
+            const float wy[4] = {fmaf(-.25f, A.w, y0), fmaf(.25f, A.w, y0), fmaf(.25f, A.w, y1), fmaf(-.25f, A.w, y1)};
+            const float u0 = fmaf(-.5f, B.x, .75f), u1 = fmaf(.5f, B.x, .25f);
+            const float v0 = fmaf(-.25f, B.y, u0), v1 = fmaf(.25f, B.y, u0), v2 = fmaf(.25f, B.y, u1), v3 = fmaf(-.25f, B.y, u1);
+            // the z weights in the walk's order
+            const float r0 = z0 & 1 ? v1 : v0, r1 = z0 & 1 ? v2 : v1, r2 = z0 & 1 ? v3 : v2, r3 = z0 & 1 ? v0 : v3;
+            const float wz[4] = {z0 & 2 ? r2 : r0, z0 & 2 ? r3 : r1, z0 & 2 ? r0 : r2, z0 & 2 ? r1 : r3};
+            const float F[3] = {B.z, B.w, C.x};
+            const bool below = fminf(fminf(fminf(wx[0], wx[1]), fminf(wy[0], wy[3])), fminf(v0, v3)) < 0.f;  // (the others are above 1/4)
+            const bool by_grid = grid && !__any_sync(0xffffffffu, on && below);
+            if (!on) continue;
+            if (by_grid) spread_item<true>(tile + pos, z0, F, wx, wy, wz);
+            else spread_item<false>(tile + pos, z0, F, wx, wy, wz);
+        }
+    }
+    __syncthreads();
+    // write-out, four nodes per thread
+    float4 *out = reinterpret_cast<float4 *>(v.tiles + (size_t)k * 3 * SP_N);
+    const float inv[3] = {pow2(ex[0] == NO_SCALE ? NO_SCALE : -ex[0]), pow2(ex[1] == NO_SCALE ? NO_SCALE : -ex[1]),
+                          pow2(ex[2] == NO_SCALE ? NO_SCALE : -ex[2])};
+    for (int q = tid; q < 3 * SP_N / 4; q += SP_CHUNK) {
+        const int4 f = reinterpret_cast<const int4 *>(tile)[q];
+        const float iv = q < SP_N / 4 ? inv[0] : (q < 2 * SP_N / 4 ? inv[1] : inv[2]);
+        out[q] = make_float4((float)f.x * iv, (float)f.y * iv, (float)f.z * iv, (float)f.w * iv);
+    }
+}
+
+// FP64: a warp takes two vertices, each half-warp's 16 lanes own one (y, z) row
+// of the stencil.
+template <typename R>
+__global__ void __launch_bounds__(256) spread_tile_kernel(View<R> v) {
     using A = typename TileAcc<R>::T;
     constexpr int CAP = Stage<R>::CAP;
     const int k = blockIdx.x;
@@ -388,13 +638,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 6 : 1) spread_tile_kerne
         if (threadIdx.x < 3) {
             R mm = R(0);
             for (int w = 0; w < nw; ++w) mm = fmax(mm, smax[threadIdx.x][w]);
-            const R bound = mm * R(e - s) * R(0.125);
-            if (!(bound <= R(3.0e38))) {  // non-finite forces
-                atomicOr(v.status, ST_NUMERIC);
-                scale[threadIdx.x] = R(0);
-            } else {
-                scale[threadIdx.x] = bound > R(0) ? ldexp(R(1), min(TileAcc<R>::E - ilogb(bound), 120)) : R(0);
-            }
+            scale[threadIdx.x] = tile_scale(mm, e - s, v.status);
         }
         __syncthreads();  // the staging below or the loop applies the scale
     }
@@ -422,20 +666,19 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 6 : 1) spread_tile_kerne
                 const R wa = wx[a];
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
-                    if constexpr (sizeof(A) == 4) atomicAdd((int *)&acc[d][row + a], fixed_of(f[d] * wa));
-                    else atomicAdd((unsigned long long *)&acc[d][row + a], (unsigned long long)fixed_of(f[d] * wa));
+                    atomicAdd((unsigned long long *)&acc[d][row + a], (unsigned long long)fixed_of(f[d] * wa));
                 }
             }
         }
     }
     __syncthreads();
-    R *out = v.tiles + (size_t)k * 3 * TILE3;
+    R *out = v.tiles + (size_t)k * 3 * TP_N;
     R inv[3];
     for (int d = 0; d < 3; ++d) inv[d] = scale[d] > R(0) ? R(1) / scale[d] : R(0);  // (exact: powers of two)
     TileWalk tw(threadIdx.x, blockDim.x);
     for (int q = threadIdx.x; q < TILE3; q += blockDim.x, tw.next()) {
         const int sidx = tw.l0 + TS_Y * tw.l1 + TS_Z * tw.l2;
-        for (int d = 0; d < 3; ++d) out[d * TILE3 + q] = (R)acc[d][sidx] * inv[d];
+        for (int d = 0; d < 3; ++d) out[d * TP_N + tile_index(tw.l0, tw.l1, tw.l2)] = (R)acc[d][sidx] * inv[d];
     }
 }
 
@@ -496,11 +739,11 @@ __global__ void __launch_bounds__(256) spread_gather_kernel(View<R> v) {
                 for (int ix = 0; ix < cnt[0][l0]; ++ix) {
                     const int kk = nbin[9 * ent_slot[2][l2][iz] + 3 * ent_slot[1][l1][iy] + ent_slot[0][l0][ix]];
                     if (kk < 0) continue;
-                    const R *tt = v.tiles + (size_t)kk * 3 * TILE3;
-                    const int ti = ent_pos[0][l0][ix] + TILE * (ent_pos[1][l1][iy] + TILE * ent_pos[2][l2][iz]);
+                    const R *tt = v.tiles + (size_t)kk * 3 * TP_N;
+                    const int ti = tile_index(ent_pos[0][l0][ix], ent_pos[1][l1][iy], ent_pos[2][l2][iz]);
                     f0 += tt[ti];
-                    f1 += tt[TILE3 + ti];
-                    f2 += tt[2 * TILE3 + ti];
+                    f1 += tt[TP_N + ti];
+                    f2 += tt[2 * TP_N + ti];
                 }
         const size_t n = (size_t)x + (size_t)v.nx * ((size_t)y + (size_t)v.ny * z);
         const bool wall = !v.spread_all_nodes && (v.ntype[n] & 0x7f);
@@ -516,8 +759,13 @@ __global__ void __launch_bounds__(256) spread_gather_kernel(View<R> v) {
 // eight (positions 1..8) and the upper neighbour's coordinate 7 (position
 // 0).  Each thread owns two nodes and adds, slot by slot in a fixed order,
 // the tile values that land on them.
+//
+// Latency-bound, so many small threads: eight CTAs per SM (32 registers; six:
+// the spreading phase of the pipe 1251 instead of 1236 us).  A thread per
+// component and z column (a third fewer instructions, all loads at constant
+// offsets, 56 registers) took 1384, one per component and node 1814.
 template <typename R>
-__global__ void __launch_bounds__(256) spread_gather3_kernel(View<R> v) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 8 : 1) spread_gather3_kernel(View<R> v) {
     __shared__ int nbin[27];  // bin of slot (sz + 1) * 9 + (sy + 1) * 3 + (sx + 1), -1 if empty or absent
     const int k = blockIdx.x;
     const int bc[3] = {k % v.nb[0], (k / v.nb[0]) % v.nb[1], k / (v.nb[0] * v.nb[1])};
@@ -573,14 +821,14 @@ __global__ void __launch_bounds__(256) spread_gather3_kernel(View<R> v) {
             const bool in = iz < ns[2] && iy < ns[1] && ix < ns[0];
             const int kk = in ? nbin[9 * sl[2][iz] + 3 * sl[1][iy] + sl[0][ix]] : -1;
             on[m] = kk >= 0;
-            src[m] = v.tiles + (size_t)(kk < 0 ? 0 : kk) * 3 * TILE3 + (ps[0][ix] + TILE * (ps[1][iy] + TILE * ps[2][iz]));
+            src[m] = v.tiles + (size_t)(kk < 0 ? 0 : kk) * 3 * TP_N + tile_index(ps[0][ix], ps[1][iy], ps[2][iz]);
         }
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
             if (on[m]) {
                 f0 += src[m][0];
-                f1 += src[m][TILE3];
-                f2 += src[m][2 * TILE3];
+                f1 += src[m][TP_N];
+                f2 += src[m][2 * TP_N];
             }
         }
         const size_t n = (size_t)x + (size_t)v.nx * ((size_t)y + (size_t)v.ny * z);
@@ -1199,7 +1447,8 @@ void launch_bin_ranges(const View<R> &v, cudaStream_t st) {
 
 template <typename R>
 void launch_spread(const View<R> &v, cudaStream_t st) {
-    spread_tile_kernel<R><<<v.nbins, 256, 0, st>>>(v);
+    if constexpr (std::is_same<R, float>::value) spread_tile_f32_kernel<<<v.nbins, SP_CHUNK, 0, st>>>(v);
+    else spread_tile_kernel<R><<<v.nbins, 256, 0, st>>>(v);
     if (v.nb[0] >= 3 && v.nb[1] >= 3 && v.nb[2] >= 3) spread_gather3_kernel<R><<<v.nbins, 256, 0, st>>>(v);
     else spread_gather_kernel<R><<<v.nbins, 256, 0, st>>>(v);
 }
