@@ -154,7 +154,7 @@ struct hemo_sim {
     std::vector<HostMesh> meshes;
     std::vector<int> cell_type, cell_first, vcell;
     std::vector<double> X0;
-    int nv = 0, ncell = 0, max_nv = 0, max_nt = 0, max_ne = 0, nsm = 1;
+    int nv = 0, ncell = 0, max_nv = 0, max_nt = 0, max_ne = 0, nsm = 1, slices = 1;
     bool finalized = false;
     long long steps_done = 0;
     // device cells and bins
@@ -351,6 +351,7 @@ View<R> make_view(hemo_sim *s) {
     v.max_nt = s->max_nt;
     v.max_ne = s->max_ne;
     v.nsm = s->nsm;
+    v.slices = s->slices;
     for (int d = 0; d < 3; ++d) v.nb[d] = s->nb[d];
     v.nbins = s->nbins;
     v.key = s->key;
@@ -477,6 +478,7 @@ int finalize_impl(hemo_sim *s) {
     HEMO_CU(cudaMemsetAsync(s->counts, 0, sizeof(int) * (s->nbins + 1), st));
     HEMO_CU(cudaMemsetAsync(s->Fv, 0, rs * 3 * std::max(nv, 1), st));
 
+    s->slices = cell_slices<R>(nc, s->nsm, cell_smem_bytes<R>(s->max_nv, s->max_nt, s->max_ne));
     // mesh tables
     std::vector<MeshDev<R>> md(MAX_TYPES);
     for (size_t t = 0; t < s->meshes.size(); ++t) {
@@ -600,6 +602,45 @@ int finalize_impl(hemo_sim *s) {
         if (!dAt0) return fail(HEMO_ERR_OOM, "device allocation of mesh tables failed");
         HEMO_CU(cudaMemcpy(dAt0, At0_p.data(), rs * m.nt, cudaMemcpyHostToDevice));
         d.At0 = dAt0;
+        if (s->slices > 1) {
+            // what the fans of each slice's vertices read: their triangles, their
+            // edges and those opposite, and the triangles of all these edges; a
+            // triangle is owned by the slice of its smallest vertex
+            const int S = s->slices, per = (m.nv + S - 1) / S;
+            std::vector<int> items, at(2 * (S + 1));
+            std::vector<std::vector<int>> se(S);
+            for (int r = 0; r < S; ++r) {
+                std::vector<char> tin(m.nt, 0), ein(m.ne, 0);
+                for (int i = std::min(m.nv, r * per); i < std::min(m.nv, (r + 1) * per); ++i)
+                    for (int k = 1; k <= maxv; ++k) {
+                        const int4 g = vfan[(size_t)k * m.nv + i];
+                        if (g.x < 0) break;
+                        tin[g.x] = 1;
+                        ein[g.z >> 1] = ein[g.w] = 1;
+                    }
+                for (int e = 0; e < m.ne; ++e)
+                    if (ein[e]) {
+                        tin[etri_p[2 * (size_t)e]] = tin[etri_p[2 * (size_t)e + 1]] = 1;
+                        se[r].push_back(e);
+                    }
+                at[r] = (int)items.size();
+                for (int t = 0; t < m.nt; ++t) {
+                    const int4 T = tri4[t];
+                    if (tin[t]) items.push_back(t << 1 | (std::min({T.x, T.y, T.z}) / per == r ? 1 : 0));
+                }
+            }
+            at[S] = (int)items.size();
+            for (int r = 0; r <= S; ++r) {
+                at[S + 1 + r] = (int)items.size();
+                if (r < S) items.insert(items.end(), se[r].begin(), se[r].end());
+            }
+            int *ditems = (int *)dalloc(s, sizeof(int) * items.size()), *dat = (int *)dalloc(s, sizeof(int) * at.size());
+            if (!ditems || !dat) return fail(HEMO_ERR_OOM, "device allocation of mesh tables failed");
+            HEMO_CU(cudaMemcpy(ditems, items.data(), sizeof(int) * items.size(), cudaMemcpyHostToDevice));
+            HEMO_CU(cudaMemcpy(dat, at.data(), sizeof(int) * at.size(), cudaMemcpyHostToDevice));
+            d.sl_items = ditems;
+            d.sl_at = dat;
+        }
         d.k_local = R(m.k_local);
         d.thm2i = m.theta_m > 0 ? R(1.0 / (m.theta_m * m.theta_m)) : R(0);
         d.A0 = m.A0;

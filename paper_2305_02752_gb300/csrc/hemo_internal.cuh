@@ -13,6 +13,7 @@ namespace hemo {
 constexpr int Q = 19;
 constexpr int BLK = 8;              // lattice block edge used for vertex bins
 constexpr int MAX_TYPES = 8;        // membrane mesh types per simulation
+constexpr int MAX_SLICES = 16;      // CTAs per cell in the membrane kernel at most
 // A bin's (BLK + 3)^3 spreading tile, [component][z][y][x]: rows padded to 12
 // nodes and planes to 136 (8 mod 32: see spread_tile_f32_kernel)
 constexpr int SPREAD_PITCH = 12, SPREAD_PLANE = 136, SPREAD_NODES = SPREAD_PLANE * (BLK + 3);
@@ -113,6 +114,10 @@ template <typename R> struct MeshDev {
     // (processing order) and local area modulus; 1 / theta_m^2 of the
     // nonlinear bending term
     const R *At0;
+    // clusters of CTAs per cell (View::slices = S > 1): the items of each slice,
+    // triangles as position << 1 | owned, edges as positions; sl_at holds the S + 1
+    // bounds of the slices' triangles, then those of their edges
+    const int *sl_items, *sl_at;
     R k_local;
     R thm2i;
     double A0, V0;
@@ -151,6 +156,7 @@ template <typename R> struct View {
     int max_nt;                // largest triangle count of a mesh type
     int max_ne;                // largest edge count of a mesh type
     int nsm;                   // multiprocessors of the device
+    int slices;                // CTAs per cell in the membrane kernel
     // bins
     int nb[3];
     int nbins;
@@ -268,6 +274,7 @@ void launch_build_links(int nx, int ny, int nz, const int *per, uint8_t *ntype, 
 // mode 1: per-cell statistics into stats (6 per cell), no writes to the state
 template <typename R> void launch_cell_forces(const View<R> &v, int mode, double *stats, cudaStream_t st);
 template <typename R> cudaError_t set_cell_smem_limit(size_t bytes);
+template <typename R> int cell_slices(int ncell, int nsm, size_t smem);
 template <typename R> size_t cell_smem_bytes(int max_nv, int max_nt, int max_ne) {
     return (4 * (size_t)max_nv + 5 * (size_t)max_nt + 4 * (size_t)max_ne) * sizeof(R);
 }

@@ -23,6 +23,8 @@
 #include <algorithm>
 #include <type_traits>
 
+#include <cooperative_groups.h>
+
 #include "hemo_internal.cuh"
 
 namespace hemo {
@@ -178,6 +180,108 @@ template <typename R> __device__ __forceinline__ void st4(R *p, R x, R y, R z, R
     }
 }
 
+// Record of triangle t with corners T: a = n / |n|^2 and |n|, with n = (x1 -
+// x0) x (x2 - x0) (and the local area coefficient); its area |n|/2 and volume
+// x0 . (x1 x x2) / 6.
+template <typename R>
+__device__ __forceinline__ void tri_record(const MeshDev<R> &m, const R *xs, R *tn, R *tl, int t, int4 T, R &area, R &vol) {
+    const V3<R> p0 = xyz(ld4(xs + 4 * T.x)), p1 = xyz(ld4(xs + 4 * T.y)), p2 = xyz(ld4(xs + 4 * T.z));
+    const V3<R> n = cross(p1 - p0, p2 - p0);
+    const R q = dot(n, n), ln = sqrt_r(q), iq = R(1) / q;
+    st4(tn + 4 * t, iq * n.x, iq * n.y, iq * n.z, ln);
+    if (m.k_local > R(0)) {
+        const R a0 = __ldg(m.At0 + t);
+        tl[t] = R(0.5) * m.k_local * (R(0.5) * ln - a0) / a0;
+    }
+    area = R(0.5) * ln;
+    vol = dot(p0, cross(p1, p2)) / R(6);
+}
+
+// Coefficients of edge e: link coefficient s (F on v0 = s (x1 - x0)), cb |e| for
+// the wing vertices, and the lever-rule coefficients cb sa0, cb sb0 of v0
+// (those of v1 are cb sa0 + cb |e| and cb sb0 + cb |e|, since sa1 - sa0 = sb1 -
+// sb0 = |e|); E = (v0, v1, a, b), the edge's triangles T are (v0, v1, a) and
+// (v1, v0, b).
+template <typename R>
+__device__ __forceinline__ void edge_record(const MeshDev<R> &m, const R *xs, const R *tn, R *es, int e, int4 E, int2 T,
+                                            R il0, R th0, unsigned *status) {
+    const V3<R> p0 = xyz(ld4(xs + 4 * E.x)), p1 = xyz(ld4(xs + 4 * E.y));
+    const V3<R> pa = xyz(ld4(xs + 4 * E.z)), pb = xyz(ld4(xs + 4 * E.w));
+    const V3<R> ed = p1 - p0;
+    const R L = sqrt_r(dot(ed, ed));
+    const R iL = R(1) / L;
+    const R eps = L * il0 - R(1);
+    const R den = m.m2 - eps * eps;
+    if (!(den > R(0))) atomicOr(status, ST_NUMERIC);
+    const R dEdL = m.K * (eps + eps / den);
+    const V3<R> a1 = xyz(ld4(tn + 4 * T.x)), a2 = xyz(ld4(tn + 4 * T.y));  // n / |n|^2
+    const R th = atan2_r(dot(cross(a1, a2), ed) * iL, dot(a1, a2));
+    const R dth = th - th0;
+    R cb = m.kb * dth;  // dE/dtheta
+    if (m.thm2i > R(0)) {  // nonlinear bending
+        const R r2 = dth * dth * m.thm2i;
+        if (!(r2 < R(1))) atomicOr(status, ST_NUMERIC);
+        cb = cb / (R(1) - r2);
+    }
+    st4(es + 4 * e, dEdL * iL, cb * L, cb * (dot(pa - p1, ed) * iL), cb * (dot(pb - p1, ed) * iL));
+}
+template <typename R> __device__ __forceinline__ bool tri_ok(const MeshDev<R> &m, int4 T, unsigned *status) {
+    return index_ok(T.x >= 0 && T.x < m.nv && T.y >= 0 && T.y < m.nv && T.z >= 0 && T.z < m.nv, status);
+}
+template <typename R> __device__ __forceinline__ bool edge_ok(const MeshDev<R> &m, int4 E, int2 T, unsigned *status) {
+    return index_ok(E.x >= 0 && E.x < m.nv && E.y >= 0 && E.y < m.nv && E.z >= 0 && E.z < m.nv && E.w >= 0 &&
+                        E.w < m.nv && T.x >= 0 && T.x < m.nt && T.y >= 0 && T.y < m.nt,
+                    status);
+}
+
+// Force on vertex i: the sum over its edges and triangles, walking the fan T_k
+// = (i, j_k, j_k+1) in cyclic order so that each triangle record and each
+// neighbour position is loaded once: at step k the edge (i, j_k) (link and
+// lever-rule bending; its triangles are T_k and T_k-1) and the triangle T_k-1
+// (wing term of its edge opposite i, area and volume).  False if the fan's
+// first entry fails its check.
+template <typename R>
+__device__ __forceinline__ bool fan_force(const MeshDev<R> &m, const R *xs, const R *tn, const R *es, const R *tl, int i,
+                                          R ha, R sv, unsigned *status, V3<R> &f) {
+    const V3<R> pi = xyz(ld4(xs + 4 * i));
+    f = {R(0), R(0), R(0)};
+    int4 g = __ldg(m.vfan + i);  // slot 0: the last entry
+    int4 gn = __ldg(m.vfan + (size_t)m.nv + i);  // slot 1, requested ahead (its L2 latency overlaps slot 0's use)
+    auto fan_ok = [&](int4 q) {
+        return index_ok(q.x >= 0 && q.x < m.nt && q.y >= 0 && q.y < m.nv && (q.z >> 1) >= 0 && (q.z >> 1) < m.ne &&
+                            q.w >= 0 && q.w < m.ne,
+                        status);
+    };
+    if (!fan_ok(g)) return false;
+    Q4<R> ap = ld4(tn + 4 * g.x);  // T_k-1: n / |n|^2 and |n|
+    V3<R> xp = xyz(ld4(xs + 4 * g.y));  // position of j_k-1
+    int op = g.w;  // edge of T_k-1 opposite i
+    int tp = g.x;  // T_k-1
+    for (int k = 1; k <= m.maxv; ++k) {
+        g = gn;
+        if (g.x < 0 || !fan_ok(g)) break;
+        if (k < m.maxv) gn = __ldg(m.vfan + (size_t)(k + 1) * m.nv + i);  // the next slot, ahead
+        const Q4<R> ak = ld4(tn + 4 * g.x);
+        const V3<R> xk = xyz(ld4(xs + 4 * g.y));
+        const Q4<R> cf = ld4(es + 4 * (g.z >> 1));
+        // the edge's triangles (v0, v1, a), (v1, v0, b) are T_k, T_k-1
+        // when i is its v0 (role 0) and T_k-1, T_k otherwise
+        const bool r1 = g.z & 1;
+        const V3<R> a1 = r1 ? xyz(ap) : xyz(ak), a2 = r1 ? xyz(ak) : xyz(ap);
+        const V3<R> lk = cf.x * (xk - pi);
+        f = r1 ? f + lk - ((cf.z + cf.y) * a1 + (cf.w + cf.y) * a2) : f + lk + (cf.z * a1 + cf.w * a2);
+        f = f + es[4 * op + 1] * xyz(ap);
+        const V3<R> nh = ap.w * xyz(ap);  // unit normal of T_k-1
+        const R hk = m.k_local > R(0) ? ha + tl[tp] : ha;  // global and local area terms
+        f = f - (hk * cross(nh, xk - xp) + sv * cross(xp, xk));
+        ap = ak;
+        xp = xk;
+        op = g.w;
+        tp = g.x;
+    }
+    return true;
+}
+
 template <typename R, int NT>
 __global__ void __launch_bounds__(NT, CellMinBlocks<R, NT>::B) cell_kernel(View<R> v, int mode, double *stats) {
     if (mode == 0 && v.adapt && !v.adapt[2]) return;  // adaptive separation: the forces are held on this step
@@ -274,8 +378,7 @@ __global__ void __launch_bounds__(NT, CellMinBlocks<R, NT>::B) cell_kernel(View<
         for (int i = threadIdx.x; i < m.nv; i += blockDim.x)
             bin_vertex(v, (size_t)(first + i), csplit[0], csplit[1], xs + 4 * i);
 
-    // per triangle: a = n / |n|^2 and |n|, with n = (x1 - x0) x (x2 - x0);
-    // area |n|/2 and volume x0 . (x1 x x2) / 6 summed per cell
+    // triangle records; area and volume summed per cell
     // (the next item's mesh records are loaded before this item is
     // processed, here and in the edge pass: their L2 latency overlaps the
     // arithmetic)
@@ -285,18 +388,11 @@ __global__ void __launch_bounds__(NT, CellMinBlocks<R, NT>::B) cell_kernel(View<
         for (int t = threadIdx.x; t < m.nt; t += blockDim.x) {
             const int4 T = Tn;
             if (t + (int)blockDim.x < m.nt) Tn = __ldg(m.tri4 + t + blockDim.x);
-            if (!index_ok(T.x >= 0 && T.x < m.nv && T.y >= 0 && T.y < m.nv && T.z >= 0 && T.z < m.nv, v.status))
-                continue;
-            const V3<R> p0 = xyz(ld4(xs + 4 * T.x)), p1 = xyz(ld4(xs + 4 * T.y)), p2 = xyz(ld4(xs + 4 * T.z));
-            const V3<R> n = cross(p1 - p0, p2 - p0);
-            const R q = dot(n, n), ln = sqrt_r(q), iq = R(1) / q;
-            st4(tn + 4 * t, iq * n.x, iq * n.y, iq * n.z, ln);
-            if (m.k_local > R(0)) {
-                const R a0 = __ldg(m.At0 + t);
-                tl[t] = R(0.5) * m.k_local * (R(0.5) * ln - a0) / a0;
-            }
-            av[0].add(R(0.5) * ln);
-            av[1].add(dot(p0, cross(p1, p2)) / R(6));
+            if (!tri_ok(m, T, v.status)) continue;
+            R area, vol;
+            tri_record(m, xs, tn, tl, t, T, area, vol);
+            av[0].add(area);
+            av[1].add(vol);
         }
     }
     double AV[2];
@@ -336,11 +432,6 @@ __global__ void __launch_bounds__(NT, CellMinBlocks<R, NT>::B) cell_kernel(View<
         cav[1] = R(m.k_volume * (V - m.V0) / (m.V0 * m.V0) / 6.0);
     }
 
-    // per edge: link coefficient s (F on v0 = s (x1 - x0)), cb |e| for the
-    // wing vertices, and the lever-rule coefficients cb sa0, cb sb0 of v0
-    // (those of v1 are cb sa0 + cb |e| and cb sb0 + cb |e|, since
-    // sa1 - sa0 = sb1 - sb0 = |e|); the edge's triangles are (v0, v1, a)
-    // and (v1, v0, b)
     const int4 *edge4 = reinterpret_cast<const int4 *>(m.edge);  // v0, v1, a, b
     const int2 *etri2 = reinterpret_cast<const int2 *>(m.etri);
     int4 En = make_int4(0, 0, 0, 0);
@@ -362,75 +453,228 @@ __global__ void __launch_bounds__(NT, CellMinBlocks<R, NT>::B) cell_kernel(View<
             il0n = __ldg(m.invL0 + e + blockDim.x);
             th0n = __ldg(m.th0 + e + blockDim.x);
         }
-        if (!index_ok(E.x >= 0 && E.x < m.nv && E.y >= 0 && E.y < m.nv && E.z >= 0 && E.z < m.nv && E.w >= 0 &&
-                          E.w < m.nv && T.x >= 0 && T.x < m.nt && T.y >= 0 && T.y < m.nt,
-                      v.status))
-            continue;
-        const V3<R> p0 = xyz(ld4(xs + 4 * E.x)), p1 = xyz(ld4(xs + 4 * E.y));
-        const V3<R> pa = xyz(ld4(xs + 4 * E.z)), pb = xyz(ld4(xs + 4 * E.w));
-        const V3<R> ed = p1 - p0;
-        const R L = sqrt_r(dot(ed, ed));
-        const R iL = R(1) / L;
-        const R eps = L * il0 - R(1);
-        const R den = m.m2 - eps * eps;
-        if (!(den > R(0))) atomicOr(v.status, ST_NUMERIC);
-        const R dEdL = m.K * (eps + eps / den);
-        const V3<R> a1 = xyz(ld4(tn + 4 * T.x)), a2 = xyz(ld4(tn + 4 * T.y));  // n / |n|^2
-        const R th = atan2_r(dot(cross(a1, a2), ed) * iL, dot(a1, a2));
-        const R dth = th - th0;
-        R cb = m.kb * dth;  // dE/dtheta
-        if (m.thm2i > R(0)) {  // nonlinear bending
-            const R r2 = dth * dth * m.thm2i;
-            if (!(r2 < R(1))) atomicOr(v.status, ST_NUMERIC);
-            cb = cb / (R(1) - r2);
-        }
-        st4(es + 4 * e, dEdL * iL, cb * L, cb * (dot(pa - p1, ed) * iL), cb * (dot(pb - p1, ed) * iL));
+        if (!edge_ok(m, E, T, v.status)) continue;
+        edge_record(m, xs, tn, es, e, E, T, il0, th0, v.status);
     }
     __syncthreads();
 
-    // per vertex: the sum over its edges and triangles, walking the fan
-    // T_k = (i, j_k, j_k+1) in cyclic order so that each triangle record and
-    // each neighbour position is loaded once: at step k the edge (i, j_k)
-    // (link and lever-rule bending; its triangles are T_k and T_k-1) and the
-    // triangle T_k-1 (wing term of its edge opposite i, area and volume)
     const R ha = cav[0], sv = cav[1];
     for (int i = threadIdx.x; i < m.nv; i += blockDim.x) {
-        const V3<R> pi = xyz(ld4(xs + 4 * i));
-        V3<R> f = {R(0), R(0), R(0)};
-        int4 g = __ldg(m.vfan + i);  // slot 0: the last entry
-        int4 gn = __ldg(m.vfan + (size_t)m.nv + i);  // slot 1, requested ahead (its L2 latency overlaps slot 0's use)
-        auto fan_ok = [&](int4 q) {
-            return index_ok(q.x >= 0 && q.x < m.nt && q.y >= 0 && q.y < m.nv && (q.z >> 1) >= 0 && (q.z >> 1) < m.ne &&
-                                q.w >= 0 && q.w < m.ne,
-                            v.status);
-        };
-        if (!fan_ok(g)) continue;
-        Q4<R> ap = ld4(tn + 4 * g.x);  // T_k-1: n / |n|^2 and |n|
-        V3<R> xp = xyz(ld4(xs + 4 * g.y));  // position of j_k-1
-        int op = g.w;  // edge of T_k-1 opposite i
-        int tp = g.x;  // T_k-1
-        for (int k = 1; k <= m.maxv; ++k) {
-            g = gn;
-            if (g.x < 0 || !fan_ok(g)) break;
-            if (k < m.maxv) gn = __ldg(m.vfan + (size_t)(k + 1) * m.nv + i);  // the next slot, ahead
-            const Q4<R> ak = ld4(tn + 4 * g.x);
-            const V3<R> xk = xyz(ld4(xs + 4 * g.y));
-            const Q4<R> cf = ld4(es + 4 * (g.z >> 1));
-            // the edge's triangles (v0, v1, a), (v1, v0, b) are T_k, T_k-1
-            // when i is its v0 (role 0) and T_k-1, T_k otherwise
-            const bool r1 = g.z & 1;
-            const V3<R> a1 = r1 ? xyz(ap) : xyz(ak), a2 = r1 ? xyz(ak) : xyz(ap);
-            const V3<R> lk = cf.x * (xk - pi);
-            f = r1 ? f + lk - ((cf.z + cf.y) * a1 + (cf.w + cf.y) * a2) : f + lk + (cf.z * a1 + cf.w * a2);
-            f = f + es[4 * op + 1] * xyz(ap);
-            const V3<R> nh = ap.w * xyz(ap);  // unit normal of T_k-1
-            const R hk = m.k_local > R(0) ? ha + tl[tp] : ha;  // global and local area terms
-            f = f - (hk * cross(nh, xk - xp) + sv * cross(xp, xk));
-            ap = ak;
-            xp = xk;
-            op = g.w;
-            tp = g.x;
+        V3<R> f;
+        if (!fan_force(m, xs, tn, es, tl, i, ha, sv, v.status, f)) continue;
+        R *o = v.Fv + 3 * (size_t)(first + i);
+        o[0] = f.x;
+        o[1] = f.y;
+        o[2] = f.z;
+    }
+}
+
+// Few cells: a cluster of CTAs per cell.  One CTA per cell leaves most of the
+// SMs idle, and in FP64 a single SM's FP64 pipe (a warp instruction takes 19
+// cycles) sets the kernel's time.  CTA `slice` of the cluster takes a range of
+// the vertices: it re-bases all of them in its own shared memory (cheap, and
+// the same bits in every CTA), computes the triangle and edge records that the
+// fans of its vertices read (lists built with the mesh tables; neighbouring
+// slices repeat the records along their border), then walks the fans of its
+// own vertices.  The CTAs exchange the sums only: each writes its part of the
+// area and volume (over the triangles it owns) into every CTA's shared memory,
+// and all add the parts in the same order.  Two cluster barriers: the offsets
+// and the centroid are overwritten only after every CTA has read them, and
+// the parts are read only after all have been written (the edge records are
+// computed in between).
+//
+// Bound by the serial chain of a slice (FP64: the edges' atan2 and divisions on
+// its SM's FP64 pipe; FP32: latency).  Membrane phase, one CTA per cell -> the
+// cluster: FP64, 1 cell (16 slices) 168 -> 41 us, 30 cells (4) 168 -> 66 us; FP32,
+// 4 cells (16) 22.3 -> 18.5 us, 6 cells 22 -> 20 us.
+template <typename R> struct SliceThreads { static constexpr int T = CellMax<R>::T; };
+template <typename R>
+__global__ void __launch_bounds__(SliceThreads<R>::T, 1) cell_slices_kernel(View<R> v, int mode, double *stats) {
+    namespace cg = cooperative_groups;
+    constexpr int NT = SliceThreads<R>::T;
+    if (mode == 0 && v.adapt && !v.adapt[2]) return;  // (every CTA of the cluster)
+    cg::cluster_group cluster = cg::this_cluster();
+    const int S = v.slices, c = blockIdx.x / S, slice = blockIdx.x % S;  // (clusters are consecutive CTAs)
+    const MeshDev<R> m = v.meshes[v.cell_type[c]];
+    const int first = v.cell_first[c];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    R *xs = reinterpret_cast<R *>(smem_raw);  // as in cell_kernel
+    R *tn = xs + 4 * v.max_nv;
+    R *es = tn + 4 * v.max_nt;
+    R *tl = es + 4 * v.max_ne;
+    __shared__ double scratch[6][32];
+    __shared__ double part[MAX_SLICES][2];  // every slice's sums
+    __shared__ R rscratch[3][32];
+    __shared__ R rmean[3];
+    __shared__ double cnew[3];
+    __shared__ R csplit[2][3];
+    __shared__ R cav[2];
+    const int per = (m.nv + S - 1) / S, v0 = min(m.nv, slice * per), v1 = min(m.nv, v0 + per);
+    const int t0 = m.sl_at[slice], t1 = m.sl_at[slice + 1], e0 = m.sl_at[S + 1 + slice], e1 = m.sl_at[S + 2 + slice];
+
+    // mean offset and re-base, as in cell_kernel
+    constexpr int KC = 4;
+    R oc[KC][3];
+    R mean[3] = {R(0), R(0), R(0)};
+#pragma unroll
+    for (int kk = 0; kk < KC; ++kk) {
+        const int i = threadIdx.x + kk * NT;
+        if (i < m.nv) {
+            const R *o = v.off + 3 * (size_t)(first + i);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                oc[kk][k] = o[k];
+                mean[k] += oc[kk][k];
+            }
         }
+    }
+    for (int i = threadIdx.x + KC * NT; i < m.nv; i += NT)
+        for (int k = 0; k < 3; ++k) mean[k] += v.off[3 * (size_t)(first + i) + k];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        for (int o = 16; o > 0; o >>= 1) mean[k] += __shfl_down_sync(0xffffffffu, mean[k], o);
+        if (lane == 0) rscratch[k][wid] = mean[k];
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        const int k = threadIdx.x;
+        R t = R(0);
+        for (int w = 0; w < NT / 32; ++w) t += rscratch[k][w];
+        t /= R(m.nv);
+        rmean[k] = t;
+        cnew[k] = v.ctr[3 * c + k] + (double)t;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (v.le && mode == 0) {  // Lees-Edwards: a centroid that left through z = 0 or nz moves to the other side
+            const double D = le_shift(v);
+            if (cnew[2] >= v.nz) {
+                cnew[0] -= D;
+                cnew[2] -= v.nz;
+            } else if (cnew[2] < 0) {
+                cnew[0] += D;
+                cnew[2] += v.nz;
+            }
+        }
+        for (int k = 0; k < 3; ++k) {
+            csplit[0][k] = R(cnew[k]);
+            csplit[1][k] = R(cnew[k] - (double)csplit[0][k]);
+        }
+    }
+    auto rebase = [&](int i, const R *o) { st4(xs + 4 * i, o[0] - rmean[0], o[1] - rmean[1], o[2] - rmean[2], R(0)); };
+#pragma unroll
+    for (int kk = 0; kk < KC; ++kk) {
+        const int i = threadIdx.x + kk * NT;
+        if (i < m.nv) rebase(i, oc[kk]);
+    }
+    for (int i = threadIdx.x + KC * NT; i < m.nv; i += NT) {
+        const R *o = v.off + 3 * (size_t)(first + i);
+        const R ol[3] = {o[0], o[1], o[2]};
+        rebase(i, ol);
+    }
+    __syncthreads();
+    cluster.barrier_arrive();  // this CTA has read the offsets and the centroid
+
+    // the slice's triangles: records, and the sums over those it owns
+    Acc<R> sum[2];
+    for (int q = t0 + threadIdx.x; q < t1; q += NT) {
+        const int id = m.sl_items[q], t = id >> 1;
+        const int4 T = __ldg(m.tri4 + t);
+        if (!tri_ok(m, T, v.status)) continue;
+        R area, vol;
+        tri_record(m, xs, tn, tl, t, T, area, vol);
+        if (id & 1) {
+            sum[0].add(area);
+            sum[1].add(vol);
+        }
+    }
+    cluster.barrier_wait();
+    if (mode == 0) {
+        for (int i = v0 + threadIdx.x; i < v1; i += NT) {
+            const size_t g = (size_t)(first + i);
+            const R *r = xs + 4 * i;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                v.off[3 * g + k] = r[k];
+                if (v.off_rec) v.off_rec[3 * g + k] = r[k];
+                if (v.off_eval) v.off_eval[3 * g + k] = r[k];  // positions of this evaluation
+            }
+            bin_vertex(v, g, csplit[0], csplit[1], r);
+        }
+        if (slice == 0 && threadIdx.x < 3) {
+            const int k = threadIdx.x;
+            v.ctr[3 * c + k] = cnew[k];
+            v.csp[6 * c + k] = csplit[0][k];
+            v.csp[6 * c + 3 + k] = csplit[1][k];
+        }
+    }
+    double tot[2];
+    block_total<R, 2>(sum, tot, scratch);  // (synchronises: tn is complete below)
+    if (threadIdx.x < S) {
+        double *p = cluster.map_shared_rank(&part[slice][0], threadIdx.x);
+        p[0] = tot[0];
+        p[1] = tot[1];
+    }
+    cluster.barrier_arrive();  // (release: the parts)
+
+    double G[6] = {};  // gyration sums, in cell_kernel's order: the deformation index of a disc is sensitive to their rounding
+    if (mode == 0) {
+        for (int q = e0 + threadIdx.x; q < e1; q += NT) {
+            const int e = m.sl_items[q];
+            const int4 E = __ldg(reinterpret_cast<const int4 *>(m.edge) + e);
+            const int2 T = __ldg(reinterpret_cast<const int2 *>(m.etri) + e);
+            if (!edge_ok(m, E, T, v.status)) continue;
+            edge_record(m, xs, tn, es, e, E, T, __ldg(m.invL0 + e), __ldg(m.th0 + e), v.status);
+        }
+    } else if (slice == 0) {
+        Acc<R> g[6];
+        for (int i = threadIdx.x; i < m.nv; i += NT) {
+            const R x = xs[4 * i], y = xs[4 * i + 1], z = xs[4 * i + 2];
+            g[0].add(x * x);
+            g[1].add(y * y);
+            g[2].add(z * z);
+            g[3].add(x * y);
+            g[4].add(x * z);
+            g[5].add(y * z);
+        }
+        block_total<R, 6>(g, G, scratch);
+    }
+    cluster.barrier_wait();  // (acquire)
+    if (mode == 1) {
+        if (slice == 0 && threadIdx.x == 0) {
+            double A = 0, V = 0, lmax, lmin;
+            for (int r = 0; r < S; ++r) {
+                A += part[r][0];
+                V += part[r][1];
+            }
+            const double in = 1.0 / m.nv;
+            sym3_eig(G[0] * in, G[1] * in, G[2] * in, G[3] * in, G[4] * in, G[5] * in, lmax, lmin);
+            const double a = sqrt(lmax), b = sqrt(lmin > 0 ? lmin : 0);
+            double *o = stats + 6 * (size_t)c;
+            o[0] = cnew[0];
+            o[1] = cnew[1];
+            o[2] = cnew[2];
+            o[3] = A;
+            o[4] = V;
+            o[5] = (a - b) / (a + b);
+        }
+        return;
+    }
+    if (threadIdx.x == 0) {
+        double A = 0, V = 0;
+        for (int r = 0; r < S; ++r) {
+            A += part[r][0];
+            V += part[r][1];
+        }
+        cav[0] = R(0.5 * m.k_area * (A - m.A0) / (m.A0 * m.A0));
+        cav[1] = R(m.k_volume * (V - m.V0) / (m.V0 * m.V0) / 6.0);
+    }
+    __syncthreads();
+    const R ha = cav[0], sv = cav[1];
+    for (int i = v0 + threadIdx.x; i < v1; i += NT) {
+        V3<R> f;
+        if (!fan_force(m, xs, tn, es, tl, i, ha, sv, v.status, f)) continue;
         R *o = v.Fv + 3 * (size_t)(first + i);
         o[0] = f.x;
         o[1] = f.y;
@@ -821,10 +1065,59 @@ template <typename R>
 bool cell_wide(const View<R> &v) { return CellMax<R>::T > 256 && v.ncell <= v.nsm; }
 
 template <typename R>
+cudaLaunchConfig_t slices_config(int slices, int ncell, size_t smem, cudaStream_t st, cudaLaunchAttribute *at) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(ncell * slices));
+    cfg.blockDim = dim3(SliceThreads<R>::T);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)slices;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+constexpr size_t SLICES_MAX_SMEM = 220 * 1024;  // dynamic shared memory beside the kernel's own 4 KB
+
+// CTAs per cell: the largest power of two up to 16 (a cluster of more than 8
+// where the device can place one) at which every cluster has its own SMs; 1:
+// cell_kernel
+template <typename R>
+int cell_slices(int ncell, int nsm, size_t smem) {
+    if (ncell == 0) return 1;
+    cudaFuncSetAttribute(cell_slices_kernel<R>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (smem > SLICES_MAX_SMEM ||  // (the same cap for every simulation)
+        cudaFuncSetAttribute(cell_slices_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SLICES_MAX_SMEM) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
+    for (int s = MAX_SLICES; s > 1; s /= 2) {
+        if ((long long)ncell * s > nsm) continue;
+        cudaLaunchAttribute at[1];
+        const cudaLaunchConfig_t cfg = slices_config<R>(s, ncell, smem, nullptr, at);
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, cell_slices_kernel<R>, &cfg) == cudaSuccess && clusters >= ncell) {
+            cudaGetLastError();
+            return s;
+        }
+    }
+    cudaGetLastError();
+    return 1;
+}
+
+template <typename R>
 void launch_cell_forces(const View<R> &v, int mode, double *stats, cudaStream_t st) {
     if (v.ncell == 0) return;
     // positions and force accumulators of the largest mesh type
     const size_t smem = cell_smem_bytes<R>(v.max_nv, v.max_nt, v.max_ne);
+    if (v.slices > 1) {
+        cudaLaunchAttribute at[1];
+        const cudaLaunchConfig_t cfg = slices_config<R>(v.slices, v.ncell, smem, st, at);
+        cudaLaunchKernelEx(&cfg, cell_slices_kernel<R>, v, mode, stats);
+        return;
+    }
     if (cell_wide(v)) cell_kernel<R, CellMax<R>::T><<<v.ncell, CellMax<R>::T, smem, st>>>(v, mode, stats);
     else cell_kernel<R, 256><<<v.ncell, 256, smem, st>>>(v, mode, stats);
 }
@@ -895,6 +1188,8 @@ template void launch_deformation_loss<float>(const View<float> &, const double *
 template void launch_cell_forces<double>(const View<double> &, int, double *, cudaStream_t);
 template void launch_cell_forces<float>(const View<float> &, int, double *, cudaStream_t);
 template cudaError_t set_cell_smem_limit<double>(size_t);
+template int cell_slices<double>(int, int, size_t);
+template int cell_slices<float>(int, int, size_t);
 template cudaError_t set_cell_smem_limit<float>(size_t);
 
 }  // namespace hemo
