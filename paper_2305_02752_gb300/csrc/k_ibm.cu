@@ -241,16 +241,13 @@ __device__ __forceinline__ void cp_async4(float *smem_dst, const float *gsrc) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gsrc) : "memory");
 }
+__device__ __forceinline__ void cp_async(double *smem_dst, const double *gsrc) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(gsrc) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // four consecutive values from 16-byte aligned shared memory
-__device__ __forceinline__ void ld4v(const float *p, float *o) {
-    const float4 q = *reinterpret_cast<const float4 *>(p);
-    o[0] = q.x;
-    o[1] = q.y;
-    o[2] = q.z;
-    o[3] = q.w;
-}
 __device__ __forceinline__ void ld4v(const double *p, double *o) {
     const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
     o[0] = a.x;
@@ -268,6 +265,39 @@ __device__ __forceinline__ void peskin4(R t, R *w) {
     w[1] = (R(3) - R(2) * t + q) * R(0.125);
     w[2] = (R(1) + R(2) * t + q) * R(0.125);
     w[3] = (R(1) + R(2) * t - q) * R(0.125);
+}
+
+// Sums of K <= 8 values over each half-warp's 16 lanes, with about K + 3 additions
+// per lane instead of 4 K (additions are what the FP64 pipe is short of): at
+// every level a lane passes on half of its values and adds the other half.
+// Returns value k in out[k] of every lane.
+template <typename R, int K>
+__device__ __forceinline__ void sum16(const R (&x)[K], R (&out)[K]) {
+    constexpr int P = K <= 4 ? 4 : 8;
+    const int lane = threadIdx.x & 31;
+    R a[P];
+#pragma unroll
+    for (int k = 0; k < P; ++k) a[k] = k < K ? x[k] : R(0);
+    int o = 8;
+#pragma unroll
+    for (int n = P / 2; n >= 1; n /= 2, o /= 2) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < n; ++k) {
+            const R keep = up ? a[k + n] : a[k], give = up ? a[k] : a[k + n];
+            a[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    for (; o >= 1; o /= 2) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+    // value k sits in the lanes whose leading bits (from 8 down) spell k
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        int src = 0;
+#pragma unroll
+        for (int n = P / 2, bit = 8; n >= 1; n /= 2, bit /= 2)
+            if (k & n) src |= bit;
+        out[k] = __shfl_sync(0xffffffffu, a[0], (lane & 16) | src);
+    }
 }
 
 // FP64 vertex kernels: CTAs per bin, each taking every FP64_BIN_PARTS-th
@@ -290,36 +320,52 @@ __device__ __forceinline__ int neighbour_blocks(int b, int nb, int periodic, int
     return cnt;
 }
 
-// Vertex records of one chunk of a bin, staged in shared memory: one thread
-// per vertex reads its anchor through the permutation, computes its row in
-// the bin's padded tile (-1 if the anchor is outside the bin, i.e. the
-// vertex left the lattice) and its twelve Peskin weights (x0..3, y0..3,
-// z0..3), and optionally its force (four entries per vertex, times fscale
-// per component if given).  The per-vertex loops below then touch
-// shared memory only.  Chunk size by precision keeps the FP64 kernels within
-// 48 KB of static shared memory.
-// (FP32: 240 keeps the spreading kernel at six CTAs per SM)
-template <typename R> struct Stage { static constexpr int CAP = sizeof(R) == 8 ? 32 : 240; };
-template <typename R>
-__device__ __forceinline__ void stage_chunk(const View<R> &v, int p0, int n, const int org[3], int *srow, R *sw,
-                                            R *sF, int *sperm, const R *fscale = nullptr) {
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+// FP64 vertex kernels: anchors and weights of one chunk of a bin, staged in
+// shared memory, a thread per vertex and axis (the square roots run on the FP64
+// pipe and are a long chain): the row in the bin's padded tile (-1 if the
+// anchor is outside the bin, i.e. the vertex left the lattice), the vertex id
+// and whatever weights(j, i, axis, t) stores for fraction t.
+template <typename R, typename Weights>
+__device__ __forceinline__ void stage_chunk(const View<R> &v, int p0, int n, const int org[3], int *srow, int *sperm,
+                                            Weights weights) {
+    for (int q = threadIdx.x; q < 3 * n; q += blockDim.x) {
+        const int j = q / 3, ax = q - 3 * j;
         const int i = v.perm[p0 + j];
         if (!index_ok(i >= 0 && i < v.nv, v.status)) {
-            srow[j] = -1;
+            if (ax == 0) srow[j] = -1;
             continue;
         }
-        int row = 0;
-        bool ok = true;
-        for (int d = 0; d < 3; ++d) {
-            const int b = v.anc_i[3 * (size_t)i + d] - org[d];
-            ok &= b >= 0 && b < BLK;
-            row += b * (d == 0 ? 1 : (d == 1 ? TS_Y : TS_Z));
-            peskin4(v.anc_t[3 * (size_t)i + d], sw + 12 * j + 4 * d);
-            if (sF) sF[4 * j + d] = fscale ? v.Fv[3 * (size_t)i + d] * fscale[d] : v.Fv[3 * (size_t)i + d];
+        weights(j, i, ax, v.anc_t[3 * (size_t)i + ax]);
+        if (ax == 0) {
+            int row = 0;
+            bool ok = true;
+            for (int d = 0; d < 3; ++d) {
+                const int b = v.anc_i[3 * (size_t)i + d] - org[d];
+                ok &= b >= 0 && b < BLK;
+                row += b * (d == 0 ? 1 : (d == 1 ? TS_Y : TS_Z));
+            }
+            srow[j] = ok ? row : -1;
+            if (sperm) sperm[j] = i;
         }
-        srow[j] = ok ? row : -1;
-        if (sperm) sperm[j] = i;
+    }
+}
+
+// the 11^3 neighbourhood of a 3-component field A ([3][N]) requested into a padded
+// shared tile by asynchronous copies (zero beyond a non-periodic edge); jtab:
+// the wrapped lattice coordinates per axis
+template <typename R>
+__device__ __forceinline__ void stage_tile(const View<R> &v, const R *A, const int (*jtab)[TILE], R (*tile)[TILE_SMEM]) {
+    const size_t N = (size_t)v.N;
+    TileWalk tw(threadIdx.x, blockDim.x);
+    for (int q = threadIdx.x; q < TILE3; q += blockDim.x, tw.next()) {
+        const int jx = jtab[0][tw.l0], jy = jtab[1][tw.l1], jz = jtab[2][tw.l2];
+        const int sidx = tw.l0 + TS_Y * tw.l1 + TS_Z * tw.l2;
+        if ((jx | jy | jz) < 0) {  // beyond a non-periodic edge: resting wall
+            tile[0][sidx] = tile[1][sidx] = tile[2][sidx] = R(0);
+        } else {
+            const size_t n = (size_t)jx + (size_t)v.nx * ((size_t)jy + (size_t)v.ny * jz);
+            for (int d = 0; d < 3; ++d) cp_async(&tile[d][sidx], A + d * N + n);
+        }
     }
 }
 
@@ -345,6 +391,7 @@ template <> struct TileAcc<float> {
     static constexpr int E = 29;
 };
 __device__ __forceinline__ long long fixed_of(double x) { return __double2ll_rn(x); }
+template <typename R> struct SpreadCap { static constexpr int CAP = 128; };  // vertices staged at a time (FP64)
 
 // the scale of a component from its largest force; 0 (and the numeric
 // status) for forces that are not finite
@@ -592,94 +639,76 @@ __global__ void __launch_bounds__(SP_CHUNK, 6) spread_tile_f32_kernel(View<float
     }
 }
 
-// FP64: a warp takes two vertices, each half-warp's 16 lanes own one (y, z) row
-// of the stencil.
+// FP64: one CTA per bin and force component (three times the CTAs on the
+// FP64 pipes, which a bin's vertices keep busy for long); a warp takes two
+// vertices, each half-warp's 16 lanes own one (y, z) row of the stencil.
+// Bound by the FP64 pipe (products and conversions) and 64-bit shared
+// atomics (12 cycles per warp).  Spreading phase of the 32^3 box with one cell
+// 51 -> 26 us, of a 48 x 39 x 64 channel with 30 cells 143 -> 78 us (one CTA
+// per bin; weights by one thread per vertex).
 template <typename R>
 __global__ void __launch_bounds__(256) spread_tile_kernel(View<R> v) {
     using A = typename TileAcc<R>::T;
-    constexpr int CAP = Stage<R>::CAP;
-    const int k = blockIdx.x;
+    constexpr int CAP = SpreadCap<R>::CAP;
+    const int k = blockIdx.x / 3, d = blockIdx.x - 3 * k;
     const int s = v.start[k], e = v.start[k + 1];
     if (s == e) return;
-    __shared__ A acc[3][TILE_SMEM];
+    __shared__ A acc[TILE_SMEM];
     __shared__ int srow[CAP];
     __shared__ __align__(16) R sw[12 * CAP];
-    __shared__ __align__(16) R sF[4 * CAP];
-    __shared__ R smax[3][8];
-    __shared__ R scale[3];
-    for (int q = threadIdx.x; q < TILE_SMEM; q += blockDim.x) acc[0][q] = acc[1][q] = acc[2][q] = A(0);
+    __shared__ R sF[CAP];
+    __shared__ R smax[8];
+    __shared__ R scale_s;
+    for (int q = threadIdx.x; q < TILE_SMEM; q += blockDim.x) acc[q] = A(0);
     int org[3];
     bin_origin(v, k, org);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int h = lane >> 4, b = lane & 3, c = (lane >> 2) & 3;
-    // A bin of at most CAP vertices is staged once, before the scale is known
-    // (its forces unscaled; the scale is applied in the loop below, exactly,
-    // being a power of two), which saves a pass over the forces; larger bins
-    // take that pass first and are staged in chunks of equal size.
-    const bool one = e - s <= CAP;
-    if (one) stage_chunk(v, s, e - s, org, srow, sw, sF, (int *)nullptr);
-    {  // one scale per component for the whole bin
-        R m[3] = {R(0), R(0), R(0)};
-        if (one) {
-            for (int j = threadIdx.x; j < e - s; j += blockDim.x)  // (the forces this thread staged)
-                for (int d = 0; d < 3; ++d) m[d] = fmax(m[d], fabs(sF[4 * j + d]));
-        } else {
-            for (int j = s + threadIdx.x; j < e; j += blockDim.x) {
-                const int i = v.perm[j];
-                if (!index_ok(i >= 0 && i < v.nv, v.status)) continue;
-                for (int d = 0; d < 3; ++d) m[d] = fmax(m[d], fabs(v.Fv[3 * (size_t)i + d]));
-            }
+    {  // the component's scale for the whole bin
+        R m = R(0);
+        for (int j = s + threadIdx.x; j < e; j += blockDim.x) {
+            const int i = v.perm[j];
+            if (!index_ok(i >= 0 && i < v.nv, v.status)) continue;
+            m = fmax(m, fabs(v.Fv[3 * (size_t)i + d]));
         }
-        for (int d = 0; d < 3; ++d) {
-            for (int o = 16; o > 0; o >>= 1) m[d] = fmax(m[d], __shfl_xor_sync(0xffffffffu, m[d], o));
-            if (lane == 0) smax[d][warp] = m[d];
+        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (lane == 0) smax[warp] = m;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < nw; ++w) m = fmax(m, smax[w]);
+            scale_s = tile_scale(m, e - s, v.status);
         }
         __syncthreads();
-        if (threadIdx.x < 3) {
-            R mm = R(0);
-            for (int w = 0; w < nw; ++w) mm = fmax(mm, smax[threadIdx.x][w]);
-            scale[threadIdx.x] = tile_scale(mm, e - s, v.status);
-        }
-        __syncthreads();  // the staging below or the loop applies the scale
     }
-    const R sc[3] = {one ? scale[0] : R(1), one ? scale[1] : R(1), one ? scale[2] : R(1)};
+    const R scale = scale_s;
     const int nch = (e - s + CAP - 1) / CAP, csz = (e - s + nch - 1) / nch;
     for (int p0 = s; p0 < e; p0 += csz) {
         const int n = min(csz, e - p0);
-        if (!one) {
-            if (p0 != s) __syncthreads();
-            stage_chunk(v, p0, n, org, srow, sw, sF, (int *)nullptr, scale);
-            __syncthreads();
-        }
+        if (p0 != s) __syncthreads();
+        stage_chunk(v, p0, n, org, srow, (int *)nullptr, [&](int j, int i, int ax, R t) {
+            peskin4(t, sw + 12 * j + 4 * ax);
+            if (ax == 0) sF[j] = v.Fv[3 * (size_t)i + d] * scale;
+        });
+        __syncthreads();
         for (int q = 2 * warp + h; q < n; q += 2 * nw) {
             const int row0 = srow[q];
             if (row0 < 0) continue;  // vertex outside the lattice (domain status already raised)
             const R *w = sw + 12 * q;
-            const R wyz = w[4 + b] * w[8 + c];
-            R wx[4], fq[4];
+            const R f = sF[q] * (w[4 + b] * w[8 + c]);
+            R wx[4];
             ld4v(w, wx);
-            ld4v(sF + 4 * q, fq);  // (times the fixed-point scale, or scaled here)
-            const R f[3] = {(fq[0] * sc[0]) * wyz, (fq[1] * sc[1]) * wyz, (fq[2] * sc[2]) * wyz};
             const int row = row0 + TS_Y * b + TS_Z * c;
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                const R wa = wx[a];
-#pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    atomicAdd((unsigned long long *)&acc[d][row + a], (unsigned long long)fixed_of(f[d] * wa));
-                }
-            }
+            for (int a = 0; a < 4; ++a)
+                atomicAdd((unsigned long long *)&acc[row + a], (unsigned long long)fixed_of(f * wx[a]));
         }
     }
     __syncthreads();
-    R *out = v.tiles + (size_t)k * 3 * TP_N;
-    R inv[3];
-    for (int d = 0; d < 3; ++d) inv[d] = scale[d] > R(0) ? R(1) / scale[d] : R(0);  // (exact: powers of two)
+    R *out = v.tiles + ((size_t)k * 3 + d) * TP_N;
+    const R inv = scale > R(0) ? R(1) / scale : R(0);  // (exact: a power of two)
     TileWalk tw(threadIdx.x, blockDim.x);
-    for (int q = threadIdx.x; q < TILE3; q += blockDim.x, tw.next()) {
-        const int sidx = tw.l0 + TS_Y * tw.l1 + TS_Z * tw.l2;
-        for (int d = 0; d < 3; ++d) out[d * TP_N + tile_index(tw.l0, tw.l1, tw.l2)] = (R)acc[d][sidx] * inv[d];
-    }
+    for (int q = threadIdx.x; q < TILE3; q += blockDim.x, tw.next())
+        out[tile_index(tw.l0, tw.l1, tw.l2)] = (R)acc[tw.l0 + TS_Y * tw.l1 + TS_Z * tw.l2] * inv;
 }
 
 // Phase 2 of spreading (owner computes): one CTA per 8^3 block sums, for
@@ -927,11 +956,16 @@ __global__ void __launch_bounds__(256) hold_bins_kernel(View<R> v) {
 // 11^3 neighbourhood in shared memory (padded strides; lattice coordinates
 // of the tile's rows from per-axis tables built once); a warp takes two
 // vertices, each half-warp's lanes own one (y, z) stencil row, and the 16
-// partial sums are reduced with warp shuffles.
+// partial sums are reduced with warp shuffles (sum16).  FP64 only; bound by the
+// staging's latency for few vertices (the tile by asynchronous copies while
+// the weights are computed, a thread per vertex and axis) and by the FP64 pipe:
+// 32^3 box with one cell 20.5 -> 16.4 us, 48 x 39 x 64 channel with 30 cells
+// 45 -> 35 us.
+constexpr int InterpCap = 32;  // vertices per chunk
 template <typename R, int INTEG>
 __global__ void __launch_bounds__(256) interpolate_kernel(View<R> v, int parts) {
     drop_dead_lines(v);
-    constexpr int CAP = Stage<R>::CAP;
+    constexpr int CAP = InterpCap;
     const int k = blockIdx.x / parts, part = blockIdx.x % parts;  // CTA part takes chunks part, part + parts, ...
     const int s = v.start[k], e = v.start[k + 1];
     if (s + part * CAP >= e) return;
@@ -950,51 +984,35 @@ __global__ void __launch_bounds__(256) interpolate_kernel(View<R> v, int parts) 
         jtab[d][l] = j;
     }
     __syncthreads();
-    const size_t N = (size_t)v.N;
-    for (int q = threadIdx.x; q < TILE3; q += blockDim.x) {
-        const int l0 = q % TILE, l1 = (q / TILE) % TILE, l2 = q / (TILE * TILE);
-        const int jx = jtab[0][l0], jy = jtab[1][l1], jz = jtab[2][l2];
-        const int sidx = l0 + TS_Y * l1 + TS_Z * l2;
-        if ((jx | jy | jz) < 0) {  // beyond a non-periodic edge: resting wall
-            tile[0][sidx] = tile[1][sidx] = tile[2][sidx] = R(0);
-        } else {
-            const size_t n = (size_t)jx + (size_t)v.nx * ((size_t)jy + (size_t)v.ny * jz);
-            tile[0][sidx] = v.u[n];
-            tile[1][sidx] = v.u[N + n];
-            tile[2][sidx] = v.u[2 * N + n];
-        }
-    }
+    stage_tile(v, (const R *)v.u, jtab, tile);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int h = lane >> 4, b = lane & 3, c = (lane >> 2) & 3;
     for (int c0 = s + part * CAP; c0 < e; c0 += parts * CAP) {
         const int n = min(CAP, e - c0);
-        __syncthreads();  // the tile (first chunk) or the previous chunk's records
-        stage_chunk(v, c0, n, org, srow, sw, (R *)nullptr, sperm);
+        if (c0 != s + part * CAP) __syncthreads();  // the previous chunk's records
+        stage_chunk(v, c0, n, org, srow, sperm, [&](int j, int, int ax, R t) { peskin4(t, sw + 12 * j + 4 * ax); });
+        if (c0 == s + part * CAP) cp_async_wait_all();  // the tile
         __syncthreads();
         for (int q0 = 2 * warp; q0 < n; q0 += 2 * nw) {  // uniform per warp: shuffles below
             const int q = q0 + h;
-            R U0 = R(0), U1 = R(0), U2 = R(0);
+            R U[3] = {R(0), R(0), R(0)};
             const int row0 = q < n ? srow[q] : -1;
             if (row0 >= 0) {
                 const R *w = sw + 12 * q;
                 const R wyz = w[4 + b] * w[8 + c];
                 const int row = row0 + TS_Y * b + TS_Z * c;
 #pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    const R wa = wyz * w[a];
-                    U0 += wa * tile[0][row + a];
-                    U1 += wa * tile[1][row + a];
-                    U2 += wa * tile[2][row + a];
+                for (int d = 0; d < 3; ++d) {
+                    R t = R(0);
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) t += w[a] * tile[d][row + a];
+                    U[d] = wyz * t;
                 }
             }
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) {
-                U0 += __shfl_xor_sync(0xffffffffu, U0, o);
-                U1 += __shfl_xor_sync(0xffffffffu, U1, o);
-                U2 += __shfl_xor_sync(0xffffffffu, U2, o);
-            }
+            R Us[3];
+            sum16(U, Us);
             double dmax = 0.0;
-            if (row0 >= 0 && (lane & 15) == 0) dmax = move_vertex<INTEG>(v, sperm[q], U0, U1, U2);
+            if (row0 >= 0 && (lane & 15) == 0) dmax = move_vertex<INTEG>(v, sperm[q], Us[0], Us[1], Us[2]);
             if (v.adapt) adapt_max(v.adapt, dmax);
         }
     }
@@ -1297,73 +1315,50 @@ __global__ void __launch_bounds__(256) vertex_field_kernel(View<R> v, const R *A
         jtab[d][l] = j;
     }
     __syncthreads();
-    const size_t N = (size_t)v.N;
-    for (int q = threadIdx.x; q < TILE3; q += blockDim.x) {
-        const int l0 = q % TILE, l1 = (q / TILE) % TILE, l2 = q / (TILE * TILE);
-        const int jx = jtab[0][l0], jy = jtab[1][l1], jz = jtab[2][l2];
-        const int sidx = l0 + TS_Y * l1 + TS_Z * l2;
-        if ((jx | jy | jz) < 0) {
-            tile[0][sidx] = tile[1][sidx] = tile[2][sidx] = R(0);
-        } else {
-            const size_t n = (size_t)jx + (size_t)v.nx * ((size_t)jy + (size_t)v.ny * jz);
-            tile[0][sidx] = A[n];
-            tile[1][sidx] = A[N + n];
-            tile[2][sidx] = A[2 * N + n];
-        }
-    }
+    stage_tile(v, A, jtab, tile);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int h = lane >> 4, b = lane & 3, c = (lane >> 2) & 3;
     for (int c0 = s + part * CAP; c0 < e; c0 += parts * CAP) {
         const int n = min(CAP, e - c0);
-        __syncthreads();  // the tile (first chunk) or the previous chunk's records
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            const int i = v.perm[c0 + j];
-            int row = 0;
-            bool ok = true;
-            for (int d = 0; d < 3; ++d) {
-                const int bb = v.anc_i[3 * (size_t)i + d] - org[d];
-                ok &= bb >= 0 && bb < BLK;
-                row += bb * (d == 0 ? 1 : (d == 1 ? TS_Y : TS_Z));
-                peskin4_d(v.anc_t[3 * (size_t)i + d], sw + 24 * j + 4 * d, sw + 24 * j + 12 + 4 * d);
-                sB[3 * j + d] = B ? B[3 * (size_t)i + d] : R(0);
-            }
-            srow[j] = ok ? row : -1;
-            sperm[j] = i;
-        }
+        if (c0 != s + part * CAP) __syncthreads();  // the previous chunk's records
+        stage_chunk(v, c0, n, org, srow, sperm, [&](int j, int i, int ax, R t) {
+            peskin4_d(t, sw + 24 * j + 4 * ax, sw + 24 * j + 12 + 4 * ax);
+            sB[3 * j + ax] = B ? B[3 * (size_t)i + ax] : R(0);
+        });
+        if (c0 == s + part * CAP) cp_async_wait_all();  // the tile
         __syncthreads();
         for (int q0 = 2 * warp; q0 < n; q0 += 2 * nw) {  // uniform per warp: shuffles below
             const int q = q0 + h;
-            R U[3] = {R(0), R(0), R(0)}, G[3] = {R(0), R(0), R(0)};
+            R UG[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
             const int row0 = q < n ? srow[q] : -1;
             if (row0 >= 0) {
                 const R *w = sw + 24 * q, *dw = w + 12;
                 const R Bv[3] = {sB[3 * q], sB[3 * q + 1], sB[3 * q + 2]};
                 const R wy = w[4 + b], wz = w[8 + c], dwy = dw[4 + b], dwz = dw[8 + c];
                 const int row = row0 + TS_Y * b + TS_Z * c;
+                // along x first: sum_a w_a A and sum_a w'_a (A . B)
+                R tx[3] = {R(0), R(0), R(0)}, dx = R(0);
 #pragma unroll
                 for (int a = 0; a < 4; ++a) {
                     const R A0 = tile[0][row + a], A1 = tile[1][row + a], A2 = tile[2][row + a];
-                    const R wxyz = w[a] * wy * wz;
-                    U[0] += wxyz * A0;
-                    U[1] += wxyz * A1;
-                    U[2] += wxyz * A2;
-                    const R sAB = A0 * Bv[0] + A1 * Bv[1] + A2 * Bv[2];
-                    G[0] += sAB * dw[a] * wy * wz;
-                    G[1] += sAB * w[a] * dwy * wz;
-                    G[2] += sAB * w[a] * wy * dwz;
+                    tx[0] += w[a] * A0;
+                    tx[1] += w[a] * A1;
+                    tx[2] += w[a] * A2;
+                    dx += dw[a] * (A0 * Bv[0] + A1 * Bv[1] + A2 * Bv[2]);
                 }
+                const R wyz = wy * wz, sx = tx[0] * Bv[0] + tx[1] * Bv[1] + tx[2] * Bv[2];
+                for (int d = 0; d < 3; ++d) UG[d] = wyz * tx[d];
+                UG[3] = dx * wyz;
+                UG[4] = sx * (dwy * wz);
+                UG[5] = sx * (wy * dwz);
             }
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1)
-                for (int d = 0; d < 3; ++d) {
-                    U[d] += __shfl_xor_sync(0xffffffffu, U[d], o);
-                    G[d] += __shfl_xor_sync(0xffffffffu, G[d], o);
-                }
+            R S[6];
+            sum16(UG, S);
             if (row0 >= 0 && (lane & 15) == 0) {
                 const size_t vid = (size_t)sperm[q];
                 for (int d = 0; d < 3; ++d) {
-                    if (out_interp) out_interp[3 * vid + d] = U[d];
-                    if (out_grad) out_grad[3 * vid + d] += G[d];
+                    if (out_interp) out_interp[3 * vid + d] = S[d];
+                    if (out_grad) out_grad[3 * vid + d] += S[3 + d];
                 }
             }
         }
@@ -1494,7 +1489,7 @@ void launch_bin_ranges(const View<R> &v, cudaStream_t st) {
 template <typename R>
 void launch_spread(const View<R> &v, cudaStream_t st) {
     if constexpr (std::is_same<R, float>::value) spread_tile_f32_kernel<<<v.nbins, SP_CHUNK, 0, st>>>(v);
-    else spread_tile_kernel<R><<<v.nbins, 256, 0, st>>>(v);
+    else spread_tile_kernel<R><<<3 * v.nbins, 256, 0, st>>>(v);
     if (v.nb[0] >= 3 && v.nb[1] >= 3 && v.nb[2] >= 3) spread_gather3_kernel<R><<<v.nbins, 256, 0, st>>>(v);
     else spread_gather_kernel<R><<<v.nbins, 256, 0, st>>>(v);
 }
