@@ -113,12 +113,13 @@ void hemo::set_last_error(const char *msg) { g_err = msg; }
 // device buffers of the reverse sweep (grown on demand, kept for reuse)
 struct AdjBuffers {
     void *lamf_in = nullptr, *lamf_out = nullptr, *lamu = nullptr, *lamF = nullptr, *amom = nullptr;
-    void *lamX = nullptr, *lamFv = nullptr, *grad = nullptr;
+    void *lamX = nullptr, *lamFv = nullptr, *grad = nullptr, *tri_rec = nullptr, *tri_part = nullptr, *ft = nullptr;
     void *fin_f = nullptr, *fin_u = nullptr, *fin_ctr = nullptr, *fin_off = nullptr, *cell_loss = nullptr, *dldx = nullptr;
     // per step of a segment
     void *seg_rec = nullptr, *seg_F = nullptr, *seg_u = nullptr, *seg_off = nullptr, *seg_Fv = nullptr;
     void *seg_anc_i = nullptr, *seg_anc_t = nullptr, *seg_perm = nullptr, *seg_start = nullptr;
     size_t sz_lamf_in = 0, sz_lamf_out = 0, sz_lamu = 0, sz_lamF = 0, sz_amom = 0, sz_lamX = 0, sz_lamFv = 0, sz_grad = 0;
+    size_t sz_tri_rec = 0, sz_tri_part = 0, sz_ft = 0;
     size_t sz_fin_f = 0, sz_fin_u = 0, sz_fin_ctr = 0, sz_fin_off = 0, sz_cell_loss = 0, sz_dldx = 0;
     size_t sz_seg_rec = 0, sz_seg_F = 0, sz_seg_u = 0, sz_seg_off = 0, sz_seg_Fv = 0;
     size_t sz_seg_anc_i = 0, sz_seg_anc_t = 0, sz_seg_perm = 0, sz_seg_start = 0;
@@ -624,9 +625,9 @@ int finalize_impl(hemo_sim *s) {
                         se[r].push_back(e);
                     }
                 at[r] = (int)items.size();
-                for (int t = 0; t < m.nt; ++t) {
-                    const int4 T = tri4[t];
-                    if (tin[t]) items.push_back(t << 1 | (std::min({T.x, T.y, T.z}) / per == r ? 1 : 0));
+                for (int q = 0; q < m.nt; ++q) {
+                    const int4 T = tri4[q];
+                    if (tin[q]) items.push_back(q << 1 | (std::min({T.x, T.y, T.z}) / per == r ? 1 : 0));
                 }
             }
             at[S] = (int)items.size();
@@ -650,6 +651,8 @@ int finalize_impl(hemo_sim *s) {
         d.kb = R(m.k_bend * m.kbt);
         d.k_area = m.k_area;
         d.k_volume = m.k_volume;
+        d.c_area = 0.5 * m.k_area / (m.A0 * m.A0);
+        d.c_volume = m.k_volume / (6.0 * m.V0 * m.V0);
         d.Ku = R(m.kbt / m.persistence);
         d.kbu = R(m.kbt);
         d.k_link = R(m.k_link);
@@ -914,7 +917,12 @@ int backward_impl(hemo_sim *s, const double *dL_dverts, double *grad, int ngrad)
         !need(b.fin_f, b.sz_fin_f, rs * Q * N) || !need(b.fin_u, b.sz_fin_u, rs * 3 * N) ||
         !need(b.fin_ctr, b.sz_fin_ctr, sizeof(double) * 3 * nc1) || !need(b.fin_off, b.sz_fin_off, rs * 3 * nv1))
         return fail(HEMO_ERR_OOM, "allocation of adjoint buffers failed");
+    if (std::is_same<R, double>::value &&
+        (!need(b.ft, b.sz_ft, rs * 3 * nv1) || !need(b.tri_rec, b.sz_tri_rec, rs * 8 * nc1 * (size_t)std::max(s->max_nt, 1)) ||
+         !need(b.tri_part, b.sz_tri_part, sizeof(double) * 4 * nc1 * (size_t)adjoint_chunks(std::max(s->max_nt, 1)))))
+        return fail(HEMO_ERR_OOM, "allocation of adjoint buffers failed");
     if (moved) clear_segment_graphs(s);  // captured pointers are stale
+    if (b.ft) HEMO_CU(cudaMemsetAsync(b.ft, 0, rs * 3 * nv1, st));
     View<R> v = make_view<R>(s);
     // final state, restored at the end
     launch_copy_natural<R>(v, s->precision, (int)(t_end & 1), (R *)b.fin_f, st);
@@ -936,6 +944,9 @@ int backward_impl(hemo_sim *s, const double *dL_dverts, double *grad, int ngrad)
     a.lamX = (R *)b.lamX;
     a.lamFv = (R *)b.lamFv;
     a.grad = (double *)b.grad;
+    a.tri_rec = (R *)b.tri_rec;
+    a.tri_part = (double *)b.tri_part;
+    a.ft = (R *)b.ft;
     a.ntypes = nt;
     int in_first = 0;  // which buffer holds the adjoint of f at the current step
     const long long nseg = (t_end - s->rec_start + K - 1) / K;

@@ -125,6 +125,7 @@ template <typename R> struct MeshDev {
     R m2;               // max_strain^2
     R kb;               // k_bend * kbt
     double k_area, k_volume;
+    double c_area, c_volume;  // 1/2 k_area / A0^2, k_volume / (6 V0^2)
     R Ku;               // kbt / persistence (link coefficient per unit k_link)
     R kbu;              // kbt (bending coefficient per unit k_bend)
     R k_link, k_bend;
@@ -239,6 +240,9 @@ template <typename R> struct AdjView {
     R *lamX;          // nv*3 adjoint of the vertex positions
     R *lamFv;         // nv*3 adjoint of the membrane forces
     double *grad;     // gradient accumulators (device)
+    R *tri_rec;       // FP64: ncell*max_nt*8 triangle records of the membrane adjoint
+    R *ft;            // FP64: nv*3 membrane terms of lamX (zero between the kernels)
+    double *tri_part; // FP64: ncell*adjoint_chunks(max_nt)*4 parts of A, dA, V, dV
     int ntypes;
 };
 
@@ -294,6 +298,7 @@ template <typename R> void launch_adj_moments(const View<R> &v, const AdjView<R>
 template <typename R> void launch_adj_collide(const View<R> &v, const AdjView<R> &a, cudaStream_t st);
 template <typename R> void launch_cell_adjoint(const View<R> &v, const AdjView<R> &a, cudaStream_t st);
 template <typename R> cudaError_t set_cell_adjoint_smem_limit(size_t bytes);
+inline int adjoint_chunks(int items) { return (items + 63) / 64; }  // CTAs of 64 items (FP64)
 template <typename R> size_t cell_adjoint_smem_bytes(int max_nv, int max_nt) { return (9 * (size_t)max_nv + 8 * (size_t)max_nt) * sizeof(R); }
 // FP32 gather form of the membrane adjoint: positions, direction, triangle
 // and edge records with their derivatives, 16 bytes each; used while it fits

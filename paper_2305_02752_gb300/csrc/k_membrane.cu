@@ -485,8 +485,8 @@ __global__ void __launch_bounds__(NT, CellMinBlocks<R, NT>::B) cell_kernel(View<
 //
 // Bound by the serial chain of a slice (FP64: the edges' atan2 and divisions on
 // its SM's FP64 pipe; FP32: latency).  Membrane phase, one CTA per cell -> the
-// cluster: FP64, 1 cell (16 slices) 168 -> 41 us, 30 cells (4) 168 -> 66 us; FP32,
-// 4 cells (16) 22.3 -> 18.5 us, 6 cells 22 -> 20 us.
+// cluster: FP64, 1 cell (16 slices) 168 -> 39 us, 30 cells (4) 168 -> 63 us; FP32,
+// 4 cells (16) 22.3 -> 16.3 us, 6 cells 22 -> 17.2 us.
 template <typename R> struct SliceThreads { static constexpr int T = CellMax<R>::T; };
 template <typename R>
 __global__ void __launch_bounds__(SliceThreads<R>::T, 1) cell_slices_kernel(View<R> v, int mode, double *stats) {
@@ -511,6 +511,11 @@ __global__ void __launch_bounds__(SliceThreads<R>::T, 1) cell_slices_kernel(View
     __shared__ R cav[2];
     const int per = (m.nv + S - 1) / S, v0 = min(m.nv, slice * per), v1 = min(m.nv, v0 + per);
     const int t0 = m.sl_at[slice], t1 = m.sl_at[slice + 1], e0 = m.sl_at[S + 1 + slice], e1 = m.sl_at[S + 2 + slice];
+    // this thread's first triangle and edge and its vertex's fan are requested
+    // ahead (a slice has about one item per thread, so nothing else hides their
+    // latency)
+    const int tf = t0 + (int)threadIdx.x, ef = e0 + (int)threadIdx.x;
+    const int ti = tf < t1 ? __ldg(m.sl_items + tf) : -1, ei = mode == 0 && ef < e1 ? __ldg(m.sl_items + ef) : -1;
 
     // mean offset and re-base, as in cell_kernel
     constexpr int KC = 4;
@@ -530,6 +535,19 @@ __global__ void __launch_bounds__(SliceThreads<R>::T, 1) cell_slices_kernel(View
     }
     for (int i = threadIdx.x + KC * NT; i < m.nv; i += NT)
         for (int k = 0; k < 3; ++k) mean[k] += v.off[3 * (size_t)(first + i) + k];
+    int4 Tf = make_int4(0, 0, 0, 0), Ef = Tf;
+    int2 Uf = make_int2(0, 0);
+    R lf = R(0), hf = R(0);
+    if (ti >= 0) Tf = __ldg(m.tri4 + (ti >> 1));
+    if (ei >= 0) {
+        Ef = __ldg(reinterpret_cast<const int4 *>(m.edge) + ei);
+        Uf = __ldg(reinterpret_cast<const int2 *>(m.etri) + ei);
+        lf = __ldg(m.invL0 + ei);
+        hf = __ldg(m.th0 + ei);
+    }
+    if (mode == 0 && v0 + (int)threadIdx.x < v1)
+        for (int k = 0; k <= m.maxv; ++k)
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(m.vfan + (size_t)k * m.nv + v0 + threadIdx.x));
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -578,9 +596,9 @@ __global__ void __launch_bounds__(SliceThreads<R>::T, 1) cell_slices_kernel(View
 
     // the slice's triangles: records, and the sums over those it owns
     Acc<R> sum[2];
-    for (int q = t0 + threadIdx.x; q < t1; q += NT) {
-        const int id = m.sl_items[q], t = id >> 1;
-        const int4 T = __ldg(m.tri4 + t);
+    for (int q = tf; q < t1; q += NT) {
+        const int id = q == tf ? ti : __ldg(m.sl_items + q), t = id >> 1;
+        const int4 T = q == tf ? Tf : __ldg(m.tri4 + t);
         if (!tri_ok(m, T, v.status)) continue;
         R area, vol;
         tri_record(m, xs, tn, tl, t, T, area, vol);
@@ -620,12 +638,17 @@ __global__ void __launch_bounds__(SliceThreads<R>::T, 1) cell_slices_kernel(View
 
     double G[6] = {};  // gyration sums, in cell_kernel's order: the deformation index of a disc is sensitive to their rounding
     if (mode == 0) {
-        for (int q = e0 + threadIdx.x; q < e1; q += NT) {
-            const int e = m.sl_items[q];
-            const int4 E = __ldg(reinterpret_cast<const int4 *>(m.edge) + e);
-            const int2 T = __ldg(reinterpret_cast<const int2 *>(m.etri) + e);
-            if (!edge_ok(m, E, T, v.status)) continue;
-            edge_record(m, xs, tn, es, e, E, T, __ldg(m.invL0 + e), __ldg(m.th0 + e), v.status);
+        for (int q = ef; q < e1; q += NT) {
+            int e = ei;
+            if (q != ef) {
+                e = __ldg(m.sl_items + q);
+                Ef = __ldg(reinterpret_cast<const int4 *>(m.edge) + e);
+                Uf = __ldg(reinterpret_cast<const int2 *>(m.etri) + e);
+                lf = __ldg(m.invL0 + e);
+                hf = __ldg(m.th0 + e);
+            }
+            if (!edge_ok(m, Ef, Uf, v.status)) continue;
+            edge_record(m, xs, tn, es, e, Ef, Uf, lf, hf, v.status);
         }
     } else if (slice == 0) {
         Acc<R> g[6];
@@ -661,14 +684,14 @@ __global__ void __launch_bounds__(SliceThreads<R>::T, 1) cell_slices_kernel(View
         }
         return;
     }
-    if (threadIdx.x == 0) {
-        double A = 0, V = 0;
-        for (int r = 0; r < S; ++r) {
-            A += part[r][0];
-            V += part[r][1];
+    if (wid == 0) {  // (lanes of the parts: FP64 additions have a long latency)
+        double A = lane < S ? part[lane][0] : 0.0, V = lane < S ? part[lane][1] : 0.0;
+        for (int o = MAX_SLICES / 2; o > 0; o >>= 1) {
+            A += __shfl_xor_sync(0xffffffffu, A, o);
+            V += __shfl_xor_sync(0xffffffffu, V, o);
         }
-        cav[0] = R(0.5 * m.k_area * (A - m.A0) / (m.A0 * m.A0));
-        cav[1] = R(m.k_volume * (V - m.V0) / (m.V0 * m.V0) / 6.0);
+        if (lane == 0) cav[0] = R(m.c_area * (A - m.A0));
+        if (lane == 1) cav[1] = R(m.c_volume * (V - m.V0));
     }
     __syncthreads();
     const R ha = cav[0], sv = cav[1];
@@ -840,6 +863,134 @@ __global__ void __launch_bounds__(NT, CellMinBlocks<R, NT>::B) cell_adjoint_kern
         for (int i = threadIdx.x; i < 3 * m.nv; i += blockDim.x) a.lamX[3 * (size_t)first + i] += ft[i];
     else
         for (int i = threadIdx.x; i < 3 * m.nv; i += blockDim.x) atomicAdd(a.lamX + 3 * (size_t)first + i, ft[i]);
+}
+
+// FP64 form of the membrane adjoint in two kernels over small CTAs, so that
+// the items of a few cells occupy every SM's FP64 pipe: triangle records (n,
+// dn, 1/|n|^2 and its derivative) and each CTA's part of A, dA, V, dV into
+// global memory; then the edge and triangle terms, summed per vertex and into
+// the gradients with atomics.  (A third adds the sums to lamX: the terms are
+// small against it, and added one by one they lost seven digits.)  One CTA per cell (or per slice of one, each with
+// all records of the cell) kept an SM busy with the records for 96 us.
+// 32^3 box, one cell: 109 -> 8.4 + 17.7 + 2.3 us.
+constexpr int ADJ_NT = 64;  // items per CTA
+__device__ __forceinline__ V3<Dual<double>> vertex_dual(const View<double> &v, const AdjView<double> &a, size_t i) {
+    return dld3(v.off + 3 * i, a.lamFv + 3 * i);
+}
+__global__ void __launch_bounds__(ADJ_NT) adjoint_records_kernel(View<double> v, AdjView<double> a, int chunks) {
+    using D = Dual<double>;
+    const int c = blockIdx.x / chunks, chunk = blockIdx.x % chunks;
+    const MeshDev<double> m = v.meshes[v.cell_type[c]];
+    const size_t first = v.cell_first[c];
+    __shared__ double scratch[4][32];
+    Acc<double> av[4];  // A, dA, V, dV
+    const int t = chunk * ADJ_NT + threadIdx.x;
+    if (t < m.nt) {
+        const int4 T = __ldg(m.tri4 + t);
+        const V3<D> p0 = vertex_dual(v, a, first + T.x), p1 = vertex_dual(v, a, first + T.y), p2 = vertex_dual(v, a, first + T.z);
+        const V3<D> n = cross(p1 - p0, p2 - p0);
+        const D q = dot(n, n);
+        const D iq = dconst(1.0) / q;
+        double *o = a.tri_rec + 8 * ((size_t)c * v.max_nt + t);
+        o[0] = n.x.v; o[1] = n.y.v; o[2] = n.z.v;
+        o[3] = n.x.t; o[4] = n.y.t; o[5] = n.z.t;
+        o[6] = iq.v; o[7] = iq.t;
+        const D ar = dconst(0.5) * dsqrt(q), vo = dot(p0, cross(p1, p2));
+        av[0].add(ar.v);
+        av[1].add(ar.t);
+        av[2].add(vo.v / 6.0);
+        av[3].add(vo.t / 6.0);
+    }
+    double AV[4];
+    block_total<double, 4>(av, AV, scratch);
+    if (threadIdx.x < 4) a.tri_part[4 * ((size_t)c * chunks + chunk) + threadIdx.x] = scratch[threadIdx.x][31];
+}
+
+__global__ void __launch_bounds__(ADJ_NT) adjoint_terms_kernel(View<double> v, AdjView<double> a, int chunks, int echunks) {
+    using D = Dual<double>;
+    using R = double;
+    const int c = blockIdx.x / (chunks + echunks), chunk = blockIdx.x % (chunks + echunks);
+    const int type = v.cell_type[c];
+    const MeshDev<R> m = v.meshes[type];
+    const size_t first = v.cell_first[c];
+    const R *rec = a.tri_rec + 8 * (size_t)c * v.max_nt;
+    __shared__ double scratch[2][32];
+    auto add = [&](int i, R s, V3<R> f) { add_into(a.ft + 3 * (first + i), s, f); };
+    Acc<R> th[2];  // lamFv . unit-modulus forces: link and bend, or area and volume
+    const bool edges = chunk < echunks;
+    if (edges) {
+        const int e = chunk * ADJ_NT + threadIdx.x;
+        if (e < m.ne) {
+            const int4 E = __ldg(reinterpret_cast<const int4 *>(m.edge) + e);
+            const int2 T = __ldg(reinterpret_cast<const int2 *>(m.etri) + e);
+            const V3<D> p0 = vertex_dual(v, a, first + E.x), p1 = vertex_dual(v, a, first + E.y);
+            const V3<D> pa = vertex_dual(v, a, first + E.z), pb = vertex_dual(v, a, first + E.w);
+            const V3<R> l0 = tans(p0), l1 = tans(p1), la = tans(pa), lb = tans(pb);
+            const V3<D> ed = p1 - p0;
+            const D L = dsqrt(dot(ed, ed));
+            const D iL = dconst(R(1)) / L;
+            const D eps = L * dconst(m.invL0[e]) - dconst(R(1));
+            const D den = dconst(m.m2) - eps * eps;
+            const D dEdL = dconst(m.Ku) * (eps + eps / den);
+            const V3<D> u0 = (dEdL * iL) * ed;  // unit link force on v0; -u0 on v1
+            th[0].add(dot(l0, vals(u0)) - dot(l1, vals(u0)));
+            const R *r1 = rec + 8 * T.x, *r2 = rec + 8 * T.y;
+            const V3<D> n1 = dld3(r1, r1 + 3), n2 = dld3(r2, r2 + 3);
+            const V3<D> a1 = D{r1[6], r1[7]} * n1, a2 = D{r2[6], r2[7]} * n2;
+            const D thd = datan2(dot(cross(n1, n2), ed) * iL, dot(n1, n2));
+            const D cb = dconst(m.kbu) * (thd - dconst(m.th0[e]));
+            const D sa0 = dot(pa - p1, ed) * iL, sb0 = dot(pb - p1, ed) * iL;
+            const D sa1 = dot(pa - p0, ed) * iL, sb1 = dot(pb - p0, ed) * iL;
+            const V3<D> fa = (cb * L) * a1, fb = (cb * L) * a2;
+            const V3<D> f0 = cb * (sa0 * a1 + sb0 * a2);
+            const V3<D> f1 = (dconst(R(0)) - cb) * (sa1 * a1 + sb1 * a2);
+            add(E.z, m.k_bend, tans(fa));
+            add(E.w, m.k_bend, tans(fb));
+            add(E.x, R(1), m.k_link * tans(u0) + m.k_bend * tans(f0));
+            add(E.y, R(1), m.k_bend * tans(f1) - m.k_link * tans(u0));
+            th[1].add(dot(la, vals(fa)) + dot(lb, vals(fb)) + dot(l0, vals(f0)) + dot(l1, vals(f1)));
+        }
+    } else {
+        __shared__ R cuv[4];  // the area and volume strain factors and their derivatives
+        if (threadIdx.x < 4) {
+            R s = R(0);
+            for (int q = 0; q < chunks; ++q) s += a.tri_part[4 * ((size_t)c * chunks + q) + threadIdx.x];
+            if (threadIdx.x == 0) s -= m.A0;
+            if (threadIdx.x == 2) s -= m.V0;
+            cuv[threadIdx.x] = threadIdx.x < 2 ? s / (m.A0 * m.A0) : s / (m.V0 * m.V0);
+        }
+        __syncthreads();
+        const D ua = {cuv[0], cuv[1]}, uv = {cuv[2], cuv[3]};
+        const int t = (chunk - echunks) * ADJ_NT + threadIdx.x;
+        if (t < m.nt) {
+            const int4 T = __ldg(m.tri4 + t);
+            const int j[3] = {T.x, T.y, T.z};
+            const V3<D> p[3] = {vertex_dual(v, a, first + T.x), vertex_dual(v, a, first + T.y), vertex_dual(v, a, first + T.z)};
+            const R *r = rec + 8 * t;
+            const V3<D> nh = dsqrt(D{r[6], r[7]}) * dld3(r, r + 3);
+            const R kA = m.k_area, kV = m.k_volume;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const V3<D> &pk1 = p[(k + 1) % 3], &pk2 = p[(k + 2) % 3];
+                const V3<D> fa = (dconst(R(-0.5)) * ua) * cross(nh, pk2 - pk1);
+                const V3<D> fv = (dconst(R(-1) / R(6)) * uv) * cross(pk1, pk2);
+                add(j[k], R(1), kA * tans(fa) + kV * tans(fv));
+                const V3<R> lk = tans(p[k]);
+                th[0].add(dot(lk, vals(fa)));
+                th[1].add(dot(lk, vals(fv)));
+            }
+        }
+    }
+    double TH[2];
+    block_total<R, 2>(th, TH, scratch);
+    if (threadIdx.x < 2) atomicAdd(a.grad + 4 * type + (edges ? 0 : 2) + threadIdx.x, scratch[threadIdx.x][31]);
+}
+
+__global__ void __launch_bounds__(256) adjoint_add_kernel(AdjView<double> a, int n) {
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= n) return;
+    a.lamX[i] += a.ft[i];
+    a.ft[i] = 0.0;
 }
 
 // FP32 form of the membrane adjoint as a gather, in the forward kernel's
@@ -1150,20 +1301,28 @@ void launch_cell_adjoint(const View<R> &v, const AdjView<R> &a, cudaStream_t st)
             return;
         }
     }
-    const size_t smem = cell_adjoint_smem_bytes<R>(v.max_nv, v.max_nt);
-    // few cells: spread each over several CTAs (FP64 arithmetic is slow per
-    // SM, so the work goes to as many SMs as there are)
-    const int slices = std::max(1, std::min(32, v.nsm / v.ncell));
-    if (slices == 1 && cell_wide(v)) cell_adjoint_kernel<R, CellMax<R>::T><<<v.ncell, CellMax<R>::T, smem, st>>>(v, a, 1);
-    else cell_adjoint_kernel<R, 256><<<v.ncell * slices, 256, smem, st>>>(v, a, slices);
+    if constexpr (std::is_same<R, double>::value) {
+        const int chunks = adjoint_chunks(v.max_nt), echunks = adjoint_chunks(v.max_ne);
+        adjoint_records_kernel<<<v.ncell * chunks, ADJ_NT, 0, st>>>(v, a, chunks);
+        adjoint_terms_kernel<<<v.ncell * (chunks + echunks), ADJ_NT, 0, st>>>(v, a, chunks, echunks);
+        adjoint_add_kernel<<<(3 * v.nv + 255) / 256, 256, 0, st>>>(a, 3 * v.nv);
+    } else {  // meshes whose gather records do not fit
+        const size_t smem = cell_adjoint_smem_bytes<R>(v.max_nv, v.max_nt);
+        const int slices = std::max(1, std::min(32, v.nsm / v.ncell));
+        if (slices == 1 && cell_wide(v)) cell_adjoint_kernel<R, CellMax<R>::T><<<v.ncell, CellMax<R>::T, smem, st>>>(v, a, 1);
+        else cell_adjoint_kernel<R, 256><<<v.ncell * slices, 256, smem, st>>>(v, a, slices);
+    }
 }
 
 template <typename R>
 cudaError_t set_cell_adjoint_smem_limit(size_t bytes) {
+    if constexpr (std::is_same<R, double>::value) return cudaSuccess;  // (its kernels use none)
+    else {
     cudaError_t e = cudaFuncSetAttribute(cell_adjoint_kernel<R, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess && CellMax<R>::T != 256)
         e = cudaFuncSetAttribute(cell_adjoint_kernel<R, CellMax<R>::T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     return e;
+    }
 }
 
 cudaError_t set_cell_adjoint_gather_smem_limit(size_t bytes) {
