@@ -745,6 +745,18 @@ double dihedral(D3 p0, D3 p1, D3 pa, D3 pb) {
     return std::atan2(dt3(crs(n1, n2), e) / std::sqrt(dt3(e, e)), dt3(n1, n2));
 }
 
+// whether a kernel on the current device can write elements of `size` bytes at p:
+// device memory of that device, aligned
+bool direct_out(const void *p, size_t size) {
+    cudaPointerAttributes at;
+    int dev = -1;
+    if ((uintptr_t)p % size || cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+
 int copy_out(hemo_sim *s, void *dst, const void *src, size_t bytes) {
     if (!dst || !bytes) return HEMO_OK;
     HEMO_CU(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, s->stream));
@@ -1538,10 +1550,9 @@ int hemo_get_inside(hemo_sim *s, uint8_t *inside) {
 int hemo_sync(hemo_sim *s) {
     NvtxRange nvtx_("hemo_sync");
     if (!s) return fail(HEMO_ERR_ARG, "null simulation");
-    HEMO_CU(cudaStreamSynchronize(s->stream));
-    unsigned st = 0;
-    HEMO_CU(cudaMemcpy(&st, s->status, sizeof(unsigned), cudaMemcpyDeviceToHost));
-    s->sticky |= st;
+    HEMO_CU(cudaMemcpyAsync(s->status_host, s->status, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
+    HEMO_CU(cudaStreamSynchronize(s->stream));  // (one wait for the stream's work and the status word)
+    s->sticky |= *s->status_host;
     s->ev_pending = false;
     return status_code(s->sticky);
 }
@@ -1570,34 +1581,48 @@ int hemo_get_fields(hemo_sim *s, unsigned what, void *rho, void *u, double *vert
     if (!s) return fail(HEMO_ERR_ARG, "null simulation");
     int rc = ensure_ready(s);
     if (rc) return rc;
-    const size_t N = (size_t)s->N, rs = rsize(s);
+    const size_t N = (size_t)s->N, rs = rsize(s), vb = sizeof(double) * 3 * (size_t)s->nv,
+                 cb = sizeof(double) * 6 * (size_t)s->ncell;
     const int layout = s->le ? 0 : (int)(s->steps_done & 1);  // (two-array streaming: natural order)
-    size_t need = std::max<size_t>({rs * 3 * N, sizeof(double) * 6 * (size_t)std::max(s->nv, 1),
-                                    sizeof(double) * 6 * (size_t)std::max(s->ncell, 1)});
-    rc = ensure_staging(s, need);
-    if (rc) return rc;
     cudaStream_t st = s->stream;
-    if ((what & HEMO_RHO) && rho) {
-        if (is_f64(s)) launch_rho_out<double>(make_view<double>(s), s->precision, layout, (double *)s->staging, st);
-        else launch_rho_out<float>(make_view<float>(s), s->precision, layout, (float *)s->staging, st);
-        if ((rc = copy_out(s, rho, s->staging, rs * N))) return rc;
+    const bool want_rho = (what & HEMO_RHO) && rho, want_u = (what & HEMO_U) && u;
+    const bool want_x = (what & HEMO_VERTS) && verts && s->nv, want_f = (what & HEMO_FORCES) && forces && s->nv;
+    const bool want_c = (what & HEMO_CELLSTATS) && cellstats && s->ncell;
+    // the kernels write fields straight into the caller's device memory; host
+    // memory (and pointers that are not aligned to an element) goes through the
+    // staging buffer and a copy (1000 x 208 x 208 pipe, all fields: 2.5 GB of
+    // traffic less)
+    const bool d_rho = want_rho && direct_out(rho, rs), d_u = want_u && direct_out(u, rs),
+               d_x = want_x && direct_out(verts, sizeof(double)), d_f = want_f && direct_out(forces, sizeof(double)),
+               d_c = want_c && direct_out(cellstats, sizeof(double));
+    const size_t need = std::max<size_t>({want_rho && !d_rho ? rs * N : 0, want_u && !d_u ? rs * 3 * N : 0,
+                                          (want_x && !d_x) || (want_f && !d_f) ? 2 * vb : 0, want_c && !d_c ? cb : 0});
+    if (need && (rc = ensure_staging(s, need))) return rc;
+    if (want_rho) {
+        void *o = d_rho ? rho : s->staging;
+        if (is_f64(s)) launch_rho_out<double>(make_view<double>(s), s->precision, layout, (double *)o, st);
+        else launch_rho_out<float>(make_view<float>(s), s->precision, layout, (float *)o, st);
+        if (!d_rho && (rc = copy_out(s, rho, o, rs * N))) return rc;
     }
-    if ((what & HEMO_U) && u) {
-        if (is_f64(s)) launch_u_out<double>(make_view<double>(s), (double *)s->staging, st);
-        else launch_u_out<float>(make_view<float>(s), (float *)s->staging, st);
-        if ((rc = copy_out(s, u, s->staging, rs * 3 * N))) return rc;
+    if (want_u) {
+        void *o = d_u ? u : s->staging;
+        if (is_f64(s)) launch_u_out<double>(make_view<double>(s), (double *)o, st);
+        else launch_u_out<float>(make_view<float>(s), (float *)o, st);
+        if (!d_u && (rc = copy_out(s, u, o, rs * 3 * N))) return rc;
     }
-    if (((what & HEMO_VERTS) && verts) || ((what & HEMO_FORCES) && forces)) {
-        double *X = (double *)s->staging, *Fo = X + 3 * (size_t)s->nv;
+    if (want_x || want_f) {
+        double *X = !want_x ? nullptr : (d_x ? verts : (double *)s->staging);
+        double *Fo = !want_f ? nullptr : (d_f ? forces : (double *)s->staging + 3 * (size_t)s->nv);
         if (is_f64(s)) launch_verts_out<double>(make_view<double>(s), X, Fo, st);
         else launch_verts_out<float>(make_view<float>(s), X, Fo, st);
-        if ((what & HEMO_VERTS) && (rc = copy_out(s, verts, X, sizeof(double) * 3 * s->nv))) return rc;
-        if ((what & HEMO_FORCES) && (rc = copy_out(s, forces, Fo, sizeof(double) * 3 * s->nv))) return rc;
+        if (want_x && !d_x && (rc = copy_out(s, verts, X, vb))) return rc;
+        if (want_f && !d_f && (rc = copy_out(s, forces, Fo, vb))) return rc;
     }
-    if ((what & HEMO_CELLSTATS) && cellstats && s->ncell) {
-        if (is_f64(s)) launch_cell_forces<double>(make_view<double>(s), 1, (double *)s->staging, st);
-        else launch_cell_forces<float>(make_view<float>(s), 1, (double *)s->staging, st);
-        if ((rc = copy_out(s, cellstats, s->staging, sizeof(double) * 6 * s->ncell))) return rc;
+    if (want_c) {
+        double *o = d_c ? cellstats : (double *)s->staging;
+        if (is_f64(s)) launch_cell_forces<double>(make_view<double>(s), 1, o, st);
+        else launch_cell_forces<float>(make_view<float>(s), 1, o, st);
+        if (!d_c && (rc = copy_out(s, cellstats, o, cb))) return rc;
     }
     HEMO_CU(cudaGetLastError());
     return hemo_sync(s);

@@ -854,6 +854,35 @@ __global__ void u_out_kernel(View<R> v, R *out) {
     out[3 * (size_t)n + 2] = v.u[2 * N + n];
 }
 
+// FP32, four nodes per thread: 16-byte loads of each component, the nodes'
+// components interleaved in shared memory, 16-byte stores (one node per thread
+// stores with a stride of 12 bytes: 284 us on the pipe, this 144)
+constexpr int UOUT_NT = 256;
+__global__ void __launch_bounds__(UOUT_NT) u_out_vec_kernel(View<float> v, float *out) {
+    __shared__ float s[12 * UOUT_NT];
+    const size_t N = (size_t)v.N, n0 = (size_t)blockIdx.x * 4 * UOUT_NT;
+    const size_t n = n0 + 4 * threadIdx.x;
+    if (n < N) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const float4 q = *reinterpret_cast<const float4 *>(v.u + d * N + n);
+            float *o = s + 12 * threadIdx.x + d;
+            o[0] = q.x;
+            o[3] = q.y;
+            o[6] = q.z;
+            o[9] = q.w;
+        }
+    }
+    __syncthreads();
+    const size_t words = 3 * (N - n0) / 4;  // 16-byte words left
+    float4 *o = reinterpret_cast<float4 *>(out + 3 * n0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int w = threadIdx.x + k * UOUT_NT;
+        if ((size_t)w < words) o[w] = reinterpret_cast<const float4 *>(s)[w];
+    }
+}
+
 // Wall links: for each fluid node, the wall id of node + c_i (2 bits per
 // direction; nodes beyond a non-periodic edge are resting walls).
 __global__ void build_links_kernel(int nx, int ny, int nz, int px, int py, int pz, uint8_t *ntype,
@@ -1087,6 +1116,13 @@ void launch_rho_out(const View<R> &v, int precision, int layout, R *out, cudaStr
 
 template <typename R>
 void launch_u_out(const View<R> &v, R *out, cudaStream_t st) {
+    if constexpr (std::is_same<R, float>::value) {
+        // (N a multiple of 4 keeps every component's start aligned with the first)
+        if (v.N % 4 == 0 && (((uintptr_t)v.u | (uintptr_t)out) & 15) == 0) {
+            u_out_vec_kernel<<<nblocks(v.N, 4 * UOUT_NT), UOUT_NT, 0, st>>>(v, out);
+            return;
+        }
+    }
     u_out_kernel<R><<<nblocks(v.N, 256), 256, 0, st>>>(v, out);
 }
 
