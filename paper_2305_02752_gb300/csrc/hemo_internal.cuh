@@ -209,6 +209,8 @@ template <typename R> struct View {
     const float2 *rref;
     int node_pairs;            // 16-bit storage, nx even: PAIR_* bits, kernels that take two nodes per thread
     int stalled_wait_test;     // staged collision: first wait on a barrier nothing completes (HEMO_OPT_TEST_STALLED_WAIT)
+    int flat;                  // per-node lattice kernels: threads over a plane's consecutive nodes (set by their launchers)
+    unsigned rdiv;             // 2^32 / nx rounded up (flat)
     int wide_index;            // lattice kernels: 64-bit population indices on any lattice (HEMO_OPT_WIDE_INDEX)
     // interpolation staging by tensor copies: the host-side tensor map of u
     // (CUtensorMap, 4-D: x, y, z, component) and the array it describes;
