@@ -192,6 +192,50 @@ __global__ void scatter_kernel(const int *key, int *cursor, int *perm_raw, int n
     if (index_ok(slot >= 0 && slot < nv, status)) perm_raw[slot] = i;
 }
 
+// Few blocks and vertices: scan and scatter by one CTA, the cursors in shared
+// memory (48^3 box, 2568 vertices: 4.1 us against 2.6 + 2.5 and the gap between
+// two launches).  Above these sizes one SM is the slower.
+constexpr int SMALL_BINS = 4096, SMALL_NV = 8192;
+__global__ void __launch_bounds__(1024) scan_scatter_kernel(int *counts, int *start, int nbins, const int *key, int *perm,
+                                                            int nv, unsigned *status) {
+    __shared__ int cur[SMALL_BINS];
+    __shared__ int wsum[32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const bool vec = ((uintptr_t)counts & 15) == 0;
+    const int k0 = 4 * t;
+    const int4 c = load_quad(counts, k0, nbins, vec);
+    const int own = c.x + c.y + c.z + c.w;
+    int x = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[w] = x;
+    __syncthreads();
+    const int total = wsum[lane];
+    const int before = __reduce_add_sync(0xffffffffu, lane < w ? total : 0);
+    const int e0 = before + x - own;
+    const int4 ex = make_int4(e0, e0 + c.x, e0 + c.x + c.y, e0 + c.x + c.y + c.z);
+    store_quad(start, k0, nbins, vec && ((uintptr_t)start & 15) == 0, ex);
+    store_quad(counts, k0, nbins, vec, make_int4(0, 0, 0, 0));
+    store_quad(cur, k0, nbins, true, ex);
+    if (t == 1023) start[nbins] = e0 + own;
+    __syncthreads();
+    for (int i = t; i < nv; i += 1024) {
+        const int k = key[i];
+        const unsigned act = __activemask();
+        const unsigned grp = __match_any_sync(act, k);
+        const int leader = __ffs(grp) - 1;
+        int base = 0;
+        const bool ok = index_ok(k >= 0 && k < nbins, status);
+        if (lane == leader && ok) base = atomicAdd(cur + k, __popc(grp));
+        base = __shfl_sync(act, base, leader);
+        const int slot = base + __popc(grp & ((1u << lane) - 1u));
+        if (ok && index_ok(slot >= 0 && slot < nv, status)) perm[slot] = i;
+    }
+}
+
 // One warp per block: each id's rank among the block's ids (ids are unique)
 // is its position.  Segments of up to SORT_SMEM ids are ranked from shared
 // memory, SORT_K ids per lane at a time held in registers (one pass over the
@@ -1397,18 +1441,20 @@ __global__ void __launch_bounds__(256) vertex_field_v4_kernel(View<float> v, con
     }
     __syncthreads();
     const size_t N = (size_t)v.N;
-    for (int q = threadIdx.x; q < TILE3; q += blockDim.x) {
-        const int l0 = q % TILE, l1 = (q / TILE) % TILE, l2 = q / (TILE * TILE);
-        const int jx = jtab[0][l0], jy = jtab[1][l1], jz = jtab[2][l2];
-        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+    TileWalk tw(threadIdx.x, blockDim.x);
+    for (int q = threadIdx.x; q < TILE3; q += blockDim.x, tw.next()) {  // (asynchronous: all loads in flight at once)
+        const int jx = jtab[0][tw.l0], jy = jtab[1][tw.l1], jz = jtab[2][tw.l2];
+        float4 *dst = tile + tw.l0 + TS_Y * tw.l1 + TS_Z * tw.l2;
         if ((jx | jy | jz) >= 0) {
             const size_t n = (size_t)jx + (size_t)v.nx * ((size_t)jy + (size_t)v.ny * jz);
-            t.x = A[n];
-            t.y = A[N + n];
-            t.z = A[2 * N + n];
+            cp_async4(&dst->x, A + n);
+            cp_async4(&dst->y, A + N + n);
+            cp_async4(&dst->z, A + 2 * N + n);
+        } else {
+            *dst = make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        tile[l0 + TS_Y * l1 + TS_Z * l2] = t;
     }
+    cp_async_wait_all();
     __syncthreads();
     for (int j = s + threadIdx.x; j < e; j += blockDim.x) {
         const int i = v.perm[j];
@@ -1523,7 +1569,12 @@ void launch_bins(const View<R> &v, cudaStream_t st, bool stable) {
 
 template <typename R>
 void launch_bin_ranges(const View<R> &v, cudaStream_t st) {
-    scan_kernel<<<1, 1024, 0, st>>>(v.counts, v.start, v.cursor, v.nbins + (v.le ? 1 : 0));  // (+ the Lees-Edwards bin)
+    const int nbins = v.nbins + (v.le ? 1 : 0);  // (+ the Lees-Edwards bin)
+    if (nbins <= SMALL_BINS && v.nv <= SMALL_NV) {
+        scan_scatter_kernel<<<1, 1024, 0, st>>>(v.counts, v.start, nbins, v.key, v.perm, v.nv, v.status);
+        return;
+    }
+    scan_kernel<<<1, 1024, 0, st>>>(v.counts, v.start, v.cursor, nbins);
     scatter_kernel<<<nblocks(v.nv, 256), 256, 0, st>>>(v.key, v.cursor, v.perm, v.nv, v.status);
 }
 
