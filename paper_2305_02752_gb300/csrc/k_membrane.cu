@@ -352,12 +352,11 @@ __global__ void __launch_bounds__(NT, CellMinBlocks<R, NT>::B) cell_kernel(View<
     if (threadIdx.x == 0) {
         for (int k = 0; k < 3; ++k) cnew[k] = v.ctr[3 * c + k] + (double)mean[k];
         if (v.le && mode == 0) {  // Lees-Edwards: a centroid that left through z = 0 or nz moves to the other side
-            const double D = le_shift(v);
             if (cnew[2] >= v.nz) {
-                cnew[0] -= D;
+                cnew[0] -= le_shift(v);
                 cnew[2] -= v.nz;
             } else if (cnew[2] < 0) {
-                cnew[0] += D;
+                cnew[0] += le_shift(v);
                 cnew[2] += v.nz;
             }
         }
@@ -566,12 +565,11 @@ __global__ void __launch_bounds__(SliceThreads<R>::T, 1) cell_slices_kernel(View
     __syncthreads();
     if (threadIdx.x == 0) {
         if (v.le && mode == 0) {  // Lees-Edwards: a centroid that left through z = 0 or nz moves to the other side
-            const double D = le_shift(v);
             if (cnew[2] >= v.nz) {
-                cnew[0] -= D;
+                cnew[0] -= le_shift(v);
                 cnew[2] -= v.nz;
             } else if (cnew[2] < 0) {
-                cnew[0] += D;
+                cnew[0] += le_shift(v);
                 cnew[2] += v.nz;
             }
         }
