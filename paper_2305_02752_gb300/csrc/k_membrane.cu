@@ -999,10 +999,12 @@ __global__ void __launch_bounds__(256) adjoint_add_kernel(AdjView<double> a, int
 // lamX; the value parts, dotted with lamFv, give the unit-modulus terms
 // summed into the gradients of the four moduli.  No shared atomics.
 //
-// With fewer cells than SMs each cell takes `slices` CTAs: every CTA builds
-// the cell's triangle and edge records, then walks the fans of its share of
-// the vertices only (each vertex's lamX written by one CTA; the modulus
-// terms added with one atomic per CTA).
+// With few cells each cell takes View::slices CTAs: every CTA builds the cell's
+// triangle records (and the sums, in the same order), the edge records that the
+// fans of its vertices read (the forward kernel's lists), then walks those fans
+// (each vertex's lamX written by one CTA; the modulus terms added with one
+// atomic per CTA).  48^3 box, 4 cells, 16 slices: 17.4 us (8 slices with all
+// edge records each: 21.7).
 template <int NT>
 __global__ void __launch_bounds__(NT, 1) cell_adjoint_gather_kernel(View<float> v, AdjView<float> a, int slices) {
     using R = float;
@@ -1025,6 +1027,16 @@ __global__ void __launch_bounds__(NT, 1) cell_adjoint_gather_kernel(View<float> 
         return {{p.x, q.x}, {p.y, q.y}, {p.z, q.z}};
     };
     auto st4 = [](R *o, R x, R y, R z, R w) { *reinterpret_cast<float4 *>(o) = make_float4(x, y, z, w); };
+    // with slices this CTA's share of the vertices and edges; the first edge and
+    // the fans are requested ahead
+    const int per = (m.nv + slices - 1) / slices, i0 = min(m.nv, slice * per), i1 = min(m.nv, i0 + per);
+    const int *items = slices > 1 ? m.sl_items : nullptr;
+    const int e0 = items ? m.sl_at[slices + 1 + slice] : 0, e1 = items ? m.sl_at[slices + 2 + slice] : m.ne;
+    int ei = e0 + (int)threadIdx.x;
+    if (items && ei < e1) ei = __ldg(items + ei);
+    if (i0 + (int)threadIdx.x < i1)
+        for (int k = 0; k <= m.maxv; ++k)
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(m.vfan + (size_t)k * m.nv + i0 + threadIdx.x));
     for (int i = threadIdx.x; i < m.nv; i += blockDim.x) {  // re-based offsets of the forward step
         const R *o = v.off + 3 * (size_t)(first + i), *l = a.lamFv + 3 * (size_t)(first + i);
         st4(xv + 4 * i, o[0], o[1], o[2], R(0));
@@ -1050,15 +1062,15 @@ __global__ void __launch_bounds__(NT, 1) cell_adjoint_gather_kernel(View<float> 
     }
     double AV[4];
     block_total<R, 4>(av, AV, scratch);  // (synchronises: the triangle records are complete below)
-    if (threadIdx.x == 0) {  // once per cell in FP64
-        cuv[0] = R(0.5 * (AV[0] - m.A0) / (m.A0 * m.A0));
-        cuv[1] = R(0.5 * AV[1] / (m.A0 * m.A0));
-        cuv[2] = R((AV[2] - m.V0) / (m.V0 * m.V0) / 6.0);
-        cuv[3] = R(AV[3] / (m.V0 * m.V0) / 6.0);
+    if (threadIdx.x < 4) {  // once per cell in FP64, a lane each
+        const int k = threadIdx.x;
+        const double x = k == 0 ? AV[0] - m.A0 : (k == 1 ? AV[1] : (k == 2 ? AV[2] - m.V0 : AV[3]));
+        cuv[k] = k < 2 ? R(0.5 * x / (m.A0 * m.A0)) : R(x / (m.V0 * m.V0) / 6.0);
     }
 
     // per edge, unit moduli: link s (F on v0 = s (x1 - x0)), cb |e|, cb sa0, cb sb0
-    for (int e = threadIdx.x; e < m.ne; e += blockDim.x) {
+    for (int q = e0 + threadIdx.x; q < e1; q += blockDim.x) {
+        const int e = q == e0 + (int)threadIdx.x ? ei : (items ? __ldg(items + q) : q);
         const int4 E = __ldg(reinterpret_cast<const int4 *>(m.edge) + e);  // v0, v1, a, b
         const int2 T = __ldg(reinterpret_cast<const int2 *>(m.etri) + e);
         const V3<D> p0 = dq(xv + 4 * E.x, xd + 4 * E.x), p1 = dq(xv + 4 * E.y, xd + 4 * E.y);
@@ -1080,7 +1092,6 @@ __global__ void __launch_bounds__(NT, 1) cell_adjoint_gather_kernel(View<float> 
     const D ha = {cuv[0], cuv[1]}, sv = {cuv[2], cuv[3]};
     const R kl = m.k_link, kb = m.k_bend, kA = R(m.k_area), kV = R(m.k_volume);
     Acc<R> th[4];  // lamFv . unit-modulus forces: link, bend, area, volume
-    const int per = (m.nv + slices - 1) / slices, i0 = slice * per, i1 = min(m.nv, i0 + per);
     for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         const V3<D> pi = dq(xv + 4 * i, xd + 4 * i);
         const V3<D> z = {dconst(R(0)), dconst(R(0)), dconst(R(0))};
@@ -1279,19 +1290,13 @@ cudaError_t set_cell_smem_limit(size_t bytes) {
     return e;
 }
 
-// CTAs per cell of the FP32 adjoint gather when cells are fewer than SMs
-// (measured on the 48^3 box with 4 cells: reverse step 124.4 -> 119.7 us;
-// 16 CTAs no better)
-constexpr int ADJ_GATHER_SLICES = 8;
 template <typename R>
 void launch_cell_adjoint(const View<R> &v, const AdjView<R> &a, cudaStream_t st) {
     if (v.ncell == 0) return;
     if constexpr (std::is_same<R, float>::value) {
         const size_t gs = cell_adjoint_gather_bytes(v.max_nv, v.max_nt, v.max_ne);
         if (gs <= CELL_ADJ_GATHER_MAX_SMEM) {
-            // few cells: several CTAs per cell, each gathering a share of
-            // the vertices (the records are rebuilt by each)
-            const int slices = std::max(1, std::min(ADJ_GATHER_SLICES, v.nsm / v.ncell));
+            const int slices = v.slices;
             if (cell_wide(v))
                 cell_adjoint_gather_kernel<CellMax<R>::T><<<v.ncell * slices, CellMax<R>::T, gs, st>>>(v, a, slices);
             else
