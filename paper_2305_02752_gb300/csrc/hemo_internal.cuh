@@ -340,6 +340,35 @@ template <> struct Acc<float> {
     __device__ double value() const { return (double)hi + (double)lo; }
 };
 
+// Kernel launches that overlap the end of the kernel before them in the stream
+// (programmatic stream serialisation): the next kernel's CTAs are scheduled as
+// those of the running one leave, and wait in wait_previous() until it has
+// completed and its writes are visible.  Every kernel launched this way calls
+// wait_previous() first, in every thread, so that completion of a kernel implies
+// completion of all before it.  A small step is a chain of kernels of a few us
+// each: 48^3 box, two steps and read-out 124 -> 117 us, with Lees-Edwards
+// boundaries 548 -> 525, 32^3 FP64 420 -> 407; large steps the same.  Letting the
+// next kernel start at the beginning of the running one (launch_dependents) was
+// slower (32^3 FP64 524 us).
+__device__ __forceinline__ void wait_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_next(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Drops this thread's share of the dead buffer's L2 lines (discard.global.L2:
 // the lines are invalidated without write-back, so data that no kernel will
 // read again costs no DRAM writes when it would be evicted).

@@ -62,6 +62,7 @@ __device__ void block_add(const R (&val)[K], double *out) {
 // added by the streaming transpose when it pulls the population.
 template <typename R>
 __global__ void __launch_bounds__(256) adj_moments_kernel(View<R> v, AdjView<R> a) {
+    wait_previous();
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     R ds[1] = {R(0)};
     if (n < v.N) {
@@ -120,6 +121,7 @@ __device__ __forceinline__ void pull_adjoint(const View<R> &v, const AdjView<R> 
 constexpr int ADJ_NT = 128;  // (FP64, 32^3 box: 25.7 us against 27.0 with 256; FP32 the same)
 template <typename R>
 __global__ void __launch_bounds__(ADJ_NT) adj_collide_kernel(View<R> v, AdjView<R> a) {
+    wait_previous();
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     R acc[4] = {R(0), R(0), R(0), R(0)};  // wall-velocity scale, g_x, g_y, g_z
     if (n < v.N && !(v.ntype[n] & 0x7f)) {
@@ -232,12 +234,12 @@ __global__ void __launch_bounds__(ADJ_NT) adj_collide_kernel(View<R> v, AdjView<
 
 template <typename R>
 void launch_adj_moments(const View<R> &v, const AdjView<R> &a, cudaStream_t st) {
-    adj_moments_kernel<R><<<nblocks(v.N, 256), 256, 0, st>>>(v, a);
+    launch_next(adj_moments_kernel<R>, nblocks(v.N, 256), 256, 0, st, v, a);
 }
 
 template <typename R>
 void launch_adj_collide(const View<R> &v, const AdjView<R> &a, cudaStream_t st) {
-    adj_collide_kernel<R><<<nblocks(v.N, ADJ_NT), ADJ_NT, 0, st>>>(v, a);
+    launch_next(adj_collide_kernel<R>, nblocks(v.N, ADJ_NT), ADJ_NT, 0, st, v, a);
 }
 
 #define HEMO_INST(R)                                                                  \

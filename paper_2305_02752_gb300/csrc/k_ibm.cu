@@ -84,6 +84,7 @@ __device__ __forceinline__ void bin_origin(const View<R> &v, int k, int org[3]) 
 
 template <typename R>
 __global__ void anchor_count_kernel(View<R> v) {
+    wait_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= v.nv) return;
     const int c = v.vcell[i];
@@ -134,6 +135,7 @@ __device__ __forceinline__ void store_quad(int *p, int k, int n, bool vec, int4 
     if (k + 3 < n) p[k + 3] = q.w;
 }
 __global__ void __launch_bounds__(1024) scan_kernel(int *counts, int *start, int *cursor, int nbins) {
+    wait_previous();
     __shared__ int wsum[32];
     __shared__ int carry_s;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -178,6 +180,7 @@ __global__ void __launch_bounds__(1024) scan_kernel(int *counts, int *start, int
 // scatter with per-block cursors; lanes of a warp with the same key reserve
 // their slots with one atomic
 __global__ void scatter_kernel(const int *key, int *cursor, int *perm_raw, int nv, unsigned *status) {
+    wait_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nv) return;
     const int k = key[i];
@@ -198,6 +201,7 @@ __global__ void scatter_kernel(const int *key, int *cursor, int *perm_raw, int n
 constexpr int SMALL_BINS = 4096, SMALL_NV = 8192;
 __global__ void __launch_bounds__(1024) scan_scatter_kernel(int *counts, int *start, int nbins, const int *key, int *perm,
                                                             int nv, unsigned *status) {
+    wait_previous();
     __shared__ int cur[SMALL_BINS];
     __shared__ int wsum[32];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -243,6 +247,7 @@ __global__ void __launch_bounds__(1024) scan_scatter_kernel(int *counts, int *st
 constexpr int SORT_SMEM = 1024;
 constexpr int SORT_K = 8;
 __global__ void __launch_bounds__(128) sort_bins_kernel(const int *start, const int *perm_raw, int *perm, int nbins) {
+    wait_previous();
     __shared__ int buf[4][SORT_SMEM];
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
@@ -547,6 +552,7 @@ __device__ __forceinline__ void spread_item(int *first, int s, const float (&F)[
 }
 
 __global__ void __launch_bounds__(SP_CHUNK, 6) spread_tile_f32_kernel(View<float> v) {
+    wait_previous();
     const int k = blockIdx.x;
     const int s = v.start[k], e = v.start[k + 1], n = e - s;
     if (n == 0) return;
@@ -703,6 +709,7 @@ __global__ void __launch_bounds__(SP_CHUNK, 6) spread_tile_f32_kernel(View<float
 // per bin; weights by one thread per vertex).
 template <typename R>
 __global__ void __launch_bounds__(256) spread_tile_kernel(View<R> v) {
+    wait_previous();
     using A = typename TileAcc<R>::T;
     constexpr int CAP = SpreadCap<R>::CAP;
     const int k = blockIdx.x / 3, d = blockIdx.x - 3 * k;
@@ -775,6 +782,7 @@ __global__ void __launch_bounds__(256) spread_tile_kernel(View<R> v) {
 constexpr int GATHER_MAXE = 2 * TILE;  // entries per (axis, local coordinate)
 template <typename R>
 __global__ void __launch_bounds__(256) spread_gather_kernel(View<R> v) {
+    wait_previous();
     __shared__ int nbin[27];  // bin of neighbour slot (sz*9 + sy*3 + sx), -1 if empty
     __shared__ int lb[3][3], nsl[3];
     __shared__ unsigned char cnt[3][BLK];
@@ -850,6 +858,7 @@ __global__ void __launch_bounds__(256) spread_gather_kernel(View<R> v) {
 // offsets, 56 registers) took 1384, one per component and node 1814.
 template <typename R>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 8 : 1) spread_gather3_kernel(View<R> v) {
+    wait_previous();
     __shared__ int nbin[27];  // bin of slot (sz + 1) * 9 + (sy + 1) * 3 + (sx + 1), -1 if empty or absent
     const int k = blockIdx.x;
     const int bc[3] = {k % v.nb[0], (k / v.nb[0]) % v.nb[1], k / (v.nb[0] * v.nb[1])};
@@ -983,6 +992,7 @@ __device__ __forceinline__ void adapt_max(unsigned long long *adapt, double d) {
 // evaluation, or when a vertex has moved more than tol since it; the
 // displacement word is cleared for the coming step's interpolation.
 __global__ void adapt_decide_kernel(unsigned long long *a, double tol, int every) {
+    wait_previous();
     const bool eval = a[3] || a[1] >= (unsigned long long)every || __longlong_as_double((long long)a[0]) > tol;
     a[2] = eval ? 1ull : 0ull;
     a[4] += eval ? 1ull : 0ull;  // evaluations so far
@@ -996,6 +1006,7 @@ __global__ void adapt_decide_kernel(unsigned long long *a, double tol, int every
 // X = (hi + lo of the centroid of the last re-base) + offset.
 template <typename R>
 __global__ void __launch_bounds__(256) hold_bins_kernel(View<R> v) {
+    wait_previous();
     if (v.adapt && v.adapt[2]) return;  // adaptive separation: this step evaluates the forces
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= v.nv) return;
@@ -1019,6 +1030,7 @@ __global__ void __launch_bounds__(256) hold_bins_kernel(View<R> v) {
 constexpr int InterpCap = 32;  // vertices per chunk
 template <typename R, int INTEG>
 __global__ void __launch_bounds__(256) interpolate_kernel(View<R> v, int parts) {
+    wait_previous();
     drop_dead_lines(v);
     constexpr int CAP = InterpCap;
     const int k = blockIdx.x / parts, part = blockIdx.x % parts;  // CTA part takes chunks part, part + parts, ...
@@ -1116,6 +1128,7 @@ __device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefe
 constexpr int IT_CHUNK = 256;  // vertices sorted at a time, one per thread
 template <int INTEG>
 __global__ void __launch_bounds__(IT_CHUNK, 6) interpolate_v4_kernel(View<float> v, const __grid_constant__ CUtensorMap umap) {
+    wait_previous();
     drop_dead_lines(v);
     const int k = blockIdx.x;
     const int s = v.start[k], e = v.start[k + 1];
@@ -1351,6 +1364,7 @@ template <typename R> struct VfStage { static constexpr int CAP = sizeof(R) == 8
 template <typename R>
 __global__ void __launch_bounds__(256) vertex_field_kernel(View<R> v, const R *A, const R *B, R *out_grad,
                                                            R *out_interp, int parts) {
+    wait_previous();
     constexpr int CAP = VfStage<R>::CAP;
     const int k = blockIdx.x / parts, part = blockIdx.x % parts;  // CTA part takes chunks part, part + parts, ...
     const int s = v.start[k], e = v.start[k + 1];
@@ -1424,6 +1438,7 @@ __global__ void __launch_bounds__(256) vertex_field_kernel(View<R> v, const R *A
 // tile, as in interpolate_v4_kernel
 __global__ void __launch_bounds__(256) vertex_field_v4_kernel(View<float> v, const float *A, const float *B,
                                                               float *out_grad, float *out_interp) {
+    wait_previous();
     const int k = blockIdx.x;
     const int s = v.start[k], e = v.start[k + 1];
     if (s == e) return;
@@ -1508,6 +1523,7 @@ __global__ void __launch_bounds__(256) vertex_field_v4_kernel(View<float> v, con
 // 12.6 M vertices; one component per thread 254, this 206)
 template <typename R>
 __global__ void __launch_bounds__(256) verts_out_kernel(View<R> v, double *X, double *F) {
+    wait_previous();
     const unsigned q0 = 4u * (blockIdx.x * 256u + threadIdx.x), n = 3u * (unsigned)v.nv;
     if (q0 >= n) return;
     const bool vec = sizeof(R) == 4 && q0 + 4 <= n && (((uintptr_t)X | (uintptr_t)F) & 15) == 0;
@@ -1557,13 +1573,13 @@ __global__ void set_vertices_kernel(View<R> v, const double *X) {
 template <typename R>
 void launch_bins(const View<R> &v, cudaStream_t st, bool stable) {
     cudaMemsetAsync(v.counts, 0, sizeof(int) * v.nbins, st);
-    anchor_count_kernel<R><<<nblocks(v.nv, 256), 256, 0, st>>>(v);
-    scan_kernel<<<1, 1024, 0, st>>>(v.counts, v.start, v.cursor, v.nbins);
+    launch_next(anchor_count_kernel<R>, nblocks(v.nv, 256), 256, 0, st, v);
+    launch_next(scan_kernel, 1, 1024, 0, st, v.counts, v.start, v.cursor, v.nbins);
     if (stable) {
-        scatter_kernel<<<nblocks(v.nv, 256), 256, 0, st>>>(v.key, v.cursor, v.perm_raw, v.nv, v.status);
-        sort_bins_kernel<<<nblocks((long long)v.nbins * 32, 128), 128, 0, st>>>(v.start, v.perm_raw, v.perm, v.nbins);
+        launch_next(scatter_kernel, nblocks(v.nv, 256), 256, 0, st, v.key, v.cursor, v.perm_raw, v.nv, v.status);
+        launch_next(sort_bins_kernel, nblocks((long long)v.nbins * 32, 128), 128, 0, st, v.start, v.perm_raw, v.perm, v.nbins);
     } else {
-        scatter_kernel<<<nblocks(v.nv, 256), 256, 0, st>>>(v.key, v.cursor, v.perm, v.nv, v.status);
+        launch_next(scatter_kernel, nblocks(v.nv, 256), 256, 0, st, v.key, v.cursor, v.perm, v.nv, v.status);
     }
 }
 
@@ -1571,19 +1587,19 @@ template <typename R>
 void launch_bin_ranges(const View<R> &v, cudaStream_t st) {
     const int nbins = v.nbins + (v.le ? 1 : 0);  // (+ the Lees-Edwards bin)
     if (nbins <= SMALL_BINS && v.nv <= SMALL_NV) {
-        scan_scatter_kernel<<<1, 1024, 0, st>>>(v.counts, v.start, nbins, v.key, v.perm, v.nv, v.status);
+        launch_next(scan_scatter_kernel, 1, 1024, 0, st, v.counts, v.start, nbins, v.key, v.perm, v.nv, v.status);
         return;
     }
-    scan_kernel<<<1, 1024, 0, st>>>(v.counts, v.start, v.cursor, nbins);
-    scatter_kernel<<<nblocks(v.nv, 256), 256, 0, st>>>(v.key, v.cursor, v.perm, v.nv, v.status);
+    launch_next(scan_kernel, 1, 1024, 0, st, v.counts, v.start, v.cursor, nbins);
+    launch_next(scatter_kernel, nblocks(v.nv, 256), 256, 0, st, v.key, v.cursor, v.perm, v.nv, v.status);
 }
 
 template <typename R>
 void launch_spread(const View<R> &v, cudaStream_t st) {
-    if constexpr (std::is_same<R, float>::value) spread_tile_f32_kernel<<<v.nbins, SP_CHUNK, 0, st>>>(v);
-    else spread_tile_kernel<R><<<3 * v.nbins, 256, 0, st>>>(v);
-    if (v.nb[0] >= 3 && v.nb[1] >= 3 && v.nb[2] >= 3) spread_gather3_kernel<R><<<v.nbins, 256, 0, st>>>(v);
-    else spread_gather_kernel<R><<<v.nbins, 256, 0, st>>>(v);
+    if constexpr (std::is_same<R, float>::value) launch_next(spread_tile_f32_kernel, v.nbins, SP_CHUNK, 0, st, v);
+    else launch_next(spread_tile_kernel<R>, 3 * v.nbins, 256, 0, st, v);
+    if (v.nb[0] >= 3 && v.nb[1] >= 3 && v.nb[2] >= 3) launch_next(spread_gather3_kernel<R>, v.nbins, 256, 0, st, v);
+    else launch_next(spread_gather_kernel<R>, v.nbins, 256, 0, st, v);
 }
 
 template <typename R, int INTEG>
@@ -1599,9 +1615,9 @@ void launch_interpolate_as(const View<R> &v, cudaStream_t st) {
             std::memset(&map, 0, sizeof(map));
             w.u_tmap = nullptr;
         }
-        interpolate_v4_kernel<INTEG><<<v.nbins, IT_CHUNK, 0, st>>>(w, map);
+        launch_next(interpolate_v4_kernel<INTEG>, v.nbins, IT_CHUNK, 0, st, w, map);
     }
-    else interpolate_kernel<R, INTEG><<<v.nbins * FP64_BIN_PARTS, 256, 0, st>>>(v, FP64_BIN_PARTS);
+    else launch_next(interpolate_kernel<R, INTEG>, v.nbins * FP64_BIN_PARTS, 256, 0, st, v, FP64_BIN_PARTS);
 }
 
 template <typename R>
@@ -1613,24 +1629,24 @@ void launch_interpolate(const View<R> &v, cudaStream_t st) {
 
 template <typename R>
 void launch_hold_bins(const View<R> &v, cudaStream_t st) {
-    if (v.nv) hold_bins_kernel<R><<<nblocks(v.nv, 256), 256, 0, st>>>(v);
+    if (v.nv) launch_next(hold_bins_kernel<R>, nblocks(v.nv, 256), 256, 0, st, v);
 }
 
 void launch_adapt_decide(unsigned long long *adapt, double tol, int every, cudaStream_t st) {
-    adapt_decide_kernel<<<1, 1, 0, st>>>(adapt, tol, every);
+    launch_next(adapt_decide_kernel, 1, 1, 0, st, adapt, tol, every);
 }
 
 template <typename R>
 void launch_vertex_field(const View<R> &v, const R *field, const R *vec, R *out_grad, R *out_interp, cudaStream_t st) {
     if constexpr (std::is_same<R, float>::value)
-        vertex_field_v4_kernel<<<v.nbins, 256, 0, st>>>(v, field, vec, out_grad, out_interp);
+        launch_next(vertex_field_v4_kernel, v.nbins, 256, 0, st, v, field, vec, out_grad, out_interp);
     else
-        vertex_field_kernel<R><<<v.nbins * FP64_BIN_PARTS, 256, 0, st>>>(v, field, vec, out_grad, out_interp, FP64_BIN_PARTS);
+        launch_next(vertex_field_kernel<R>, v.nbins * FP64_BIN_PARTS, 256, 0, st, v, field, vec, out_grad, out_interp, FP64_BIN_PARTS);
 }
 
 template <typename R>
 void launch_verts_out(const View<R> &v, double *X, double *F, cudaStream_t st) {
-    if (v.nv) verts_out_kernel<R><<<nblocks(3LL * v.nv, 1024), 256, 0, st>>>(v, X, F);
+    if (v.nv) launch_next(verts_out_kernel<R>, nblocks(3LL * v.nv, 1024), 256, 0, st, v, X, F);
 }
 
 template <typename R>

@@ -35,6 +35,7 @@ __device__ __forceinline__ R edge_fn(const R (*P)[3], const int *id, int u, int 
 // one thread per triangle: grid (cells, triangle blocks of 256)
 template <typename R>
 __global__ void __launch_bounds__(256) inside_toggle_kernel(View<R> v) {
+    wait_previous();
     const int c = blockIdx.x;
     const MeshDev<R> m = v.meshes[v.cell_type[c]];
     const int first = v.cell_first[c];
@@ -109,6 +110,7 @@ __global__ void __launch_bounds__(256) inside_toggle_kernel(View<R> v) {
 constexpr int SCAN_G = 8;
 template <typename R>
 __global__ void __launch_bounds__(32 * SCAN_G) inside_scan_kernel(View<R> v) {
+    wait_previous();
     __shared__ int ssum[SCAN_G][32], smin[SCAN_G][32];
     const int lx = threadIdx.x, g = threadIdx.y;
     const int x = blockIdx.x * 32 + lx, y = blockIdx.y;
@@ -147,8 +149,8 @@ __global__ void __launch_bounds__(32 * SCAN_G) inside_scan_kernel(View<R> v) {
 
 template <typename R>
 void launch_inside(const View<R> &v, cudaStream_t st) {
-    if (v.ncell) inside_toggle_kernel<R><<<dim3(v.ncell, (v.max_nt + 255) / 256), 256, 0, st>>>(v);
-    inside_scan_kernel<R><<<dim3((v.nx + 31) / 32, v.ny), dim3(32, SCAN_G), 0, st>>>(v);
+    if (v.ncell) launch_next(inside_toggle_kernel<R>, dim3(v.ncell, (v.max_nt + 255) / 256), 256, 0, st, v);
+    launch_next(inside_scan_kernel<R>, dim3((v.nx + 31) / 32, v.ny), dim3(32, SCAN_G), 0, st, v);
 }
 
 template void launch_inside<double>(const View<double> &, cudaStream_t);

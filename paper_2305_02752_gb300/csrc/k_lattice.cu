@@ -225,6 +225,7 @@ __device__ __forceinline__ bool node_xy(const View<R> &v, int &x, int &y) {
 // all nodes, grid of NODE_BX x NODE_BY blocks over (x, y, z)
 template <typename T, typename R, int PARITY, typename I, bool VISC>
 __global__ void __launch_bounds__(NODE_BX * NODE_BY, sizeof(R) == 4 ? 4 : 1) collide_stream_kernel(View<R> v) {
+    wait_previous();
     drop_dead_lines(v);
     int x, y;
     const int z = blockIdx.z;
@@ -311,6 +312,7 @@ constexpr int TILE_COPIES = Q + 3;  // lanes of the producer warp that issue the
 
 template <typename T, typename R, int PARITY, typename I>
 __global__ void __launch_bounds__(TILE_THREADS, 1) collide_tiles_kernel(View<R> v) {
+    wait_previous();
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *full = reinterpret_cast<uint64_t *>(smem);  // [stage]: the stage's copies have landed
     uint64_t *empty = full + TILE_MAX_STAGES;             // [stage]: the consumers are done with it
@@ -494,6 +496,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) collide_tiles_kernel(View<R> 
 // the order of the two kernels does not matter.
 template <typename T, typename R, int PARITY, typename I>
 __global__ void __launch_bounds__(256, 4) collide_erows_kernel(View<R> v) {
+    wait_previous();
     const int nx = v.nx;
     const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
     if (t >= (long long)v.nerows * nx) return;
@@ -529,6 +532,7 @@ __device__ __forceinline__ void moments_core(const View<R> &v, int n, const Nbr 
 
 template <typename T, typename R, int LAYOUT, typename I>
 __global__ void __launch_bounds__(NODE_BX * MOM_BY) moments_kernel(View<R> v) {
+    wait_previous();
     int x, y;
     const int z = blockIdx.z;
     if (!node_xy<MOM_BY>(v, x, y)) return;
@@ -625,6 +629,7 @@ __device__ __forceinline__ void load_pair_words(const View<float> &v, int n0, in
 
 template <typename T, int PARITY, typename I, bool VISC>
 __global__ void __launch_bounds__(NODE_BX * NODE_BY) collide_pair_kernel(View<float> v) {
+    wait_previous();
     drop_dead_lines(v);
     const int lane = threadIdx.x;
     const int x0 = blockIdx.x * PAIR_X + 2 * lane, y = blockIdx.y * NODE_BY + threadIdx.y, z = blockIdx.z;
@@ -711,6 +716,7 @@ __global__ void __launch_bounds__(NODE_BX * NODE_BY) collide_pair_kernel(View<fl
 // as in load_pops
 template <typename T, int LAYOUT, typename I>
 __global__ void __launch_bounds__(NODE_BX * MOM_BY) moments_pair_kernel(View<float> v) {
+    wait_previous();
     const int lane = threadIdx.x;
     const int x0 = blockIdx.x * PAIR_X + 2 * lane, y = blockIdx.y * MOM_BY + threadIdx.y, z = blockIdx.z;
     if (y >= v.ny) return;
@@ -838,6 +844,7 @@ __global__ void init_equilibrium_kernel(View<R> v, const double *u0) {
 
 template <typename T, typename R, int LAYOUT>
 __global__ void populations_out_kernel(View<R> v, double *out) {
+    wait_previous();
     int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= v.N) return;
     const uint8_t nt = v.ntype[n];
@@ -855,6 +862,7 @@ __global__ void populations_out_kernel(View<R> v, double *out) {
 
 template <typename T, typename R, int LAYOUT>
 __global__ void rho_out_kernel(View<R> v, R *out) {
+    wait_previous();
     int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= v.N) return;
     const uint8_t nt = v.ntype[n];
@@ -873,6 +881,7 @@ __global__ void rho_out_kernel(View<R> v, R *out) {
 
 template <typename R>
 __global__ void u_out_kernel(View<R> v, R *out) {
+    wait_previous();
     int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= v.N) return;
     const size_t N = (size_t)v.N;
@@ -886,6 +895,7 @@ __global__ void u_out_kernel(View<R> v, R *out) {
 // stores with a stride of 12 bytes: 284 us on the pipe, this 144)
 constexpr int UOUT_NT = 256;
 __global__ void __launch_bounds__(UOUT_NT) u_out_vec_kernel(View<float> v, float *out) {
+    wait_previous();
     __shared__ float s[12 * UOUT_NT];
     const size_t N = (size_t)v.N, n0 = (size_t)blockIdx.x * 4 * UOUT_NT;
     const size_t n = n0 + 4 * threadIdx.x;
@@ -948,6 +958,7 @@ __global__ void mark_near_wall_kernel(int N, uint8_t *ntype, const uint64_t *lin
 // Natural-layout copy of the deviations (R, SoA [i][n]); wall nodes get 0.
 template <typename T, typename R, int LAYOUT>
 __global__ void copy_natural_kernel(View<R> v, R *out) {
+    wait_previous();
     int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= v.N) return;
     const size_t N = (size_t)v.N;
@@ -970,6 +981,7 @@ __global__ void copy_natural_kernel(View<R> v, R *out) {
 // by exactly one thread.
 template <typename T, typename R, int LAYOUT>
 __global__ void restore_natural_kernel(View<R> v, const R *in) {
+    wait_previous();
     int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= v.N) return;
     const size_t N = (size_t)v.N;
@@ -1021,12 +1033,12 @@ void launch_collide_as(const View<R> &v, cudaStream_t st) {
     if constexpr (std::is_same<R, float>::value && sizeof(T) == 2) {
         if (v.node_pairs & PAIR_COLLIDE) {
             const dim3 g((unsigned)nblocks(v.nx, PAIR_X), (unsigned)nblocks(v.ny, NODE_BY), (unsigned)v.nz);
-            collide_pair_kernel<T, PARITY, I, VISC><<<g, dim3(NODE_BX, NODE_BY), 0, st>>>(v);
+            launch_next(collide_pair_kernel<T, PARITY, I, VISC>, g, dim3(NODE_BX, NODE_BY), 0, st, v);
             return;
         }
     }
     const View<R> w = with_flat(v);
-    collide_stream_kernel<T, R, PARITY, I, VISC><<<node_grid(w, NODE_BY), dim3(NODE_BX, NODE_BY), 0, st>>>(w);
+    launch_next(collide_stream_kernel<T, R, PARITY, I, VISC>, node_grid(w, NODE_BY), dim3(NODE_BX, NODE_BY), 0, st, w);
 }
 
 template <typename T, typename R, typename I>
@@ -1043,9 +1055,9 @@ void launch_collide_parity(const View<R> &v, int parity, cudaStream_t st) {
 
 template <typename T, typename R, int PARITY, typename I>
 void launch_tiles_pi(const View<R> &v, cudaStream_t st) {
-    collide_tiles_kernel<T, R, PARITY, I><<<v.tile_grid, TILE_THREADS, v.tile_smem, st>>>(v);
+    launch_next(collide_tiles_kernel<T, R, PARITY, I>, v.tile_grid, TILE_THREADS, v.tile_smem, st, v);
     const long long ne = (long long)v.nerows * v.nx;
-    if (ne > 0) collide_erows_kernel<T, R, PARITY, I><<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(v);
+    if (ne > 0) launch_next(collide_erows_kernel<T, R, PARITY, I>, (unsigned)((ne + 255) / 256), 256, 0, st, v);
 }
 
 template <typename T, typename R>
@@ -1097,12 +1109,12 @@ void launch_moments_as(const View<R> &v, cudaStream_t st) {
     if constexpr (std::is_same<R, float>::value && sizeof(T) == 2) {
         if (v.node_pairs & PAIR_MOMENTS) {
             const dim3 g((unsigned)nblocks(v.nx, PAIR_X), (unsigned)nblocks(v.ny, MOM_BY), (unsigned)v.nz);
-            moments_pair_kernel<T, LAYOUT, I><<<g, dim3(NODE_BX, MOM_BY), 0, st>>>(v);
+            launch_next(moments_pair_kernel<T, LAYOUT, I>, g, dim3(NODE_BX, MOM_BY), 0, st, v);
             return;
         }
     }
     const View<R> w = with_flat(v);
-    moments_kernel<T, R, LAYOUT, I><<<node_grid(w, MOM_BY), dim3(NODE_BX, MOM_BY), 0, st>>>(w);
+    launch_next(moments_kernel<T, R, LAYOUT, I>, node_grid(w, MOM_BY), dim3(NODE_BX, MOM_BY), 0, st, w);
 }
 
 template <typename R>
@@ -1137,18 +1149,18 @@ template <typename R>
 void launch_populations_out(const View<R> &v, int precision, int layout, double *out, cudaStream_t st) {
     const int g = nblocks(v.N, 256);
     if (layout == 0)
-        HEMO_DISPATCH_T(precision, R, (populations_out_kernel<T, R, 0><<<g, 256, 0, st>>>(v, out)));
+        HEMO_DISPATCH_T(precision, R, (launch_next(populations_out_kernel<T, R, 0>, g, 256, 0, st, v, out)));
     else
-        HEMO_DISPATCH_T(precision, R, (populations_out_kernel<T, R, 1><<<g, 256, 0, st>>>(v, out)));
+        HEMO_DISPATCH_T(precision, R, (launch_next(populations_out_kernel<T, R, 1>, g, 256, 0, st, v, out)));
 }
 
 template <typename R>
 void launch_rho_out(const View<R> &v, int precision, int layout, R *out, cudaStream_t st) {
     const int g = nblocks(v.N, 256);
     if (layout == 0)
-        HEMO_DISPATCH_T(precision, R, (rho_out_kernel<T, R, 0><<<g, 256, 0, st>>>(v, out)));
+        HEMO_DISPATCH_T(precision, R, (launch_next(rho_out_kernel<T, R, 0>, g, 256, 0, st, v, out)));
     else
-        HEMO_DISPATCH_T(precision, R, (rho_out_kernel<T, R, 1><<<g, 256, 0, st>>>(v, out)));
+        HEMO_DISPATCH_T(precision, R, (launch_next(rho_out_kernel<T, R, 1>, g, 256, 0, st, v, out)));
 }
 
 template <typename R>
@@ -1156,11 +1168,11 @@ void launch_u_out(const View<R> &v, R *out, cudaStream_t st) {
     if constexpr (std::is_same<R, float>::value) {
         // (N a multiple of 4 keeps every component's start aligned with the first)
         if (v.N % 4 == 0 && (((uintptr_t)v.u | (uintptr_t)out) & 15) == 0) {
-            u_out_vec_kernel<<<nblocks(v.N, 4 * UOUT_NT), UOUT_NT, 0, st>>>(v, out);
+            launch_next(u_out_vec_kernel, nblocks(v.N, 4 * UOUT_NT), UOUT_NT, 0, st, v, out);
             return;
         }
     }
-    u_out_kernel<R><<<nblocks(v.N, 256), 256, 0, st>>>(v, out);
+    launch_next(u_out_kernel<R>, nblocks(v.N, 256), 256, 0, st, v, out);
 }
 
 void launch_build_links(int nx, int ny, int nz, const int *per, uint8_t *ntype, uint64_t *links, cudaStream_t st) {
@@ -1173,18 +1185,18 @@ template <typename R>
 void launch_copy_natural(const View<R> &v, int precision, int layout, R *out, cudaStream_t st) {
     const int g = nblocks(v.N, 256);
     if (layout == 0)
-        HEMO_DISPATCH_T(precision, R, (copy_natural_kernel<T, R, 0><<<g, 256, 0, st>>>(v, out)));
+        HEMO_DISPATCH_T(precision, R, (launch_next(copy_natural_kernel<T, R, 0>, g, 256, 0, st, v, out)));
     else
-        HEMO_DISPATCH_T(precision, R, (copy_natural_kernel<T, R, 1><<<g, 256, 0, st>>>(v, out)));
+        HEMO_DISPATCH_T(precision, R, (launch_next(copy_natural_kernel<T, R, 1>, g, 256, 0, st, v, out)));
 }
 
 template <typename R>
 void launch_restore_natural(const View<R> &v, int precision, int layout, const R *in, cudaStream_t st) {
     const int g = nblocks(v.N, 256);
     if (layout == 0)
-        HEMO_DISPATCH_T(precision, R, (restore_natural_kernel<T, R, 0><<<g, 256, 0, st>>>(v, in)));
+        HEMO_DISPATCH_T(precision, R, (launch_next(restore_natural_kernel<T, R, 0>, g, 256, 0, st, v, in)));
     else
-        HEMO_DISPATCH_T(precision, R, (restore_natural_kernel<T, R, 1><<<g, 256, 0, st>>>(v, in)));
+        HEMO_DISPATCH_T(precision, R, (launch_next(restore_natural_kernel<T, R, 1>, g, 256, 0, st, v, in)));
 }
 
 #define HEMO_INST(R)                                                                              \

@@ -36,6 +36,7 @@ __device__ __forceinline__ void peskin4_le(R t, R *w) {
 // collision of every node, A (natural order) -> B (natural order)
 template <typename T, typename R>
 __global__ void __launch_bounds__(NODE_BX * NODE_BY) le_collide_kernel(View<R> v) {
+    wait_previous();
     const int x = blockIdx.x * NODE_BX + threadIdx.x, y = blockIdx.y * NODE_BY + threadIdx.y, z = blockIdx.z;
     if (x >= v.nx || y >= v.ny) return;
     const size_t N = (size_t)v.N, n = (size_t)x + (size_t)v.nx * ((size_t)y + (size_t)v.ny * z);
@@ -82,6 +83,7 @@ __device__ __forceinline__ R eq_shift(int i, R w, R rho, R ux, R uy, R uz, R dU)
 // F/2 of the streamed populations
 template <typename T, typename R>
 __global__ void __launch_bounds__(NODE_BX * NODE_BY) le_stream_kernel(View<R> v) {
+    wait_previous();
     const int x = blockIdx.x * NODE_BX + threadIdx.x, y = blockIdx.y * NODE_BY + threadIdx.y;
     const int z = blockIdx.z;
     // the images' displacement as whole nodes and the remaining fraction ([0] the
@@ -183,6 +185,7 @@ __device__ __forceinline__ void le_layer(const View<R> &v, double D, double X, i
 // b and z-layer c of the stencil each)
 template <typename R>
 __global__ void __launch_bounds__(256) le_spread_kernel(View<R> v) {
+    wait_previous();
     const int s = v.start[v.nbins], e = v.start[v.nbins + 1];
     const int q = s + (blockIdx.x * blockDim.x + threadIdx.x) / 16;
     if (q >= e) return;
@@ -217,6 +220,7 @@ __global__ void __launch_bounds__(256) le_spread_kernel(View<R> v) {
 // thread per vertex
 template <typename R>
 __global__ void __launch_bounds__(256) le_interp_kernel(View<R> v) {
+    wait_previous();
     const int s = v.start[v.nbins], e = v.start[v.nbins + 1];
     const int q = s + blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= e) return;
@@ -254,7 +258,8 @@ __global__ void __launch_bounds__(256) le_interp_kernel(View<R> v) {
     o[2] += U2;
 }
 
-__global__ void le_advance_kernel(long long *n) { *n += 1; }
+__global__ void le_advance_kernel(long long *n) {
+    wait_previous(); *n += 1; }
 
 }  // namespace
 
@@ -262,22 +267,22 @@ template <typename R>
 void launch_le_lattice(const View<R> &v, int precision, cudaStream_t st) {
     const dim3 g((unsigned)((v.nx + NODE_BX - 1) / NODE_BX), (unsigned)((v.ny + NODE_BY - 1) / NODE_BY), (unsigned)v.nz),
         b(NODE_BX, NODE_BY);
-    HEMO_DISPATCH_T(precision, R, (le_collide_kernel<T, R><<<g, b, 0, st>>>(v)));
-    HEMO_DISPATCH_T(precision, R, (le_stream_kernel<T, R><<<g, b, 0, st>>>(v)));
+    HEMO_DISPATCH_T(precision, R, (launch_next(le_collide_kernel<T, R>, g, b, 0, st, v)));
+    HEMO_DISPATCH_T(precision, R, (launch_next(le_stream_kernel<T, R>, g, b, 0, st, v)));
 }
 
 template <typename R>
 void launch_le_spread(const View<R> &v, cudaStream_t st) {
     // every vertex could be in the extra bin: the grid covers nv of them
-    if (v.nv) le_spread_kernel<R><<<(unsigned)((16 * (size_t)v.nv + 255) / 256), 256, 0, st>>>(v);
+    if (v.nv) launch_next(le_spread_kernel<R>, (unsigned)((16 * (size_t)v.nv + 255) / 256), 256, 0, st, v);
 }
 
 template <typename R>
 void launch_le_interp(const View<R> &v, cudaStream_t st) {
-    if (v.nv) le_interp_kernel<R><<<(unsigned)((v.nv + 255) / 256), 256, 0, st>>>(v);
+    if (v.nv) launch_next(le_interp_kernel<R>, (unsigned)((v.nv + 255) / 256), 256, 0, st, v);
 }
 
-void launch_le_advance(long long *n, cudaStream_t st) { le_advance_kernel<<<1, 1, 0, st>>>(n); }
+void launch_le_advance(long long *n, cudaStream_t st) { launch_next(le_advance_kernel, 1, 1, 0, st, n); }
 
 template void launch_le_lattice<double>(const View<double> &, int, cudaStream_t);
 template void launch_le_lattice<float>(const View<float> &, int, cudaStream_t);

@@ -284,6 +284,7 @@ __device__ __forceinline__ bool fan_force(const MeshDev<R> &m, const R *xs, cons
 
 template <typename R, int NT>
 __global__ void __launch_bounds__(NT, CellMinBlocks<R, NT>::B) cell_kernel(View<R> v, int mode, double *stats) {
+    wait_previous();
     if (mode == 0 && v.adapt && !v.adapt[2]) return;  // adaptive separation: the forces are held on this step
     const int c = blockIdx.x;
     const MeshDev<R> m = v.meshes[v.cell_type[c]];
@@ -489,6 +490,7 @@ __global__ void __launch_bounds__(NT, CellMinBlocks<R, NT>::B) cell_kernel(View<
 template <typename R> struct SliceThreads { static constexpr int T = CellMax<R>::T; };
 template <typename R>
 __global__ void __launch_bounds__(SliceThreads<R>::T, 1) cell_slices_kernel(View<R> v, int mode, double *stats) {
+    wait_previous();
     namespace cg = cooperative_groups;
     constexpr int NT = SliceThreads<R>::T;
     if (mode == 0 && v.adapt && !v.adapt[2]) return;  // (every CTA of the cluster)
@@ -749,6 +751,7 @@ template <typename R> __device__ __forceinline__ void add_into(R *f, R s, V3<R> 
 //                            linear in its modulus).
 template <typename R, int NT>
 __global__ void __launch_bounds__(NT, CellMinBlocks<R, NT>::B) cell_adjoint_kernel(View<R> v, AdjView<R> a, int slices) {
+    wait_previous();
     using D = Dual<R>;
     const int c = blockIdx.x / slices, slice = blockIdx.x % slices;
     const int type = v.cell_type[c];
@@ -876,6 +879,7 @@ __device__ __forceinline__ V3<Dual<double>> vertex_dual(const View<double> &v, c
     return dld3(v.off + 3 * i, a.lamFv + 3 * i);
 }
 __global__ void __launch_bounds__(ADJ_NT) adjoint_records_kernel(View<double> v, AdjView<double> a, int chunks) {
+    wait_previous();
     using D = Dual<double>;
     const int c = blockIdx.x / chunks, chunk = blockIdx.x % chunks;
     const MeshDev<double> m = v.meshes[v.cell_type[c]];
@@ -905,6 +909,7 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_records_kernel(View<double> v,
 }
 
 __global__ void __launch_bounds__(ADJ_NT) adjoint_terms_kernel(View<double> v, AdjView<double> a, int chunks, int echunks) {
+    wait_previous();
     using D = Dual<double>;
     using R = double;
     const int c = blockIdx.x / (chunks + echunks), chunk = blockIdx.x % (chunks + echunks);
@@ -985,6 +990,7 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_terms_kernel(View<double> v, A
 }
 
 __global__ void __launch_bounds__(256) adjoint_add_kernel(AdjView<double> a, int n) {
+    wait_previous();
     const int i = blockIdx.x * 256 + threadIdx.x;
     if (i >= n) return;
     a.lamX[i] += a.ft[i];
@@ -1007,6 +1013,7 @@ __global__ void __launch_bounds__(256) adjoint_add_kernel(AdjView<double> a, int
 // edge records each: 21.7).
 template <int NT>
 __global__ void __launch_bounds__(NT, 1) cell_adjoint_gather_kernel(View<float> v, AdjView<float> a, int slices) {
+    wait_previous();
     using R = float;
     using D = Dual<R>;
     const int c = blockIdx.x / slices, slice = blockIdx.x % slices;
@@ -1165,6 +1172,7 @@ __device__ void sym3_vec(const double *g, double lam, double *e) {
 // (the loss is the mean over cells): d l_k / dX_v = (2/n)(e_k . r_v) e_k.
 template <typename R>
 __global__ void __launch_bounds__(256) deformation_loss_kernel(View<R> v, const double *c0, double *cell_loss, R *dLdX) {
+    wait_previous();
     const int c = blockIdx.x;
     const MeshDev<R> m = v.meshes[v.cell_type[c]];
     const int first = v.cell_first[c];
@@ -1273,13 +1281,16 @@ void launch_cell_forces(const View<R> &v, int mode, double *stats, cudaStream_t 
     // positions and force accumulators of the largest mesh type
     const size_t smem = cell_smem_bytes<R>(v.max_nv, v.max_nt, v.max_ne);
     if (v.slices > 1) {
-        cudaLaunchAttribute at[1];
-        const cudaLaunchConfig_t cfg = slices_config<R>(v.slices, v.ncell, smem, st, at);
+        cudaLaunchAttribute at[2];
+        cudaLaunchConfig_t cfg = slices_config<R>(v.slices, v.ncell, smem, st, at);
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // (as launch_next)
+        at[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.numAttrs = 2;
         cudaLaunchKernelEx(&cfg, cell_slices_kernel<R>, v, mode, stats);
         return;
     }
-    if (cell_wide(v)) cell_kernel<R, CellMax<R>::T><<<v.ncell, CellMax<R>::T, smem, st>>>(v, mode, stats);
-    else cell_kernel<R, 256><<<v.ncell, 256, smem, st>>>(v, mode, stats);
+    if (cell_wide(v)) launch_next(cell_kernel<R, CellMax<R>::T>, v.ncell, CellMax<R>::T, smem, st, v, mode, stats);
+    else launch_next(cell_kernel<R, 256>, v.ncell, 256, smem, st, v, mode, stats);
 }
 
 template <typename R>
@@ -1298,22 +1309,22 @@ void launch_cell_adjoint(const View<R> &v, const AdjView<R> &a, cudaStream_t st)
         if (gs <= CELL_ADJ_GATHER_MAX_SMEM) {
             const int slices = v.slices;
             if (cell_wide(v))
-                cell_adjoint_gather_kernel<CellMax<R>::T><<<v.ncell * slices, CellMax<R>::T, gs, st>>>(v, a, slices);
+                launch_next(cell_adjoint_gather_kernel<CellMax<R>::T>, v.ncell * slices, CellMax<R>::T, gs, st, v, a, slices);
             else
-                cell_adjoint_gather_kernel<256><<<v.ncell * slices, 256, gs, st>>>(v, a, slices);
+                launch_next(cell_adjoint_gather_kernel<256>, v.ncell * slices, 256, gs, st, v, a, slices);
             return;
         }
     }
     if constexpr (std::is_same<R, double>::value) {
         const int chunks = adjoint_chunks(v.max_nt), echunks = adjoint_chunks(v.max_ne);
-        adjoint_records_kernel<<<v.ncell * chunks, ADJ_NT, 0, st>>>(v, a, chunks);
-        adjoint_terms_kernel<<<v.ncell * (chunks + echunks), ADJ_NT, 0, st>>>(v, a, chunks, echunks);
-        adjoint_add_kernel<<<(3 * v.nv + 255) / 256, 256, 0, st>>>(a, 3 * v.nv);
+        launch_next(adjoint_records_kernel, v.ncell * chunks, ADJ_NT, 0, st, v, a, chunks);
+        launch_next(adjoint_terms_kernel, v.ncell * (chunks + echunks), ADJ_NT, 0, st, v, a, chunks, echunks);
+        launch_next(adjoint_add_kernel, (3 * v.nv + 255) / 256, 256, 0, st, a, 3 * v.nv);
     } else {  // meshes whose gather records do not fit
         const size_t smem = cell_adjoint_smem_bytes<R>(v.max_nv, v.max_nt);
         const int slices = std::max(1, std::min(32, v.nsm / v.ncell));
-        if (slices == 1 && cell_wide(v)) cell_adjoint_kernel<R, CellMax<R>::T><<<v.ncell, CellMax<R>::T, smem, st>>>(v, a, 1);
-        else cell_adjoint_kernel<R, 256><<<v.ncell * slices, 256, smem, st>>>(v, a, slices);
+        if (slices == 1 && cell_wide(v)) launch_next(cell_adjoint_kernel<R, CellMax<R>::T>, v.ncell, CellMax<R>::T, smem, st, v, a, 1);
+        else launch_next(cell_adjoint_kernel<R, 256>, v.ncell * slices, 256, smem, st, v, a, slices);
     }
 }
 
@@ -1338,7 +1349,7 @@ cudaError_t set_cell_adjoint_gather_smem_limit(size_t bytes) {
 template <typename R>
 void launch_deformation_loss(const View<R> &v, const double *c0, double *cell_loss, R *dLdX, cudaStream_t st) {
     if (v.ncell == 0) return;
-    deformation_loss_kernel<R><<<v.ncell, 256, 0, st>>>(v, c0, cell_loss, dLdX);
+    launch_next(deformation_loss_kernel<R>, v.ncell, 256, 0, st, v, c0, cell_loss, dLdX);
 }
 
 template void launch_cell_adjoint<double>(const View<double> &, const AdjView<double> &, cudaStream_t);
