@@ -148,7 +148,7 @@ __device__ __forceinline__ void collide_core(const View<R> &v, int n, const Nbr 
     const size_t N = (size_t)v.N;
     R rho, ux, uy, uz;
     const R om = (VISC && v.ind && v.ind[n]) ? v.omega_in : v.omega;  // inside a cell: internal viscosity
-    bgk_guo<R>(d, v.F[n], v.F[N + n], v.F[2 * N + n], om, p, rho, ux, uy, uz);
+    bgk_guo(d, v.F[n], v.F[N + n], v.F[2 * N + n], om, p, rho, ux, uy, uz);
     if (v.rec) {
         v.rec[n] = rho;
         v.rec[N + n] = ux;
@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) collide_tiles_kernel(View<R> 
                                      cx(i) != 0);
                 R rho, ux, uy, uz;
                 const R om = (v.ind && v.ind[(size_t)tl.x * nx + L]) ? v.omega_in : v.omega;
-                bgk_guo<R>(d, Fs[L], Fs[TNM + L], Fs[2 * TNM + L], om, p, rho, ux, uy, uz);
+                bgk_guo(d, Fs[L], Fs[TNM + L], Fs[2 * TNM + L], om, p, rho, ux, uy, uz);
                 if (v.rec) {
                     const size_t n = (size_t)tl.x * nx + L;
                     v.rec[n] = rho;
@@ -511,12 +511,20 @@ __device__ __forceinline__ void moments_core(const View<R> &v, int n, const Nbr 
     R d[Q];
     load_pops<T, R, LAYOUT, LINKS, I>(v, n, lk, o, rr, d);
     R drho = R(0), mx = R(0), my = R(0), mz = R(0);
+    if constexpr (std::is_same<R, double>::value) {
+        R s[9], t[9], m[3];
+        pair_moments<R>(d, s, t, drho, m);
+        mx = m[0];
+        my = m[1];
+        mz = m[2];
+    } else {
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        drho += d[i];
-        if (cx(i)) mx += cx(i) > 0 ? d[i] : -d[i];
-        if (cy(i)) my += cy(i) > 0 ? d[i] : -d[i];
-        if (cz(i)) mz += cz(i) > 0 ? d[i] : -d[i];
+        for (int i = 0; i < Q; ++i) {
+            drho += d[i];
+            if (cx(i)) mx += cx(i) > 0 ? d[i] : -d[i];
+            if (cy(i)) my += cy(i) > 0 ? d[i] : -d[i];
+            if (cz(i)) mz += cz(i) > 0 ? d[i] : -d[i];
+        }
     }
     const size_t N = (size_t)v.N;
     const R inv = recip(R(1) + drho);

@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(NODE_BX * NODE_BY) le_collide_kernel(View<R> v
     for (int i = 0; i < Q; ++i) d[i] = Store<T>::ld(A[(size_t)i * N + n]);
     const R om = (v.ind && v.ind[n]) ? v.omega_in : v.omega;
     R rho, ux, uy, uz;
-    bgk_guo<R>(d, v.F[n], v.F[N + n], v.F[2 * N + n], om, p, rho, ux, uy, uz);
+    bgk_guo(d, v.F[n], v.F[N + n], v.F[2 * N + n], om, p, rho, ux, uy, uz);
 #pragma unroll
     for (int i = 0; i < Q; ++i) B[(size_t)i * N + n] = Store<T>::st(p[i]);
     if (z == 0 || z == v.nz - 1) {  // post-collision moments of the stored values
