@@ -26,6 +26,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include <cooperative_groups.h>
 #include <cuda.h>
 
 #include "hemo_internal.cuh"
@@ -307,15 +308,6 @@ __device__ __forceinline__ void ld4_any(const float *p, float *o) {
 __device__ __forceinline__ void ld4_any(const double *p, double *o) {
     for (int k = 0; k < 4; ++k) o[k] = p[k];
 }
-// four consecutive values from 16-byte aligned shared memory
-__device__ __forceinline__ void ld4v(const double *p, double *o) {
-    const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
-    o[0] = a.x;
-    o[1] = a.y;
-    o[2] = b.x;
-    o[3] = b.y;
-}
-
 // Peskin 4-point weights of nodes floor(X) - 1 .. floor(X) + 2 for the
 // fraction t = X - floor(X) in [0, 1); one square root serves all four.
 template <typename R>
@@ -443,15 +435,12 @@ __device__ __forceinline__ void stage_tile(const View<R> &v, const R *A, const i
 // 64-bit integers with 2^62 in place of 2^30 (quantum max|F| n 2^-65, below
 // FP64 rounding).
 template <typename R> struct TileAcc {
-    using T = long long;
     static constexpr int E = 61;  // log2 of the bound minus one
 };
 template <> struct TileAcc<float> {
-    using T = int;
     static constexpr int E = 29;
 };
-__device__ __forceinline__ long long fixed_of(double x) { return __double2ll_rn(x); }
-template <typename R> struct SpreadCap { static constexpr int CAP = 128; };  // vertices staged at a time (FP64)
+constexpr int SPREAD_CAP = 128, SP64_THREADS = 256;  // vertices staged at a time, threads (FP64)
 
 // the scale of a component from its largest force; 0 (and the numeric
 // status) for forces that are not finite
@@ -700,77 +689,117 @@ __global__ void __launch_bounds__(SP_CHUNK, 6) spread_tile_f32_kernel(View<float
     }
 }
 
-// FP64: one CTA per bin and force component (three times the CTAs on the
-// FP64 pipes, which a bin's vertices keep busy for long); a warp takes two
+// FP64: a cluster of three CTAs per bin, one for each force component (three
+// times the CTAs on the FP64 pipes, which a bin's vertices keep busy for long);
+// each computes the weights of one axis for all three.  A warp takes two
 // vertices, each half-warp's 16 lanes own one (y, z) row of the stencil.
-// Bound by the FP64 pipe (products and conversions) and 64-bit shared
-// atomics (12 cycles per warp).  Spreading phase of the 32^3 box with one cell
-// 51 -> 26 us, of a 48 x 39 x 64 channel with 30 cells 143 -> 78 us (one CTA
-// per bin; weights by one thread per vertex).
-template <typename R>
-__global__ void __launch_bounds__(256) spread_tile_kernel(View<R> v) {
+// Bound by the FP64 pipe (19 cycles per warp instruction), then by the shared
+// atomics: the four weights along x are w0, 1/2 - w3, 1/2 - w0, w3, so a row
+// takes three conversions and two products, the other two nodes a subtraction
+// of integers; the 64-bit sums are kept as two words with the carry taken from
+// the first atomic (4 cycles per warp instruction; a 64-bit shared atomic takes
+// 12).  48 x 39 x 64 channel with 30 cells: 65 ->
+// 50 us; 32^3 box with one cell: 16.7 -> 11.7 us.
+__device__ __forceinline__ void fixed_add(unsigned *lo, unsigned *hi, long long x) {
+    const unsigned xl = (unsigned)x, old = atomicAdd(lo, xl);
+    atomicAdd(hi, (unsigned)((unsigned long long)x >> 32) + (old + xl < xl));
+}
+__global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(SP64_THREADS) spread_tile_kernel(View<double> v) {
     wait_previous();
-    using A = typename TileAcc<R>::T;
-    constexpr int CAP = SpreadCap<R>::CAP;
-    const int k = blockIdx.x / 3, d = blockIdx.x - 3 * k;
+    constexpr int CAP = SPREAD_CAP, W = 10;  // 2 w0 and 2 w3 along x, four weights along y and z
+    const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const int k = blockIdx.x / 3, d = (int)cluster.block_rank();
     const int s = v.start[k], e = v.start[k + 1];
-    if (s == e) return;
-    __shared__ A acc[TILE_SMEM];
+    if (s == e) return;  // (the whole cluster)
+    __shared__ unsigned lo[TILE_SMEM], hi[TILE_SMEM];
     __shared__ int srow[CAP];
-    __shared__ __align__(16) R sw[12 * CAP];
-    __shared__ R sF[CAP];
-    __shared__ R smax[8];
-    __shared__ R scale_s;
-    for (int q = threadIdx.x; q < TILE_SMEM; q += blockDim.x) acc[q] = A(0);
+    __shared__ __align__(16) double sw[W * CAP];
+    __shared__ double sF[CAP];
+    __shared__ unsigned long long smax[SP64_THREADS / 32];
+    __shared__ double scale_s;
+    for (int q = threadIdx.x; q < TILE_SMEM; q += blockDim.x) lo[q] = hi[q] = 0u;
     int org[3];
     bin_origin(v, k, org);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int h = lane >> 4, b = lane & 3, c = (lane >> 2) & 3;
-    {  // the component's scale for the whole bin
-        R m = R(0);
+    {  // the component's scale for the whole bin: largest |F|, compared as integers (as fmax, ignoring NaN)
+        constexpr unsigned long long INF = 0x7ff0000000000000ull;
+        unsigned long long m = 0;
         for (int j = s + threadIdx.x; j < e; j += blockDim.x) {
             const int i = v.perm[j];
             if (!index_ok(i >= 0 && i < v.nv, v.status)) continue;
-            m = fmax(m, fabs(v.Fv[3 * (size_t)i + d]));
+            const unsigned long long f = (unsigned long long)__double_as_longlong(fabs(v.Fv[3 * (size_t)i + d]));
+            if (f <= INF && f > m) m = f;
         }
-        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (lane == 0) smax[warp] = m;
+        const unsigned mh = (unsigned)(m >> 32), wh = __reduce_max_sync(0xffffffffu, mh);
+        const unsigned wl = __reduce_max_sync(0xffffffffu, mh == wh ? (unsigned)m : 0u);
+        if (lane == 0) smax[warp] = (unsigned long long)wh << 32 | wl;
         __syncthreads();
         if (threadIdx.x == 0) {
-            for (int w = 1; w < nw; ++w) m = fmax(m, smax[w]);
-            scale_s = tile_scale(m, e - s, v.status);
+            for (int w = 0; w < nw; ++w) m = max(m, smax[w]);
+            scale_s = tile_scale(__longlong_as_double((long long)m), e - s, v.status);
         }
-        __syncthreads();
+        cluster.sync();  // (and the cluster's shared memory is in place)
     }
-    const R scale = scale_s;
+    const double scale = scale_s;
+    double *peer[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) peer[r] = cluster.map_shared_rank(sw, r) + (d == 0 ? 0 : 4 * d - 2);
     const int nch = (e - s + CAP - 1) / CAP, csz = (e - s + nch - 1) / nch;
     for (int p0 = s; p0 < e; p0 += csz) {
         const int n = min(csz, e - p0);
-        if (p0 != s) __syncthreads();
-        stage_chunk(v, p0, n, org, srow, (int *)nullptr, [&](int j, int i, int ax, R t) {
-            peskin4(t, sw + 12 * j + 4 * ax);
-            if (ax == 0) sF[j] = v.Fv[3 * (size_t)i + d] * scale;
-        });
-        __syncthreads();
+        if (p0 != s) cluster.sync();
+        for (int j = threadIdx.x; j < n; j += blockDim.x) {
+            const int i = v.perm[p0 + j];
+            int row = 0;
+            bool ok = index_ok(i >= 0 && i < v.nv, v.status);
+            if (ok) {
+                double w[4];
+                peskin4(v.anc_t[3 * (size_t)i + d], w);
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    double *o = peer[r] + W * j;
+                    if (d == 0) {
+                        o[0] = 2.0 * w[0];
+                        o[1] = 2.0 * w[3];
+                    } else {
+                        for (int a = 0; a < 4; ++a) o[a] = w[a];
+                    }
+                }
+                sF[j] = v.Fv[3 * (size_t)i + d] * (0.5 * scale);
+                for (int a = 0; a < 3; ++a) {
+                    const int q = v.anc_i[3 * (size_t)i + a] - org[a];
+                    ok &= q >= 0 && q < BLK;
+                    row += q * (a == 0 ? 1 : (a == 1 ? TS_Y : TS_Z));
+                }
+            }
+            srow[j] = ok ? row : -1;
+        }
+        cluster.sync();
         for (int q = 2 * warp + h; q < n; q += 2 * nw) {
             const int row0 = srow[q];
             if (row0 < 0) continue;  // vertex outside the lattice (domain status already raised)
-            const R *w = sw + 12 * q;
-            const R f = sF[q] * (w[4 + b] * w[8 + c]);
-            R wx[4];
-            ld4v(w, wx);
+            const double *w = sw + W * q;
+            const double g = sF[q] * (w[2 + b] * w[6 + c]);  // half the row's force
+            const double2 x = *reinterpret_cast<const double2 *>(w);
+            const long long qh = __double2ll_rn(g), q0 = __double2ll_rn(g * x.x), q3 = __double2ll_rn(g * x.y);
+            const long long f[4] = {q0, qh - q3, qh - q0, q3};
             const int row = row0 + TS_Y * b + TS_Z * c;
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
-                atomicAdd((unsigned long long *)&acc[row + a], (unsigned long long)fixed_of(f * wx[a]));
+            for (int a = 0; a < 4; ++a) fixed_add(lo + row + a, hi + row + a, f[a]);
         }
     }
     __syncthreads();
-    R *out = v.tiles + ((size_t)k * 3 + d) * TP_N;
-    const R inv = scale > R(0) ? R(1) / scale : R(0);  // (exact: a power of two)
+    // write-out, divided by the scale (a power of two) through the exponent
+    double *out = v.tiles + ((size_t)k * 3 + d) * TP_N;
+    const long long ex = scale > 0.0 ? (long long)ilogb(scale) << 52 : 0;
     TileWalk tw(threadIdx.x, blockDim.x);
-    for (int q = threadIdx.x; q < TILE3; q += blockDim.x, tw.next())
-        out[tile_index(tw.l0, tw.l1, tw.l2)] = (R)acc[tw.l0 + TS_Y * tw.l1 + TS_Z * tw.l2] * inv;
+    for (int q = threadIdx.x; q < TILE3; q += blockDim.x, tw.next()) {
+        const int p = tw.l0 + TS_Y * tw.l1 + TS_Z * tw.l2;
+        const long long x = scale > 0.0 ? (long long)((unsigned long long)hi[p] << 32 | lo[p]) : 0;
+        const long long f = __double_as_longlong((double)x);
+        out[tile_index(tw.l0, tw.l1, tw.l2)] = __longlong_as_double(x ? f - ex : 0);
+    }
 }
 
 // Phase 2 of spreading (owner computes): one CTA per 8^3 block sums, for
@@ -1597,7 +1626,7 @@ void launch_bin_ranges(const View<R> &v, cudaStream_t st) {
 template <typename R>
 void launch_spread(const View<R> &v, cudaStream_t st) {
     if constexpr (std::is_same<R, float>::value) launch_next(spread_tile_f32_kernel, v.nbins, SP_CHUNK, 0, st, v);
-    else launch_next(spread_tile_kernel<R>, 3 * v.nbins, 256, 0, st, v);
+    else launch_next(spread_tile_kernel, 3 * v.nbins, SP64_THREADS, 0, st, v);
     if (v.nb[0] >= 3 && v.nb[1] >= 3 && v.nb[2] >= 3) launch_next(spread_gather3_kernel<R>, v.nbins, 256, 0, st, v);
     else launch_next(spread_gather_kernel<R>, v.nbins, 256, 0, st, v);
 }
