@@ -164,7 +164,7 @@ struct hemo_sim {
     int *vcell_d = nullptr, *cell_first_d = nullptr, *cell_type_d = nullptr;
     void *meshes_d = nullptr;
     int nb[3] = {1, 1, 1}, nbins = 1;
-    int *key = nullptr, *counts = nullptr, *start = nullptr, *cursor = nullptr, *perm_raw = nullptr, *perm = nullptr;
+    int *key = nullptr, *counts = nullptr, *start = nullptr, *cursor = nullptr, *perm_raw = nullptr, *perm = nullptr, *order = nullptr;
     int *anc_i = nullptr;
     void *anc_t = nullptr;
     void *tiles = nullptr;
@@ -359,6 +359,7 @@ View<R> make_view(hemo_sim *s) {
     v.counts = s->counts;
     v.start = s->start;
     v.cursor = s->cursor;
+    v.order = s->order;
     v.perm_raw = s->perm_raw;
     v.perm = s->perm;
     v.anc_i = s->anc_i;
@@ -466,6 +467,8 @@ int finalize_impl(hemo_sim *s) {
     // one more bin than the lattice has: the vertices at the Lees-Edwards plane
     s->counts = (int *)dalloc(s, sizeof(int) * (s->nbins + 1));
     s->cursor = (int *)dalloc(s, sizeof(int) * (s->nbins + 1));
+    // the bins by size for the vertex kernels' grids, where the scan of a step lists them
+    if (bins_ordered(s->nbins + 1, nv)) s->order = (int *)dalloc(s, sizeof(int) * s->nbins);
     s->start = (int *)dalloc(s, sizeof(int) * (s->nbins + 2));
     s->tiles = dalloc(s, rs * 3 * (size_t)SPREAD_NODES * s->nbins);
     s->Uprev = dalloc(s, rs * 3 * std::max(nv, 1));

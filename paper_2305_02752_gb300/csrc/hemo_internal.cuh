@@ -165,6 +165,7 @@ template <typename R> struct View {
     int *counts;               // nbins
     int *start;                // nbins + 1
     int *cursor;               // nbins
+    int *order;                // nbins: the bins by size, or null: as they come
     int *perm_raw;             // nv, unsorted within bins
     int *perm;                 // nv, stable (key, vertex id)
     int *anc_i;                // nv*3 stencil base floor(X) (wrapped on periodic axes)
@@ -287,6 +288,10 @@ template <typename R> size_t cell_smem_bytes(int max_nv, int max_nt, int max_ne)
 template <typename R> void launch_bins(const View<R> &v, cudaStream_t st, bool stable);
 // the bin ranges and the (unstable) order once the step's membrane kernel
 // has written the anchors, keys and counts
+// up to this many bins and vertices scan and scatter are one CTA's work; above
+// this many vertices, and up to as many bins, the scan also lists the bins by size
+constexpr int SMALL_BINS = 4096, SMALL_NV = 8192;
+inline bool bins_ordered(int nbins, int nv) { return nbins <= SMALL_BINS && nv > SMALL_NV; }
 template <typename R> void launch_bin_ranges(const View<R> &v, cudaStream_t st);
 template <typename R> void launch_spread(const View<R> &v, cudaStream_t st);
 template <typename R> void launch_interpolate(const View<R> &v, cudaStream_t st);

@@ -135,9 +135,13 @@ __device__ __forceinline__ void store_quad(int *p, int k, int n, bool vec, int4 
     if (k + 2 < n) p[k + 2] = q.z;
     if (k + 3 < n) p[k + 3] = q.w;
 }
-__global__ void __launch_bounds__(1024) scan_kernel(int *counts, int *start, int *cursor, int nbins) {
+// With `order` (norder <= nbins <= 4096) also the bins by size: those of more than
+// 2 `mean` vertices, then those of more than mean / 2, then the rest, each in
+// natural order.
+__global__ void __launch_bounds__(1024) scan_kernel(int *counts, int *start, int *cursor, int nbins, int *order,
+                                                    int norder, int mean) {
     wait_previous();
-    __shared__ int wsum[32];
+    __shared__ int wsum[32], wclass[32];
     __shared__ int carry_s;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const bool vec = (((uintptr_t)counts | (uintptr_t)start | (uintptr_t)cursor) & 15) == 0;
@@ -172,6 +176,32 @@ __global__ void __launch_bounds__(1024) scan_kernel(int *counts, int *start, int
         store_quad(start, k0, nbins, vec, ex);
         store_quad(cursor, k0, nbins, vec, ex);
         store_quad(counts, k0, nbins, vec, make_int4(0, 0, 0, 0));
+        if (order) {  // ranks within the first two classes, 16 bits each
+            const int n[4] = {c.x, c.y, c.z, c.w};
+            int mine = 0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (k0 + j < norder) mine += n[j] > 2 * mean ? 1 : (2 * n[j] > mean ? 0x10000 : 0);
+            int y = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int z = __shfl_up_sync(0xffffffffu, y, o);
+                if (lane >= o) y += z;
+            }
+            if (lane == 31) wclass[w] = y;
+            __syncthreads();
+            const int tot = wclass[lane], all = __reduce_add_sync(0xffffffffu, tot);
+            const int at = __reduce_add_sync(0xffffffffu, lane < w ? tot : 0) + y - mine;
+            int r0 = at & 0xffff, r1 = at >> 16;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int k = k0 + j, n0 = all & 0xffff, n1 = all >> 16;
+                if (k >= norder) break;
+                if (n[j] > 2 * mean) order[r0++] = k;
+                else if (2 * n[j] > mean) order[n0 + r1++] = k;
+                else order[n0 + n1 + k - r0 - r1] = k;
+            }
+        }
         carry += carry_s;
         __syncthreads();  // (wsum and carry_s are rewritten by the next tile)
     }
@@ -199,7 +229,6 @@ __global__ void scatter_kernel(const int *key, int *cursor, int *perm_raw, int n
 // Few blocks and vertices: scan and scatter by one CTA, the cursors in shared
 // memory (48^3 box, 2568 vertices: 4.1 us against 2.6 + 2.5 and the gap between
 // two launches).  Above these sizes one SM is the slower.
-constexpr int SMALL_BINS = 4096, SMALL_NV = 8192;
 __global__ void __launch_bounds__(1024) scan_scatter_kernel(int *counts, int *start, int nbins, const int *key, int *perm,
                                                             int nv, unsigned *status) {
     wait_previous();
@@ -372,6 +401,18 @@ __device__ __forceinline__ int neighbour_blocks(int b, int nb, int periodic, int
     return cnt;
 }
 
+// The b-th bin of a vertex kernel's grid: by size where the list is kept.
+// Bins hold from none to several times the mean, and a grid of a few CTAs per
+// SM ends when its largest does: with the largest first, 48 x 39 x 64 channel,
+// FP64 interpolation 33 -> 30 us; 64 x 64 x 256 channel, FP32 spreading 27.4 ->
+// 25.9, interpolation 29.6 -> 28.3, for 0.7 us more in the scan.  Not for more
+// than 4096 bins, where neighbours' tiles share the cache and the end matters
+// less.
+template <typename R>
+__device__ __forceinline__ int bin_of(const View<R> &v, int b) {
+    return v.order ? v.order[b] : b;
+}
+
 // FP64 vertex kernels: anchors and weights of one chunk of a bin, staged in
 // shared memory, a thread per vertex and axis (the square roots run on the FP64
 // pipe and are a long chain): the row in the bin's padded tile (-1 if the
@@ -440,7 +481,7 @@ template <typename R> struct TileAcc {
 template <> struct TileAcc<float> {
     static constexpr int E = 29;
 };
-constexpr int SPREAD_CAP = 128, SP64_THREADS = 256;  // vertices staged at a time, threads (FP64)
+constexpr int SPREAD_CAP = 352, SP64_THREADS = 512;  // vertices staged at a time, threads (FP64)
 
 // the scale of a component from its largest force; 0 (and the numeric
 // status) for forces that are not finite
@@ -542,7 +583,7 @@ __device__ __forceinline__ void spread_item(int *first, int s, const float (&F)[
 
 __global__ void __launch_bounds__(SP_CHUNK, 6) spread_tile_f32_kernel(View<float> v) {
     wait_previous();
-    const int k = blockIdx.x;
+    const int k = bin_of(v, blockIdx.x);
     const int s = v.start[k], e = v.start[k + 1], n = e - s;
     if (n == 0) return;
     __shared__ __align__(16) int tile[3 * SP_N];
@@ -699,7 +740,9 @@ __global__ void __launch_bounds__(SP_CHUNK, 6) spread_tile_f32_kernel(View<float
 // of integers; the 64-bit sums are kept as two words with the carry taken from
 // the first atomic (4 cycles per warp instruction; a 64-bit shared atomic takes
 // 12).  48 x 39 x 64 channel with 30 cells: 65 ->
-// 50 us; 32^3 box with one cell: 16.7 -> 11.7 us.
+// 50 us; 32^3 box with one cell: 16.7 -> 11.7 us.  Threads for a whole SM's
+// registers, so that three CTAs fit and the others follow as these end, the
+// largest bins first: the channel 50 -> 35 us.
 __device__ __forceinline__ void fixed_add(unsigned *lo, unsigned *hi, long long x) {
     const unsigned xl = (unsigned)x, old = atomicAdd(lo, xl);
     atomicAdd(hi, (unsigned)((unsigned long long)x >> 32) + (old + xl < xl));
@@ -708,7 +751,7 @@ __global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(SP64_THREADS) spread
     wait_previous();
     constexpr int CAP = SPREAD_CAP, W = 10;  // 2 w0 and 2 w3 along x, four weights along y and z
     const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
-    const int k = blockIdx.x / 3, d = (int)cluster.block_rank();
+    const int k = bin_of(v, blockIdx.x / 3), d = (int)cluster.block_rank();
     const int s = v.start[k], e = v.start[k + 1];
     if (s == e) return;  // (the whole cluster)
     __shared__ unsigned lo[TILE_SMEM], hi[TILE_SMEM];
@@ -1062,7 +1105,7 @@ __global__ void __launch_bounds__(256) interpolate_kernel(View<R> v, int parts) 
     wait_previous();
     drop_dead_lines(v);
     constexpr int CAP = InterpCap;
-    const int k = blockIdx.x / parts, part = blockIdx.x % parts;  // CTA part takes chunks part, part + parts, ...
+    const int k = bin_of(v, blockIdx.x % v.nbins), part = blockIdx.x / v.nbins;  // CTA part takes chunks part, part + parts, ...
     const int s = v.start[k], e = v.start[k + 1];
     if (s + part * CAP >= e) return;
     __shared__ R tile[3][TILE_SMEM];
@@ -1159,7 +1202,7 @@ template <int INTEG>
 __global__ void __launch_bounds__(IT_CHUNK, 6) interpolate_v4_kernel(View<float> v, const __grid_constant__ CUtensorMap umap) {
     wait_previous();
     drop_dead_lines(v);
-    const int k = blockIdx.x;
+    const int k = bin_of(v, blockIdx.x);
     const int s = v.start[k], e = v.start[k + 1];
     if (s == e) return;
     __shared__ __align__(128) unsigned char tile_raw[INTERP_SMEM];
@@ -1395,7 +1438,7 @@ __global__ void __launch_bounds__(256) vertex_field_kernel(View<R> v, const R *A
                                                            R *out_interp, int parts) {
     wait_previous();
     constexpr int CAP = VfStage<R>::CAP;
-    const int k = blockIdx.x / parts, part = blockIdx.x % parts;  // CTA part takes chunks part, part + parts, ...
+    const int k = bin_of(v, blockIdx.x % v.nbins), part = blockIdx.x / v.nbins;  // CTA part takes chunks part, part + parts, ...
     const int s = v.start[k], e = v.start[k + 1];
     if (s + part * CAP >= e) return;
     __shared__ R tile[3][TILE_SMEM];
@@ -1468,7 +1511,7 @@ __global__ void __launch_bounds__(256) vertex_field_kernel(View<R> v, const R *A
 __global__ void __launch_bounds__(256) vertex_field_v4_kernel(View<float> v, const float *A, const float *B,
                                                               float *out_grad, float *out_interp) {
     wait_previous();
-    const int k = blockIdx.x;
+    const int k = bin_of(v, blockIdx.x);
     const int s = v.start[k], e = v.start[k + 1];
     if (s == e) return;
     __shared__ float4 tile[TILE_SMEM];
@@ -1603,7 +1646,7 @@ template <typename R>
 void launch_bins(const View<R> &v, cudaStream_t st, bool stable) {
     cudaMemsetAsync(v.counts, 0, sizeof(int) * v.nbins, st);
     launch_next(anchor_count_kernel<R>, nblocks(v.nv, 256), 256, 0, st, v);
-    launch_next(scan_kernel, 1, 1024, 0, st, v.counts, v.start, v.cursor, v.nbins);
+    launch_next(scan_kernel, 1, 1024, 0, st, v.counts, v.start, v.cursor, v.nbins, nullptr, 0, 0);
     if (stable) {
         launch_next(scatter_kernel, nblocks(v.nv, 256), 256, 0, st, v.key, v.cursor, v.perm_raw, v.nv, v.status);
         launch_next(sort_bins_kernel, nblocks((long long)v.nbins * 32, 128), 128, 0, st, v.start, v.perm_raw, v.perm, v.nbins);
@@ -1619,7 +1662,7 @@ void launch_bin_ranges(const View<R> &v, cudaStream_t st) {
         launch_next(scan_scatter_kernel, 1, 1024, 0, st, v.counts, v.start, nbins, v.key, v.perm, v.nv, v.status);
         return;
     }
-    launch_next(scan_kernel, 1, 1024, 0, st, v.counts, v.start, v.cursor, nbins);
+    launch_next(scan_kernel, 1, 1024, 0, st, v.counts, v.start, v.cursor, nbins, v.order, v.nbins, v.nv / v.nbins);
     launch_next(scatter_kernel, nblocks(v.nv, 256), 256, 0, st, v.key, v.cursor, v.perm, v.nv, v.status);
 }
 
@@ -1797,7 +1840,7 @@ extern "C" int hemo_bin_vertices_noalloc(const double *verts, int nv, int nx, in
     if (nv > 0)
         abs_key_count_kernel<<<(nv + 255) / 256, 256, 0, st>>>(verts, nv, nx, ny, nz, periodic[0] != 0, periodic[1] != 0,
                                                                periodic[2] != 0, (int)nb0, (int)nb1, key, counts);
-    scan_kernel<<<1, 1024, 0, st>>>(counts, start, cursor, nbins);
+    scan_kernel<<<1, 1024, 0, st>>>(counts, start, cursor, nbins, nullptr, 0, 0);
     if (nv > 0) {
         scatter_kernel<<<(nv + 255) / 256, 256, 0, st>>>(key, cursor, perm_raw, nv, nullptr);
         sort_bins_kernel<<<(int)(((long long)nbins * 32 + 127) / 128), 128, 0, st>>>(start, perm_raw, perm, nbins);
