@@ -503,7 +503,7 @@ int finalize_impl(hemo_sim *s) {
         // over far-apart mesh parts, made for scattering atomics).  The FP64
         // adjoint, which still scatters with atomics, walks the same tables
         // with a coprime stride (MeshDev::tstride, estride).
-        std::vector<int> edge_p(4 * (size_t)m.ne), tri_p(3 * (size_t)m.nt), tpos(m.nt), etri_p(2 * (size_t)m.ne);
+        std::vector<int> edge_p(4 * (size_t)m.ne), tri_p(3 * (size_t)m.nt), etri_p(2 * (size_t)m.ne);
         std::vector<R> invL0(m.ne), th0(m.ne);
         std::vector<R> At0_p(m.nt);
         std::vector<int> tord(m.nt), eord(m.ne);
@@ -516,23 +516,7 @@ int finalize_impl(hemo_sim *s) {
         for (int q = 0; q < m.nt; ++q) {
             const int t = tord[q];
             for (int j = 0; j < 3; ++j) tri_p[3 * (size_t)q + j] = m.tri[3 * (size_t)t + j];
-            tpos[t] = q;
             At0_p[q] = R(m.At0[t]);
-        }
-        // triangle of each directed edge: (v0, v1) -> triangle containing it
-        std::unordered_map<long long, int> dir_tri;
-        dir_tri.reserve(3 * (size_t)m.nt);
-        for (int t = 0; t < m.nt; ++t)
-            for (int k = 0; k < 3; ++k)
-                dir_tri[(long long)m.tri[3 * t + k] * m.nv + m.tri[3 * t + (k + 1) % 3]] = t;
-        for (int q = 0; q < m.ne; ++q) {
-            const int e = eord[q];
-            const int *E = &m.edge[4 * (size_t)e];
-            for (int j = 0; j < 4; ++j) edge_p[4 * (size_t)q + j] = E[j];
-            etri_p[2 * (size_t)q] = tpos[dir_tri.at((long long)E[0] * m.nv + E[1])];
-            etri_p[2 * (size_t)q + 1] = tpos[dir_tri.at((long long)E[1] * m.nv + E[0])];
-            invL0[q] = R(1.0 / m.L0[e]);
-            th0[q] = R(m.th0[e]);
         }
         // the triangles of each vertex (processing order): {triangle, next
         // corner, the one after}
@@ -543,6 +527,21 @@ int finalize_impl(hemo_sim *s) {
             tri4[q] = make_int4(T[0], T[1], T[2], 0);
             for (int r = 0; r < 3; ++r) tris[T[r]].push_back(make_int4(q, T[(r + 1) % 3], T[(r + 2) % 3], 0));
         }
+        // the triangle containing the directed edge (a, b), or -1 (a vertex has few triangles)
+        auto tri_of = [&](int a, int b) {
+            for (const int4 &g : tris[a])
+                if (g.y == b) return g.x;
+            return -1;
+        };
+        for (int q = 0; q < m.ne; ++q) {
+            const int e = eord[q];
+            const int *E = &m.edge[4 * (size_t)e];
+            for (int j = 0; j < 4; ++j) edge_p[4 * (size_t)q + j] = E[j];
+            for (int r = 0; r < 2; ++r)
+                if ((etri_p[2 * (size_t)q + r] = tri_of(E[r], E[1 - r])) < 0) return fail(HEMO_ERR_ARG, "mesh: an edge without its triangles");
+            invL0[q] = R(1.0 / m.L0[e]);
+            th0[q] = R(m.th0[e]);
+        }
         int maxv = 0;  // largest valence (on a closed manifold: triangles = edges per vertex)
         for (int i = 0; i < m.nv; ++i) maxv = std::max(maxv, (int)tris[i].size());
         // the fan of each vertex i in cyclic order: triangles T_k = (i, j_k,
@@ -550,25 +549,28 @@ int finalize_impl(hemo_sim *s) {
         // Slot 0 repeats the last entry (the loop's carried values start
         // from it), slots 1..deg hold k = 0..deg-1; per entry {T_k, j_k,
         // edge (i, j_k) << 1 | role of i in it, edge (j_k, j_k+1)}.
-        std::unordered_map<long long, int> pair_edge;
-        pair_edge.reserve(2 * (size_t)m.ne);
+        std::vector<std::vector<std::pair<int, int>>> edges(m.nv);  // by the smaller vertex: {the larger, edge}
         for (int q = 0; q < m.ne; ++q) {
             const int a = edge_p[4 * (size_t)q], b = edge_p[4 * (size_t)q + 1];
-            pair_edge[(long long)std::min(a, b) * m.nv + std::max(a, b)] = q;
+            edges[std::min(a, b)].push_back({std::max(a, b), q});
         }
-        auto edge_of = [&](int a, int b) { return pair_edge.at((long long)std::min(a, b) * m.nv + std::max(a, b)); };
+        auto edge_of = [&](int a, int b) {
+            for (const auto &e : edges[std::min(a, b)])
+                if (e.first == std::max(a, b)) return e.second;
+            return -1;
+        };
         std::vector<int4> vfan((size_t)(maxv + 1) * m.nv, make_int4(-1, 0, 0, 0));
         for (int i = 0; i < m.nv; ++i) {
-            std::unordered_map<int, int4> from;  // j_k -> {T_k, j_k, j_k+1}
-            for (const int4 &g : tris[i]) from[g.y] = make_int4(g.x, g.y, g.z, 0);
             const int deg = (int)tris[i].size();
             std::vector<int4> fan;
             int j = tris[i][0].y;
             for (int k = 0; k < deg; ++k) {
-                const auto it = from.find(j);
-                if (it == from.end()) return fail(HEMO_ERR_ARG, "mesh: a vertex's triangles do not form one fan");
-                const int4 T = it->second;
-                const int e = edge_of(i, j), role = edge_p[4 * (size_t)e] == i ? 0 : 1;
+                int4 T = make_int4(-1, 0, 0, 0);  // {T_k, j_k, j_k+1}
+                for (const int4 &g : tris[i])
+                    if (g.y == j) T = g;
+                const int e = edge_of(i, j);
+                if (T.x < 0 || e < 0 || edge_of(T.y, T.z) < 0) return fail(HEMO_ERR_ARG, "mesh: a vertex's triangles do not form one fan");
+                const int role = edge_p[4 * (size_t)e] == i ? 0 : 1;
                 // the edge's triangle lists: (v0, v1, a) first, (v1, v0, b) second
                 const int t_in = etri_p[2 * (size_t)e + role];  // contains i -> j
                 if (t_in != T.x) return fail(HEMO_ERR_ARG, "mesh: inconsistent orientation in a vertex fan");
@@ -611,33 +613,39 @@ int finalize_impl(hemo_sim *s) {
             // edges and those opposite, and the triangles of all these edges; a
             // triangle is owned by the slice of its smallest vertex
             const int S = s->slices, per = (m.nv + S - 1) / S;
-            std::vector<int> items, at(2 * (S + 1));
-            std::vector<std::vector<int>> se(S);
+            std::vector<int> items, at(2 * (S + 1)), edges_of, tin(m.nt, -1), ein(m.ne, -1), tl, el;
             for (int r = 0; r < S; ++r) {
-                std::vector<char> tin(m.nt, 0), ein(m.ne, 0);
-                for (int i = std::min(m.nv, r * per); i < std::min(m.nv, (r + 1) * per); ++i)
-                    for (int k = 1; k <= maxv; ++k) {
+                tl.clear();
+                el.clear();
+                auto add = [&](std::vector<int> &in, std::vector<int> &list, int q) {
+                    if (in[q] == r) return;
+                    in[q] = r;
+                    list.push_back(q);
+                };
+                for (int k = 1; k <= maxv; ++k)
+                    for (int i = std::min(m.nv, r * per); i < std::min(m.nv, (r + 1) * per); ++i) {
                         const int4 g = vfan[(size_t)k * m.nv + i];
-                        if (g.x < 0) break;
-                        tin[g.x] = 1;
-                        ein[g.z >> 1] = ein[g.w] = 1;
+                        if (g.x < 0) continue;
+                        add(tin, tl, g.x);
+                        add(ein, el, g.z >> 1);
+                        add(ein, el, g.w);
                     }
-                for (int e = 0; e < m.ne; ++e)
-                    if (ein[e]) {
-                        tin[etri_p[2 * (size_t)e]] = tin[etri_p[2 * (size_t)e + 1]] = 1;
-                        se[r].push_back(e);
-                    }
+                for (int e : el)
+                    for (int j = 0; j < 2; ++j) add(tin, tl, etri_p[2 * (size_t)e + j]);
+                std::sort(tl.begin(), tl.end());
+                std::sort(el.begin(), el.end());
                 at[r] = (int)items.size();
-                for (int q = 0; q < m.nt; ++q) {
+                for (int q : tl) {
                     const int4 T = tri4[q];
-                    if (tin[q]) items.push_back(q << 1 | (std::min({T.x, T.y, T.z}) / per == r ? 1 : 0));
+                    items.push_back(q << 1 | (std::min({T.x, T.y, T.z}) / per == r ? 1 : 0));
                 }
+                at[S + 1 + r] = (int)edges_of.size();
+                edges_of.insert(edges_of.end(), el.begin(), el.end());
             }
             at[S] = (int)items.size();
-            for (int r = 0; r <= S; ++r) {
-                at[S + 1 + r] = (int)items.size();
-                if (r < S) items.insert(items.end(), se[r].begin(), se[r].end());
-            }
+            at[2 * S + 1] = (int)edges_of.size();
+            for (int r = 0; r <= S; ++r) at[S + 1 + r] += at[S];
+            items.insert(items.end(), edges_of.begin(), edges_of.end());
             int *ditems = (int *)dalloc(s, sizeof(int) * items.size()), *dat = (int *)dalloc(s, sizeof(int) * at.size());
             if (!ditems || !dat) return fail(HEMO_ERR_OOM, "device allocation of mesh tables failed");
             HEMO_CU(cudaMemcpy(ditems, items.data(), sizeof(int) * items.size(), cudaMemcpyHostToDevice));
