@@ -387,10 +387,13 @@ __device__ __forceinline__ void sum16(const R (&x)[K], R (&out)[K]) {
 // others are done)
 constexpr int FP64_BIN_PARTS = 8;
 
-// distinct neighbour block coordinates along one axis
-__device__ __forceinline__ int neighbour_blocks(int b, int nb, int periodic, int out[3]) {
+// distinct coordinates of the blocks whose vertices reach block b along an axis
+// of n nodes: the neighbours, and for the first block of a periodic axis whose
+// last block has a single node the block before that one too (a stencil reaches
+// two nodes beyond its block)
+__device__ __forceinline__ int neighbour_blocks(int b, int nb, int n, int periodic, int out[4]) {
     int cnt = 0;
-    for (int d = -1; d <= 1; ++d) {
+    for (int d = periodic && b == 0 && n % BLK == 1 ? -2 : -1; d <= 1; ++d) {
         int q = b + d;
         if (periodic) q = wrap(q, nb);
         else if (q < 0 || q >= nb) continue;
@@ -855,15 +858,15 @@ constexpr int GATHER_MAXE = 2 * TILE;  // entries per (axis, local coordinate)
 template <typename R>
 __global__ void __launch_bounds__(256) spread_gather_kernel(View<R> v) {
     wait_previous();
-    __shared__ int nbin[27];  // bin of neighbour slot (sz*9 + sy*3 + sx), -1 if empty
-    __shared__ int lb[3][3], nsl[3];
+    __shared__ int nbin[64];  // bin of neighbour slot (sz*16 + sy*4 + sx), -1 if empty
+    __shared__ int lb[3][4], nsl[3];
     __shared__ unsigned char cnt[3][BLK];
     __shared__ unsigned char ent_slot[3][BLK][GATHER_MAXE], ent_pos[3][BLK][GATHER_MAXE];
     const int k = blockIdx.x;
     const int bc[3] = {k % v.nb[0], (k / v.nb[0]) % v.nb[1], k / (v.nb[0] * v.nb[1])};
     const int dims[3] = {v.nx, v.ny, v.nz};
     const int t = threadIdx.x;
-    if (t < 3) nsl[t] = neighbour_blocks(bc[t], v.nb[t], v.per[t], lb[t]);
+    if (t < 3) nsl[t] = neighbour_blocks(bc[t], v.nb[t], dims[t], v.per[t], lb[t]);
     __syncthreads();
     if (t < 3 * BLK) {  // table of axis d, local coordinate l
         const int d = t / BLK, l = t % BLK;
@@ -882,8 +885,8 @@ __global__ void __launch_bounds__(256) spread_gather_kernel(View<R> v) {
             }
         }
         cnt[d][l] = (unsigned char)n;
-    } else if (t >= 32 && t < 32 + 27) {  // neighbour slot -> bin
-        const int sl = t - 32, a = sl / 9, b = (sl / 3) % 3, c = sl % 3;
+    } else if (t >= 32 && t < 32 + 64) {  // neighbour slot -> bin
+        const int sl = t - 32, a = sl / 16, b = (sl / 4) % 4, c = sl % 4;
         int kk = -1;
         if (a < nsl[2] && b < nsl[1] && c < nsl[0]) {
             kk = lb[0][c] + v.nb[0] * (lb[1][b] + v.nb[1] * lb[2][a]);
@@ -901,7 +904,7 @@ __global__ void __launch_bounds__(256) spread_gather_kernel(View<R> v) {
         for (int iz = 0; iz < cnt[2][l2]; ++iz)
             for (int iy = 0; iy < cnt[1][l1]; ++iy)
                 for (int ix = 0; ix < cnt[0][l0]; ++ix) {
-                    const int kk = nbin[9 * ent_slot[2][l2][iz] + 3 * ent_slot[1][l1][iy] + ent_slot[0][l0][ix]];
+                    const int kk = nbin[16 * ent_slot[2][l2][iz] + 4 * ent_slot[1][l1][iy] + ent_slot[0][l0][ix]];
                     if (kk < 0) continue;
                     const R *tt = v.tiles + (size_t)kk * 3 * TP_N;
                     const int ti = tile_index(ent_pos[0][l0][ix], ent_pos[1][l1][iy], ent_pos[2][l2][iz]);
@@ -918,7 +921,7 @@ __global__ void __launch_bounds__(256) spread_gather_kernel(View<R> v) {
 }
 
 // Phase 2 with at least three blocks along every axis (neighbour blocks
-// distinct): along an axis the lower neighbour's tile covers this block's
+// distinct) and whole blocks along the periodic ones: along an axis the lower neighbour's tile covers this block's
 // local coordinates 0, 1 (tile positions 9, 10), the block's own tile all
 // eight (positions 1..8) and the upper neighbour's coordinate 7 (position
 // 0).  Each thread owns two nodes and adds, slot by slot in a fixed order,
@@ -1670,7 +1673,11 @@ template <typename R>
 void launch_spread(const View<R> &v, cudaStream_t st) {
     if constexpr (std::is_same<R, float>::value) launch_next(spread_tile_f32_kernel, v.nbins, SP_CHUNK, 0, st, v);
     else launch_next(spread_tile_kernel, 3 * v.nbins, SP64_THREADS, 0, st, v);
-    if (v.nb[0] >= 3 && v.nb[1] >= 3 && v.nb[2] >= 3) launch_next(spread_gather3_kernel<R>, v.nbins, 256, 0, st, v);
+    // (across a periodic edge the tiles' positions are those of whole blocks only)
+    const int dims[3] = {v.nx, v.ny, v.nz};
+    bool regular = true;
+    for (int d = 0; d < 3; ++d) regular &= v.nb[d] >= 3 && (!v.per[d] || dims[d] % BLK == 0);
+    if (regular) launch_next(spread_gather3_kernel<R>, v.nbins, 256, 0, st, v);
     else launch_next(spread_gather_kernel<R>, v.nbins, 256, 0, st, v);
 }
 
