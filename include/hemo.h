@@ -87,10 +87,11 @@ typedef struct {
  * one-node x-shift applied in shared memory) instead of every node through
  * the per-node kernel; the rows next to walls stay per node.  It applies to
  * 16-bit storage with x periodic and rows of at most 1024 nodes whose bytes
- * are a multiple of 16, and is used by default where rows hold at least 512
- * nodes (where it is the faster of the two).  HEMO_OPT_STAGED_COLLISION:
- * also for shorter rows; HEMO_OPT_UNSTAGED_COLLISION: never (it wins over
- * the former).  The results are the same bits in every case. */
+ * are a multiple of 16, and is used by default where it is the faster of the
+ * two: rows of at least 512 nodes, or of at least 64 in large lattices (13
+ * tiles of up to 1024 nodes per multiprocessor) unless one of the two options
+ * below asks for an unstaged kernel.  HEMO_OPT_STAGED_COLLISION: for all
+ * others too; HEMO_OPT_UNSTAGED_COLLISION: never (it wins over the former).  The results are the same bits in every case. */
 enum { HEMO_OPT_STAGED_COLLISION = 1u, HEMO_OPT_UNSTAGED_COLLISION = 64u };
 
 /* 16-bit storage with nx even computes the post-streaming velocity two

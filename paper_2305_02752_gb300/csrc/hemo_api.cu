@@ -324,7 +324,8 @@ View<R> make_view(hemo_sim *s) {
     v.rref = s->rref;
     // 16-bit storage, nx even: the velocity pass two nodes per thread (the
     // faster form, measured); the collision two nodes per thread only on
-    // request (the per-node kernel is faster on odd steps and as fast on even)
+    // request (the per-node kernel is faster on odd steps, 207 against 247 us on
+    // the 128 x 128 x 512 vessel, and as fast on even, 178 and 180)
     v.node_pairs = 0;
     if (tsize(s) == 2 && (s->nx % 2) == 0 && !(s->options & HEMO_OPT_NODE_COLLISION))
         v.node_pairs = PAIR_MOMENTS | ((s->options & HEMO_OPT_PAIR_COLLISION) ? PAIR_COLLIDE : 0);
@@ -1118,19 +1119,25 @@ int hemo_velocity_set(int32_t *c, double *w) {
 // needs 16-byte aligned rows (bulk copies), rows of at most 1024 nodes (a
 // stage's range) and at least two stages of the ring in shared memory (one
 // CTA per SM takes up to four), and is for 2-byte storage only.  By default
-// it is used for rows of at least 512 nodes (measured: on the 1000-node
-// rows of the pipe it takes 13 % less time than the per-node kernel, on
-// 128-node rows about as long); on request (HEMO_OPT_STAGED_COLLISION) for
-// shorter rows too; never with HEMO_OPT_UNSTAGED_COLLISION.
+// it is used for rows of at least 512 nodes (pipe: 523 and 568 us against 754
+// and 860 per node), and for rows of at least 64 where the tiles are at least
+// 13 per SM, so that the ring's start and end are small against the rest: 128 x
+// 128 x 512 channel 141 and 153 us against 171 and 198 per node, 128^3 47.4 and
+// 51.5 against 47.8 and 54.9, 64 x 128 x 256 46.8 and 53.0 against 49.5 and 54.9;
+// below, 192 x 96 x 96 (12 per SM) 42.5 and 46.6 against 40.8 and 48.6, 128 x 64
+// x 64 20.2 and 21.7 against 18.4 and 20.4, 48 x 160 x 160 33.1 and 37.0 against
+// 28.2 and 33.5.  On request (HEMO_OPT_STAGED_COLLISION) for the others too;
+// never with HEMO_OPT_UNSTAGED_COLLISION.
 constexpr size_t TILE_RING_BYTES = 227 * 1024;  // the largest dynamic shared memory of a CTA
 constexpr int TILE_STAGE_NODES = 1024;          // as the kernel's stage layout
-constexpr int TILE_DEFAULT_MIN_NX = 512;
+constexpr int TILE_DEFAULT_MIN_NX = 512, TILE_MIN_NX = 64, TILE_MIN_PER_SM = 13;
 
 int plan_rows(hemo_sim *s, const uint8_t *mask) {
     const int nx = s->nx, ny = s->ny, nz = s->nz;
     const size_t S = tsize(s), Rb = rsize(s);
     if (S != 2 || (s->options & HEMO_OPT_UNSTAGED_COLLISION) || !s->per[0]) return HEMO_OK;
-    if (!(s->options & HEMO_OPT_STAGED_COLLISION) && nx < TILE_DEFAULT_MIN_NX) return HEMO_OK;
+    const bool asked = (s->options & HEMO_OPT_STAGED_COLLISION) || nx >= TILE_DEFAULT_MIN_NX;
+    if (!asked && (nx < TILE_MIN_NX || (s->options & (HEMO_OPT_NODE_COLLISION | HEMO_OPT_PAIR_COLLISION)))) return HEMO_OK;
     if (((size_t)nx * S) % 16 || ((size_t)nx * Rb) % 16) return HEMO_OK;
     if (nx > TILE_STAGE_NODES) return HEMO_OK;
     // whole rows per tile, as many as a stage's ranges hold
@@ -1141,12 +1148,16 @@ int plan_rows(hemo_sim *s, const uint8_t *mask) {
     if (stages < 2) return HEMO_OK;
     std::vector<uint8_t> fluid((size_t)ny * nz, 1), any((size_t)ny * nz, mask ? 0 : 1);
     if (mask)
-        for (int r = 0; r < ny * nz; ++r)
+        for (int r = 0; r < ny * nz; ++r) {
+            uint8_t wall = 0, fl = 0;
+            const uint8_t *m = mask + (size_t)r * nx;
             for (int x = 0; x < nx; ++x) {
-                const bool fl = mask[(size_t)r * nx + x] == 0;
-                fluid[r] &= fl;
-                any[r] |= fl;
+                wall |= m[x];
+                fl |= m[x] == 0;
             }
+            fluid[r] = wall == 0;
+            any[r] = fl;
+        }
     auto row_fluid = [&](int y, int z) {
         if (y < 0 || y >= ny) {
             if (!s->per[1]) return false;
@@ -1178,8 +1189,8 @@ int plan_rows(hemo_sim *s, const uint8_t *mask) {
                 ++y;
             }
         }
-    if (tiles.empty()) return HEMO_OK;
     const int nsm = s->nsm;
+    if (tiles.empty() || (!asked && (long long)tiles.size() < (long long)TILE_MIN_PER_SM * nsm)) return HEMO_OK;
     const int smem = (int)(128 + stages * stage);
     HEMO_CU(set_tile_smem_limit(s->precision, (int)TILE_RING_BYTES));  // the cap of every plan
     s->rtiles = (int4 *)dalloc(s, sizeof(int4) * tiles.size());

@@ -233,6 +233,37 @@ __global__ void __launch_bounds__(NODE_BX * NODE_BY, sizeof(R) == 4 ? 4 : 1) col
     collide_at<T, R, PARITY, I, VISC>(v, x + v.nx * (y + v.ny * z), x, y, z);
 }
 
+// two 16-bit values in a word (low half: the first node) and their conversions,
+// with the reference of their slots (not added when has_ref is false, as in dec)
+template <typename T> struct Bits;
+template <> struct Bits<__half> {
+    static __device__ __forceinline__ __half of(unsigned short b) { return __ushort_as_half(b); }
+    static __device__ __forceinline__ unsigned short to(__half h) { return __half_as_ushort(h); }
+};
+template <> struct Bits<__nv_bfloat16> {
+    static __device__ __forceinline__ __nv_bfloat16 of(unsigned short b) { return __ushort_as_bfloat16(b); }
+    static __device__ __forceinline__ unsigned short to(__nv_bfloat16 h) { return __bfloat16_as_ushort(h); }
+};
+template <typename T> __device__ __forceinline__ F2 dec2(unsigned w, float ref, bool has_ref) {
+    F2 x;
+    if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+        x = pk(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+    } else {
+        x = pk(Store<T>::ld(Bits<T>::of((unsigned short)(w & 0xffffu))), Store<T>::ld(Bits<T>::of((unsigned short)(w >> 16))));
+    }
+    return has_ref ? x + pk(ref) : x;
+}
+template <typename T> __device__ __forceinline__ unsigned enc2(F2 q, float ref) {
+    const float2 x = unpk(q - pk(ref));
+    if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(x.x, x.y);
+        return *reinterpret_cast<const unsigned *>(&h);
+    } else {
+        const __half2 h = __floats2half2_rn(x.x, x.y);
+        return *reinterpret_cast<const unsigned *>(&h);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Staged collision for tiles of interior rows.
 //
@@ -254,8 +285,15 @@ __global__ void __launch_bounds__(NODE_BX * NODE_BY, sizeof(R) == 4 ? 4 : 1) col
 // they compute the fourth, without holding them in registers (what 2-byte
 // populations need to reach the HBM bandwidth).  A second kernel
 // (collide_erows_kernel) collides the rows next to walls node by node.
+//
+// The consumers' instruction issue bounds it, so a thread collides two
+// neighbouring nodes in packed arithmetic, whole words in and out where the
+// populations allow.  A pair needs up to 128 registers, which 16 warps have:
+// 15 consumer warps.  Pipe, 31.4 M nodes: 656 and 691 us (a node per thread, 18
+// consumer warps) -> 523 and 568 us even and odd (0.78 and 0.72 of the measured
+// copy bandwidth).
 constexpr int TILE_NODES = 1024;           // stride of a direction's range in a stage (nodes)
-constexpr int TILE_CONSUMER_WARPS = 18;
+constexpr int TILE_CONSUMER_WARPS = 15;
 constexpr int TILE_THREADS = 32 * (1 + TILE_CONSUMER_WARPS);  // warp 0: the producer
 constexpr int TILE_MAX_STAGES = 4;
 
@@ -416,12 +454,14 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) collide_tiles_kernel(View<R> 
         return;
     }
 
-    // Consumers: the nodes of a tile (row j, column x) spread over all
-    // consumer threads; this thread's first node (j0, x0) and the step to
-    // its next one (dj, dx), taken once
+    // Consumers: the pairs of nodes of a tile (row j, columns x and x + 1; rows have
+    // an even number of nodes) spread over all consumer threads, each tile
+    // starting where the one before ended, so that the warps get the same number;
+    // the step from one pair of a thread to its next one (dj, dx) is taken once
+    static_assert(sizeof(T) == 2, "two values per word");
     constexpr int CT = 32 * TILE_CONSUMER_WARPS;
-    const int ct = threadIdx.x - 32;
-    const int x0 = ct % nx, j0 = ct / nx, dx = CT % nx, dj = CT / nx;
+    const int ct = threadIdx.x - 32, np = nx / 2, dx = 2 * (CT % np), dj = CT / np;
+    int first = ct;  // this thread's first pair of the tile
     // the tile table entry is read one tile ahead, and the references of
     // the thread's first row before the wait for the stage's data, so that
     // their latency overlaps the wait
@@ -430,6 +470,14 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) collide_tiles_kernel(View<R> 
         const int s = it % S;
         const int4 tl_next = tile_of(it + 1) < ntiles ? v.rtiles[tile_of(it + 1)] : tl;
         const int y0 = tl.z, z0 = tl.w;  // a tile's rows lie in one z-plane
+        int x0 = first, j0 = 0;
+        while (x0 >= np) {
+            x0 -= np;
+            ++j0;
+        }
+        x0 *= 2;
+        first -= tl.y * np % CT;
+        if (first < 0) first += CT;
         // the node's row and its neighbours' references (direction i arrives
         // from the row shifted by -c_i and leaves to the row shifted by
         // +c_i), reloaded when the row changes
@@ -443,39 +491,58 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) collide_tiles_kernel(View<R> 
         T *P = (T *)(ring + s * stage_bytes);
         const R *Fs = (const R *)(ring + s * stage_bytes + Q * pop_bytes);
         for (int j = j0, x = x0; j < tl.y;) {
-            {
-                if (j != rj) {
-                    rj = j;
-                    rr = row_refs<T>(v, y0 + j, z0, PARITY == 1);
-                }
-                const int L = j * nx + x;
-                const int xm = (x == 0 ? nx : x) - 1, xp = (x == nx - 1 ? -1 : x) + 1;
-                // the value arriving from direction i sits in direction i's
-                // range at x - c_i on odd steps (x wrapped), at x on even
-                // steps; the range offsets i * TNM are constants
-                T *const b0 = P + L, *const bm = P + (j * nx + xm), *const bp = P + (j * nx + xp);
-                auto at = [&](int i) -> T & {
-                    return (PARITY == 0 ? b0 : (cx(i) > 0 ? bm : (cx(i) < 0 ? bp : b0)))[i * TNM];
-                };
-                R d[Q], p[Q];
+            if (j != rj) {
+                rj = j;
+                rr = row_refs<T>(v, y0 + j, z0, PARITY == 1);
+            }
+            // The values arriving from direction i at nodes x and x + 1 sit in
+            // direction i's range at x - c_i and x + 1 - c_i on odd steps (x
+            // wrapped), at x and x + 1 on even steps: a whole word where that
+            // starts at an even x, else two halves.  The range offsets i * TNM
+            // are constants.
+            const int L = j * nx + x;
+            T *const b0 = P + L, *const bm = P + (j * nx + (x == 0 ? nx : x) - 1),
+                     *const bp = P + (j * nx + (x + 2 == nx ? 0 : x + 2));
+            F2 d[Q], p[Q], rho, ux, uy, uz;
 #pragma unroll
-                for (int i = 0; i < Q; ++i)
-                    d[i] = dec<T, R>(at(i), PARITY ? ref_dir(i, rr.at(-cy(i), -cz(i))) : ref_dir(i, rr.own),
-                                     cx(i) != 0);
-                R rho, ux, uy, uz;
-                const R om = (v.ind && v.ind[(size_t)tl.x * nx + L]) ? v.omega_in : v.omega;
-                bgk_guo(d, Fs[L], Fs[TNM + L], Fs[2 * TNM + L], om, p, rho, ux, uy, uz);
-                if (v.rec) {
-                    const size_t n = (size_t)tl.x * nx + L;
-                    v.rec[n] = rho;
-                    v.rec[N + n] = ux;
-                    v.rec[2 * N + n] = uy;
-                    v.rec[3 * N + n] = uz;
-                }
-                // outgoing direction i takes the place of incoming opp(i)
+            for (int i = 0; i < Q; ++i) {
+                unsigned w;
+                if (PARITY == 0 || cx(i) == 0) w = *reinterpret_cast<const unsigned *>(b0 + i * TNM);
+                else if (cx(i) > 0) w = Bits<T>::to(bm[i * TNM]) | (unsigned)Bits<T>::to(b0[i * TNM]) << 16;
+                else w = Bits<T>::to(b0[i * TNM + 1]) | (unsigned)Bits<T>::to(bp[i * TNM]) << 16;
+                d[i] = dec2<T>(w, PARITY ? ref_dir(i, rr.at(-cy(i), -cz(i))) : ref_dir(i, rr.own), cx(i) != 0);
+            }
+            const size_t n = (size_t)tl.x * nx + L;
+            const float oma = (v.ind && v.ind[n]) ? v.omega_in : v.omega, omb = (v.ind && v.ind[n + 1]) ? v.omega_in : v.omega;
+            F2 F[3];
 #pragma unroll
-                for (int i = 0; i < Q; ++i)
-                    at(opp(i)) = enc<T, R>(p[i], PARITY ? ref_dir(i, rr.at(cy(i), cz(i))) : ref_dir(i, rr.own));
+            for (int k = 0; k < 3; ++k) {
+                const float2 f = *reinterpret_cast<const float2 *>(Fs + k * TNM + L);
+                F[k] = pk(f.x, f.y);
+            }
+            bgk_guo(d, F[0], F[1], F[2], pk(oma, omb), p, rho, ux, uy, uz);
+            if (v.rec) {
+                const float2 q[4] = {unpk(rho), unpk(ux), unpk(uy), unpk(uz)};
+                for (int k = 0; k < 4; ++k) {
+                    v.rec[k * N + n] = q[k].x;
+                    v.rec[k * N + n + 1] = q[k].y;
+                }
+            }
+            // outgoing direction opp(i) takes the place of incoming i
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const int o = opp(i);
+                const unsigned w = enc2<T>(p[o], PARITY ? ref_dir(o, rr.at(cy(o), cz(o))) : ref_dir(o, rr.own));
+                const T lo = Bits<T>::of((unsigned short)(w & 0xffffu)), hi = Bits<T>::of((unsigned short)(w >> 16));
+                if (PARITY == 0 || cx(i) == 0) {
+                    *reinterpret_cast<unsigned *>(b0 + i * TNM) = w;
+                } else if (cx(i) > 0) {
+                    bm[i * TNM] = lo;
+                    b0[i * TNM] = hi;
+                } else {
+                    b0[i * TNM + 1] = lo;
+                    bp[i * TNM] = hi;
+                }
             }
             x += dx;
             j += dj;
@@ -578,15 +645,6 @@ __global__ void __launch_bounds__(NODE_BX * MOM_BY) moments_kernel(View<R> v) {
 // (collide_at).  The arithmetic per node is the per-node kernel's, so the
 // results are the same bits.
 // ---------------------------------------------------------------------------
-template <typename T> struct Bits;
-template <> struct Bits<__half> {
-    static __device__ __forceinline__ __half of(unsigned short b) { return __ushort_as_half(b); }
-    static __device__ __forceinline__ unsigned short to(__half h) { return __half_as_ushort(h); }
-};
-template <> struct Bits<__nv_bfloat16> {
-    static __device__ __forceinline__ __nv_bfloat16 of(unsigned short b) { return __ushort_as_bfloat16(b); }
-    static __device__ __forceinline__ unsigned short to(__nv_bfloat16 h) { return __bfloat16_as_ushort(h); }
-};
 // the low / high 16-bit value of a pair word, decoded with reference ref
 // (not added when has_ref is false, as in dec)
 template <typename T> __device__ __forceinline__ float dec_lo(unsigned w, float ref, bool has_ref) {
@@ -596,9 +654,6 @@ template <typename T> __device__ __forceinline__ float dec_lo(unsigned w, float 
 template <typename T> __device__ __forceinline__ float dec_hi(unsigned w, float ref, bool has_ref) {
     const float x = Store<T>::ld(Bits<T>::of((unsigned short)(w >> 16)));
     return has_ref ? x + ref : x;
-}
-template <typename T> __device__ __forceinline__ unsigned enc16(float q, float ref) {
-    return Bits<T>::to(Store<T>::st(q - ref));
 }
 template <typename T> __device__ __forceinline__ unsigned ld_pair(const T *p) { return *reinterpret_cast<const unsigned *>(p); }
 template <typename T> __device__ __forceinline__ unsigned ld_one(const T *p) { return Bits<T>::to(*p); }
@@ -662,33 +717,25 @@ __global__ void __launch_bounds__(NODE_BX * NODE_BY) collide_pair_kernel(View<fl
     const size_t N = (size_t)v.N;
     const float2 F0 = act ? *reinterpret_cast<const float2 *>(v.F + n0) : make_float2(0.f, 0.f);
     const float2 F1 = act ? *reinterpret_cast<const float2 *>(v.F + N + n0) : make_float2(0.f, 0.f);
-    const float2 F2 = act ? *reinterpret_cast<const float2 *>(v.F + 2 * N + n0) : make_float2(0.f, 0.f);
+    const float2 F2_ = act ? *reinterpret_cast<const float2 *>(v.F + 2 * N + n0) : make_float2(0.f, 0.f);
     // reference of direction i as read and as written (the slots' rows)
     auto ref_rd = [&](int i) { return PARITY == 0 ? ref_dir(i, rr.own) : ref_dir(i, rr.at(-cy(i), -cz(i))); };
     auto ref_wr = [&](int i) { return PARITY == 0 ? ref_dir(i, rr.own) : ref_dir(i, rr.at(cy(i), cz(i))); };
+    {
+        F2 d[Q], p[Q], rho, ux, uy, uz;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {  // node x0 (low halves), then x0 + 1 (high halves)
-        const int n = n0 + h;
-        float d[Q], p[Q];
-#pragma unroll
-        for (int i = 0; i < Q; ++i)
-            d[i] = h ? dec_hi<T>(w[i], ref_rd(i), cx(i) != 0) : dec_lo<T>(w[i], ref_rd(i), cx(i) != 0);
-        const float om = (VISC && act && v.ind && v.ind[n]) ? v.omega_in : v.omega;
-        float rho, ux, uy, uz;
-        bgk_guo<float>(d, h ? F0.y : F0.x, h ? F1.y : F1.x, h ? F2.y : F2.x, om, p, rho, ux, uy, uz);
+        for (int i = 0; i < Q; ++i) d[i] = dec2<T>(w[i], ref_rd(i), cx(i) != 0);
+        const float om0 = (VISC && act && v.ind && v.ind[n0]) ? v.omega_in : v.omega;
+        const float om1 = (VISC && act && v.ind && v.ind[n0 + 1]) ? v.omega_in : v.omega;
+        bgk_guo(d, pk(F0.x, F0.y), pk(F1.x, F1.y), pk(F2_.x, F2_.y), pk(om0, om1), p, rho, ux, uy, uz);
         if (v.rec && act) {
-            v.rec[n] = rho;
-            v.rec[N + n] = ux;
-            v.rec[2 * N + n] = uy;
-            v.rec[3 * N + n] = uz;
+            *reinterpret_cast<float2 *>(v.rec + n0) = unpk(rho);
+            *reinterpret_cast<float2 *>(v.rec + N + n0) = unpk(ux);
+            *reinterpret_cast<float2 *>(v.rec + 2 * N + n0) = unpk(uy);
+            *reinterpret_cast<float2 *>(v.rec + 3 * N + n0) = unpk(uz);
         }
-        // the outputs replace this node's half of the words (the other
-        // node's inputs stay in the other half)
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const unsigned e = enc16<T>(p[i], ref_wr(i));
-            w[i] = h ? ((w[i] & 0xffffu) | (e << 16)) : ((w[i] & 0xffff0000u) | e);
-        }
+        for (int i = 0; i < Q; ++i) w[i] = enc2<T>(p[i], ref_wr(i));
     }
     T *f = (T *)v.f;
     const I NI = (I)N;

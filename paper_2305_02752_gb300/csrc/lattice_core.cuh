@@ -176,6 +176,109 @@ __device__ __forceinline__ void bgk_guo(const double (&d)[Q], double Fx, double 
     p[0] = om1 * d[0] + (om * drho - 12.0 * A - 18.0 * tr);  // - 2 times the even parts of the nine pairs
 }
 
+// Two floats in a 64-bit register: one instruction for both
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 pk(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ F2 pk(float a) { return pk(a, a); }
+__device__ __forceinline__ float2 unpk(F2 p) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(p.v));
+    return r;
+}
+__device__ __forceinline__ F2 operator+(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) {
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 operator*(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+
+// bgk_guo<float> of two nodes at once, for 16-bit storage, whose kernels are
+// bound by instruction issue.  The same bits as two calls of it: every product
+// that the compiler fuses with an addition there is fused here.
+__device__ __forceinline__ void bgk_guo(const F2 (&d)[Q], F2 Fx, F2 Fy, F2 Fz, F2 om, F2 (&p)[Q], F2 &rho, F2 &ux,
+                                        F2 &uy, F2 &uz) {
+    F2 drho = d[0] + d[1], m[3];
+#pragma unroll
+    for (int i = 2; i < Q; ++i) drho = drho + d[i];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        m[k] = d[2 * k + 1] - d[2 * k + 2];
+#pragma unroll
+        for (int i = 7; i < Q; ++i) {
+            const int c = k == 0 ? cx(i) : (k == 1 ? cy(i) : cz(i));
+            if (c) m[k] = c > 0 ? m[k] + d[i] : m[k] - d[i];
+        }
+    }
+    const F2 half = pk(0.5f), one = pk(1.f), w1 = pk((float)(1.0 / 18.0));
+    rho = one + drho;
+    const float2 r = unpk(rho);
+    const F2 inv = pk(recip(r.x), recip(r.y));
+    ux = fma2(half, Fx, m[0]) * inv;
+    uy = fma2(half, Fy, m[1]) * inv;
+    uz = fma2(half, Fz, m[2]) * inv;
+    const F2 uu = fma2(uz, uz, fma2(ux, ux, uy * uy));
+    const F2 uF = fma2(uz, Fz, fma2(ux, Fx, uy * Fy));
+    const F2 om1 = one - om, src = fma2(pk(-0.5f), om, one);
+    const F2 ow = om * w1, sw = src * w1, H = pk(3.f) * sw, nH = pk(-3.f) * sw, C = pk(9.f) * sw;
+    const F2 in = fma2(pk(-1.5f) * rho, uu, drho);
+    const F2 A = fma2(ow, in, nH * uF);
+    const F2 B = pk(4.5f) * ow * rho, G = pk(3.f) * ow * rho;
+    F2 sx, sy, sz, se, od[6];
+#pragma unroll
+    for (int a = 7; a < Q; a += 2) {  // diagonal pairs (1, sg) in a plane
+        const bool up = (cx(a) ? cy(a) + cz(a) : cz(a)) > 0;
+        const F2 u0 = cx(a) ? ux : uy, u1 = cz(a) ? uz : uy, F0 = cx(a) ? Fx : Fy, F1 = cz(a) ? Fz : Fy;
+        const F2 cu = up ? u0 + u1 : u0 - u1, cF = up ? F0 + F1 : F0 - F1;
+        const F2 even = half * fma2(cu, fma2(B, cu, C * cF), A);
+        const F2 odd = half * fma2(G, cu, H * cF);
+        p[a] = fma2(om1, d[a], even);
+        p[a + 1] = fma2(om1, d[a + 1], even);
+        od[(a - 7) / 2] = odd;
+        se = a == 7 ? even : se + even;
+        // (7, 9: the xy plane; 11, 13: xz; 15, 17: yz)
+        if (cx(a)) sx = a == 7 ? odd : sx + odd;
+        if (cy(a)) sy = a == 7 ? odd : (cy(a) > 0 ? sy + odd : sy - odd);
+        if (cz(a)) sz = a == 11 ? odd : (cz(a) > 0 ? sz + odd : sz - odd);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int a = 1 + 2 * k;
+        const F2 cu = k == 0 ? ux : (k == 1 ? uy : uz), cF = k == 0 ? Fx : (k == 1 ? Fy : Fz);
+        const F2 sk = k == 0 ? sx : (k == 1 ? sy : sz);
+        const F2 even = fma2(cu, fma2(B, cu, C * cF), A);
+        const F2 odd = half * fma2(om, m[k], cF) - sk;
+        se = se + even;
+        p[a] = fma2(om1, d[a], even) + odd;
+        p[a + 1] = fma2(om1, d[a + 1], even) - odd;
+    }
+    p[0] = fma2(om1, d[0], fma2(om, drho, pk(-2.f) * se));
+#pragma unroll
+    for (int a = 7; a < Q; a += 2) {
+        p[a] = p[a] + od[(a - 7) / 2];
+        p[a + 1] = p[a + 1] - od[(a - 7) / 2];
+    }
+}
+
 // storage type by precision: FP64 arithmetic only with FP64 storage
 #define HEMO_DISPATCH_T(prec, R, CALL)                           \
     do {                                                         \
