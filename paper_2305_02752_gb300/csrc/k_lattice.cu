@@ -290,7 +290,7 @@ template <typename T> __device__ __forceinline__ unsigned enc2(F2 q, float ref) 
 // neighbouring nodes in packed arithmetic, whole words in and out where the
 // populations allow.  A pair needs up to 128 registers, which 16 warps have:
 // 15 consumer warps.  Pipe, 31.4 M nodes: 656 and 691 us (a node per thread, 18
-// consumer warps) -> 523 and 568 us even and odd (0.78 and 0.72 of the measured
+// consumer warps) -> 520 and 564 us even and odd (0.75 and 0.69 of the measured
 // copy bandwidth).
 constexpr int TILE_NODES = 1024;           // stride of a direction's range in a stage (nodes)
 constexpr int TILE_CONSUMER_WARPS = 15;

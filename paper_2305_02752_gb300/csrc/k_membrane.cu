@@ -1,4 +1,4 @@
-// Membrane mechanics, one CTA per cell (Sec. 2.3: F_total = F_link + F_bend
+// Membrane mechanics, one CTA per cell or, with few cells, a cluster (Sec. 2.3: F_total = F_link + F_bend
 // + F_area + F_volume; vertices are Lagrangian points of a triangulated
 // membrane).
 //
