@@ -8,9 +8,10 @@
 // the triangles in FP64, and accumulates the four force terms per vertex in
 // shared memory before one coalesced write.  The edge and triangle tables
 // arrive in a processing order sorted on the host by smallest vertex id, so
-// that the lanes of a warp load nearby shared-memory records; the FP64
-// adjoint, which scatters with shared-memory atomics, walks them with a
-// coprime stride instead (lanes on far-apart mesh parts).  Energies (forms documented in
+// that the lanes of a warp load nearby shared-memory records; the FP32 adjoint of
+// meshes too large for the gather, which scatters with shared-memory atomics,
+// walks them with a coprime stride instead (lanes on far-apart mesh parts).
+// Energies (forms documented in
 // hemo.h):
 //   link   K L0 [eps^2/2 - 1/2 ln(1 - eps^2/m^2)],   eps = (L - L0)/L0
 //   bend   1/2 kb (theta - theta0)^2, theta = signed angle between the
@@ -791,7 +792,8 @@ template <typename R> __device__ __forceinline__ void add_into(R *f, R s, V3<R> 
     atomicAdd(f + 2, s * a.z);
 }
 
-// Adjoint of the membrane forces of one cell (`slices` CTAs per cell: each
+// Adjoint of the membrane forces of one cell, FP32, for meshes whose records do
+// not fit the gather below (`slices` CTAs per cell: each
 // computes the cell's triangle records, area and volume, then its share of
 // the edge and triangle terms, and adds its part of the product to lamX,
 // atomically when a cell has several CTAs), at the
