@@ -757,16 +757,31 @@ double dihedral(D3 p0, D3 p1, D3 pa, D3 pb) {
     return std::atan2(dt3(crs(n1, n2), e) / std::sqrt(dt3(e, e)), dt3(n1, n2));
 }
 
-// whether a kernel on the current device can write elements of `size` bytes at p:
-// device memory of that device, aligned
-bool direct_out(const void *p, size_t size) {
+// whether a kernel on the current device can write `bytes` bytes, elements of
+// `size` bytes, at p: device memory of that device, aligned, and all of it in
+// one allocation.  What does not lie in one goes through a copy, which the
+// driver checks: a destination shorter than its field is an error, not a write
+// past its end.
+bool direct_out(const void *p, size_t size, size_t bytes) {
+    using RangeFn = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const RangeFn range = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            fn = nullptr;
+        return reinterpret_cast<RangeFn>(fn);
+    }();
     cudaPointerAttributes at;
     int dev = -1;
     if ((uintptr_t)p % size || cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return at.type == cudaMemoryTypeDevice && at.device == dev;
+    if (at.type != cudaMemoryTypeDevice || at.device != dev || !range) return false;
+    CUdeviceptr base = 0;
+    size_t len = 0;
+    return range(&base, &len, (CUdeviceptr)(uintptr_t)p) == CUDA_SUCCESS && (uintptr_t)p - (uintptr_t)base + bytes <= len;
 }
 
 int copy_out(hemo_sim *s, void *dst, const void *src, size_t bytes) {
@@ -1611,12 +1626,12 @@ int hemo_get_fields(hemo_sim *s, unsigned what, void *rho, void *u, double *vert
     const bool want_x = (what & HEMO_VERTS) && verts && s->nv, want_f = (what & HEMO_FORCES) && forces && s->nv;
     const bool want_c = (what & HEMO_CELLSTATS) && cellstats && s->ncell;
     // the kernels write fields straight into the caller's device memory; host
-    // memory (and pointers that are not aligned to an element) goes through the
-    // staging buffer and a copy (1000 x 208 x 208 pipe, all fields: 2.5 GB of
-    // traffic less)
-    const bool d_rho = want_rho && direct_out(rho, rs), d_u = want_u && direct_out(u, rs),
-               d_x = want_x && direct_out(verts, sizeof(double)), d_f = want_f && direct_out(forces, sizeof(double)),
-               d_c = want_c && direct_out(cellstats, sizeof(double));
+    // memory (and pointers that are not aligned to an element, or whose allocation
+    // ends before the field does) goes through the staging buffer and a copy
+    // (1000 x 208 x 208 pipe, all fields: 2.5 GB of traffic less)
+    const bool d_rho = want_rho && direct_out(rho, rs, rs * N), d_u = want_u && direct_out(u, rs, rs * 3 * N),
+               d_x = want_x && direct_out(verts, sizeof(double), vb), d_f = want_f && direct_out(forces, sizeof(double), vb),
+               d_c = want_c && direct_out(cellstats, sizeof(double), cb);
     const size_t need = std::max<size_t>({want_rho && !d_rho ? rs * N : 0, want_u && !d_u ? rs * 3 * N : 0,
                                           (want_x && !d_x) || (want_f && !d_f) ? 2 * vb : 0, want_c && !d_c ? cb : 0});
     if (need && (rc = ensure_staging(s, need))) return rc;
