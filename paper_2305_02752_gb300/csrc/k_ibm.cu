@@ -768,14 +768,12 @@ __global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(SP64_THREADS) spread
     bin_origin(v, k, org);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int h = lane >> 4, b = lane & 3, c = (lane >> 2) & 3;
-    {  // the component's scale for the whole bin: largest |F|, compared as integers (as fmax, ignoring NaN)
-        constexpr unsigned long long INF = 0x7ff0000000000000ull;
+    {  // the component's scale for the whole bin: largest |F|, compared as integers (NaN above all)
         unsigned long long m = 0;
         for (int j = s + threadIdx.x; j < e; j += blockDim.x) {
             const int i = v.perm[j];
             if (!index_ok(i >= 0 && i < v.nv, v.status)) continue;
-            const unsigned long long f = (unsigned long long)__double_as_longlong(fabs(v.Fv[3 * (size_t)i + d]));
-            if (f <= INF && f > m) m = f;
+            m = max(m, (unsigned long long)__double_as_longlong(fabs(v.Fv[3 * (size_t)i + d])));
         }
         const unsigned mh = (unsigned)(m >> 32), wh = __reduce_max_sync(0xffffffffu, mh);
         const unsigned wl = __reduce_max_sync(0xffffffffu, mh == wh ? (unsigned)m : 0u);
@@ -812,7 +810,7 @@ __global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(SP64_THREADS) spread
                         for (int a = 0; a < 4; ++a) o[a] = w[a];
                     }
                 }
-                sF[j] = v.Fv[3 * (size_t)i + d] * (0.5 * scale);
+                sF[j] = scale > 0.0 ? v.Fv[3 * (size_t)i + d] * (0.5 * scale) : 0.0;
                 for (int a = 0; a < 3; ++a) {
                     const int q = v.anc_i[3 * (size_t)i + a] - org[a];
                     ok &= q >= 0 && q < BLK;
