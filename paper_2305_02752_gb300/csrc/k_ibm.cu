@@ -601,7 +601,9 @@ __global__ void __launch_bounds__(SP_CHUNK, 6) spread_tile_f32_kernel(View<float
     bin_origin(v, k, org);
     // chunks of equal size
     const int nch = (n + SP_CHUNK - 1) / SP_CHUNK, csz = (n + nch - 1) / nch;
-    // a vertex's record; row -1 outside the bin (domain status already raised)
+    // a vertex's record; row -1 outside the bin (domain status already raised) and
+    // for a position that is not a number, whose contributions convert to zero
+    // but would be the largest integer on the denormal grid
     auto load = [&](int j, float t[3], float F[3]) -> int {
         const int i = v.perm[j];
         if (!index_ok(i >= 0 && i < v.nv, v.status)) return -1;
@@ -613,6 +615,7 @@ __global__ void __launch_bounds__(SP_CHUNK, 6) spread_tile_f32_kernel(View<float
             ok &= b >= 0 && b < BLK;
             row += b * (d == 0 ? 1 : (d == 1 ? SP_Y : SP_Z));
             t[d] = v.anc_t[3 * (size_t)i + d];
+            ok &= t[d] == t[d];
             F[d] = v.Fv[3 * (size_t)i + d];
         }
         return ok ? row : -1;
@@ -813,7 +816,9 @@ __global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(SP64_THREADS) spread
                 sF[j] = scale > 0.0 ? v.Fv[3 * (size_t)i + d] * (0.5 * scale) : 0.0;
                 for (int a = 0; a < 3; ++a) {
                     const int q = v.anc_i[3 * (size_t)i + a] - org[a];
-                    ok &= q >= 0 && q < BLK;
+                    // (exponent bits all set: a position that is not a number adds nothing)
+                    const int th = __double2hiint(v.anc_t[3 * (size_t)i + a]);
+                    ok &= q >= 0 && q < BLK && (th & 0x7ff00000) != 0x7ff00000;
                     row += q * (a == 0 ? 1 : (a == 1 ? TS_Y : TS_Z));
                 }
             }
