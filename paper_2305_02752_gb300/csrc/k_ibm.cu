@@ -232,7 +232,7 @@ __global__ void scatter_kernel(const int *key, int *cursor, int *perm_raw, int n
 __global__ void __launch_bounds__(1024) scan_scatter_kernel(int *counts, int *start, int nbins, const int *key, int *perm,
                                                             int nv, unsigned *status) {
     wait_previous();
-    __shared__ int cur[SMALL_BINS];
+    __shared__ __align__(16) int cur[SMALL_BINS];
     __shared__ int wsum[32];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const bool vec = ((uintptr_t)counts & 15) == 0;
