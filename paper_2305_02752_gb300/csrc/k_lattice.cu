@@ -951,7 +951,7 @@ __global__ void u_out_kernel(View<R> v, R *out) {
 constexpr int UOUT_NT = 256;
 __global__ void __launch_bounds__(UOUT_NT) u_out_vec_kernel(View<float> v, float *out) {
     wait_previous();
-    __shared__ float s[12 * UOUT_NT];
+    __shared__ __align__(16) float s[12 * UOUT_NT];
     const size_t N = (size_t)v.N, n0 = (size_t)blockIdx.x * 4 * UOUT_NT;
     const size_t n = n0 + 4 * threadIdx.x;
     if (n < N) {

@@ -41,7 +41,7 @@ def test_finds_a_narrow_array():
     assert _narrow(src) == [('s', 16, 0)]
 
 
-@pytest.mark.parametrize('source', ['k_ibm.cu'])
+@pytest.mark.parametrize('source', sorted(f for f in os.listdir(CSRC) if f.endswith('.cu')))
 def test_wide_shared_arrays_are_aligned(source):
     with open(os.path.join(CSRC, source)) as f:
         assert _narrow(f.read()) == []
