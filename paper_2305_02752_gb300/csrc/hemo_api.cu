@@ -956,12 +956,14 @@ int backward_impl(hemo_sim *s, const double *dL_dverts, double *grad, int ngrad)
         !need(b.fin_f, b.sz_fin_f, rs * Q * N) || !need(b.fin_u, b.sz_fin_u, rs * 3 * N) ||
         !need(b.fin_ctr, b.sz_fin_ctr, sizeof(double) * 3 * nc1) || !need(b.fin_off, b.sz_fin_off, rs * 3 * nv1))
         return fail(HEMO_ERR_OOM, "allocation of adjoint buffers failed");
+    const size_t batch = (size_t)adjoint_batch(s->ncell, s->max_nt);
+    const size_t ft_bytes = rs * 3 * batch * (size_t)std::max(s->max_nv, 1);
     if (std::is_same<R, double>::value &&
-        (!need(b.ft, b.sz_ft, rs * 3 * nv1) || !need(b.tri_rec, b.sz_tri_rec, rs * 8 * nc1 * (size_t)std::max(s->max_nt, 1)) ||
-         !need(b.tri_part, b.sz_tri_part, sizeof(double) * 4 * nc1 * (size_t)adjoint_chunks(std::max(s->max_nt, 1)))))
+        (!need(b.ft, b.sz_ft, ft_bytes) || !need(b.tri_rec, b.sz_tri_rec, rs * 8 * batch * (size_t)std::max(s->max_nt, 1)) ||
+         !need(b.tri_part, b.sz_tri_part, sizeof(double) * 4 * batch * (size_t)adjoint_chunks(std::max(s->max_nt, 1)))))
         return fail(HEMO_ERR_OOM, "allocation of adjoint buffers failed");
     if (moved) clear_segment_graphs(s);  // captured pointers are stale
-    if (b.ft) HEMO_CU(cudaMemsetAsync(b.ft, 0, rs * 3 * nv1, st));
+    if (b.ft) HEMO_CU(cudaMemsetAsync(b.ft, 0, ft_bytes, st));
     View<R> v = make_view<R>(s);
     // final state, restored at the end
     launch_copy_natural<R>(v, s->precision, (int)(t_end & 1), (R *)b.fin_f, st);

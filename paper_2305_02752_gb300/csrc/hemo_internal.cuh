@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "../../include/hemo.h"
 
 namespace hemo {
@@ -243,9 +245,10 @@ template <typename R> struct AdjView {
     R *lamX;          // nv*3 adjoint of the vertex positions
     R *lamFv;         // nv*3 adjoint of the membrane forces
     double *grad;     // gradient accumulators (device)
-    R *tri_rec;       // FP64: ncell*max_nt*8 triangle records of the membrane adjoint
-    R *ft;            // FP64: nv*3 membrane terms of lamX (zero between the kernels)
-    double *tri_part; // FP64: ncell*adjoint_chunks(max_nt)*4 parts of A, dA, V, dV
+    // FP64 membrane adjoint, of adjoint_batch() cells at a time
+    R *tri_rec;       // batch*max_nt*8 triangle records
+    R *ft;            // batch*max_nv*3 membrane terms of lamX (zero between the kernels)
+    double *tri_part; // batch*adjoint_chunks(max_nt)*4 parts of A, dA, V, dV
     int ntypes;
 };
 
@@ -306,6 +309,10 @@ template <typename R> void launch_adj_collide(const View<R> &v, const AdjView<R>
 template <typename R> void launch_cell_adjoint(const View<R> &v, const AdjView<R> &a, cudaStream_t st);
 template <typename R> cudaError_t set_cell_adjoint_smem_limit(size_t bytes);
 inline int adjoint_chunks(int items) { return (items + 63) / 64; }  // CTAs of 64 items (FP64)
+// cells whose triangle records (64 bytes each) fill 64 MB: 819 red cells, 16,000 CTAs
+inline int adjoint_batch(int ncell, int max_nt) {
+    return std::max(1, std::min(ncell, (64 << 20) / (64 * std::max(max_nt, 1))));
+}
 template <typename R> size_t cell_adjoint_smem_bytes(int max_nv, int max_nt) { return (9 * (size_t)max_nv + 8 * (size_t)max_nt) * sizeof(R); }
 // FP32 gather form of the membrane adjoint: positions, direction, triangle
 // and edge records with their derivatives, 16 bytes each; used while it fits

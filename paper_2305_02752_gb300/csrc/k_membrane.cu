@@ -925,17 +925,19 @@ __global__ void __launch_bounds__(NT, CellMinBlocks<R, NT>::B) cell_adjoint_kern
 // dn, 1/|n|^2 and its derivative) and each CTA's part of A, dA, V, dV into
 // global memory; then the edge and triangle terms, summed per vertex and into
 // the gradients with atomics.  (A third adds the sums to lamX: the terms are
-// small against it, and added one by one they lost seven digits.)  One CTA per cell (or per slice of one, each with
-// all records of the cell) kept an SM busy with the records for 96 us.
-// 32^3 box, one cell: 109 -> 8.4 + 17.7 + 2.3 us.
+// small against it, and added one by one they lost seven digits.)  One CTA per
+// cell (or per slice of one, each with all records of the cell) kept an SM busy
+// with the records for 96 us.  32^3 box, one cell: 109 -> 8.4 + 17.7 + 2.3 us.
+// Many cells go through the three kernels adjoint_batch() at a time, from cell
+// c0: their records would take 1.6 GB for the 19,600 cells of the pipe.
 constexpr int ADJ_NT = 64;  // items per CTA
 __device__ __forceinline__ V3<Dual<double>> vertex_dual(const View<double> &v, const AdjView<double> &a, size_t i) {
     return dld3(v.off + 3 * i, a.lamFv + 3 * i);
 }
-__global__ void __launch_bounds__(ADJ_NT) adjoint_records_kernel(View<double> v, AdjView<double> a, int chunks) {
+__global__ void __launch_bounds__(ADJ_NT) adjoint_records_kernel(View<double> v, AdjView<double> a, int c0, int chunks) {
     wait_previous();
     using D = Dual<double>;
-    const int c = blockIdx.x / chunks, chunk = blockIdx.x % chunks;
+    const int lc = blockIdx.x / chunks, c = c0 + lc, chunk = blockIdx.x % chunks;
     const MeshDev<double> m = v.meshes[v.cell_type[c]];
     const size_t first = v.cell_first[c];
     __shared__ double scratch[4][32];
@@ -947,7 +949,7 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_records_kernel(View<double> v,
         const V3<D> n = cross(p1 - p0, p2 - p0);
         const D q = dot(n, n);
         const D iq = dconst(1.0) / q;
-        double *o = a.tri_rec + 8 * ((size_t)c * v.max_nt + t);
+        double *o = a.tri_rec + 8 * ((size_t)lc * v.max_nt + t);
         o[0] = n.x.v; o[1] = n.y.v; o[2] = n.z.v;
         o[3] = n.x.t; o[4] = n.y.t; o[5] = n.z.t;
         o[6] = iq.v; o[7] = iq.t;
@@ -959,20 +961,21 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_records_kernel(View<double> v,
     }
     double AV[4];
     block_total<double, 4>(av, AV, scratch);
-    if (threadIdx.x < 4) a.tri_part[4 * ((size_t)c * chunks + chunk) + threadIdx.x] = scratch[threadIdx.x][31];
+    if (threadIdx.x < 4) a.tri_part[4 * ((size_t)lc * chunks + chunk) + threadIdx.x] = scratch[threadIdx.x][31];
 }
 
-__global__ void __launch_bounds__(ADJ_NT) adjoint_terms_kernel(View<double> v, AdjView<double> a, int chunks, int echunks) {
+__global__ void __launch_bounds__(ADJ_NT) adjoint_terms_kernel(View<double> v, AdjView<double> a, int c0, int chunks, int echunks) {
     wait_previous();
     using D = Dual<double>;
     using R = double;
-    const int c = blockIdx.x / (chunks + echunks), chunk = blockIdx.x % (chunks + echunks);
+    const int lc = blockIdx.x / (chunks + echunks), c = c0 + lc, chunk = blockIdx.x % (chunks + echunks);
     const int type = v.cell_type[c];
     const MeshDev<R> m = v.meshes[type];
     const size_t first = v.cell_first[c];
-    const R *rec = a.tri_rec + 8 * (size_t)c * v.max_nt;
+    const R *rec = a.tri_rec + 8 * (size_t)lc * v.max_nt;
+    R *ft = a.ft + 3 * (first - (size_t)v.cell_first[c0]);
     __shared__ double scratch[2][32];
-    auto add = [&](int i, R s, V3<R> f) { add_into(a.ft + 3 * (first + i), s, f); };
+    auto add = [&](int i, R s, V3<R> f) { add_into(ft + 3 * i, s, f); };
     Acc<R> th[2];  // lamFv . unit-modulus forces: link and bend, or area and volume
     const bool edges = chunk < echunks;
     if (edges) {
@@ -1011,7 +1014,7 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_terms_kernel(View<double> v, A
         __shared__ R cuv[4];  // the area and volume strain factors and their derivatives
         if (threadIdx.x < 4) {
             R s = R(0);
-            for (int q = 0; q < chunks; ++q) s += a.tri_part[4 * ((size_t)c * chunks + q) + threadIdx.x];
+            for (int q = 0; q < chunks; ++q) s += a.tri_part[4 * ((size_t)lc * chunks + q) + threadIdx.x];
             if (threadIdx.x == 0) s -= m.A0;
             if (threadIdx.x == 2) s -= m.V0;
             cuv[threadIdx.x] = threadIdx.x < 2 ? s / (m.A0 * m.A0) : s / (m.V0 * m.V0);
@@ -1043,11 +1046,12 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_terms_kernel(View<double> v, A
     if (threadIdx.x < 2) atomicAdd(a.grad + 4 * type + (edges ? 0 : 2) + threadIdx.x, scratch[threadIdx.x][31]);
 }
 
-__global__ void __launch_bounds__(256) adjoint_add_kernel(AdjView<double> a, int n) {
+__global__ void __launch_bounds__(256) adjoint_add_kernel(View<double> v, AdjView<double> a, int c0, int cells) {
     wait_previous();
-    const int i = blockIdx.x * 256 + threadIdx.x;
-    if (i >= n) return;
-    a.lamX[i] += a.ft[i];
+    const size_t base = 3 * (size_t)v.cell_first[c0], end = 3 * (size_t)(c0 + cells < v.ncell ? v.cell_first[c0 + cells] : v.nv);
+    const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+    if (base + i >= end) return;
+    a.lamX[base + i] += a.ft[i];
     a.ft[i] = 0.0;
 }
 
@@ -1371,9 +1375,13 @@ void launch_cell_adjoint(const View<R> &v, const AdjView<R> &a, cudaStream_t st)
     }
     if constexpr (std::is_same<R, double>::value) {
         const int chunks = adjoint_chunks(v.max_nt), echunks = adjoint_chunks(v.max_ne);
-        launch_next(adjoint_records_kernel, v.ncell * chunks, ADJ_NT, 0, st, v, a, chunks);
-        launch_next(adjoint_terms_kernel, v.ncell * (chunks + echunks), ADJ_NT, 0, st, v, a, chunks, echunks);
-        launch_next(adjoint_add_kernel, (3 * v.nv + 255) / 256, 256, 0, st, a, 3 * v.nv);
+        const int batch = adjoint_batch(v.ncell, v.max_nt);
+        for (int c0 = 0; c0 < v.ncell; c0 += batch) {
+            const int n = std::min(batch, v.ncell - c0);
+            launch_next(adjoint_records_kernel, n * chunks, ADJ_NT, 0, st, v, a, c0, chunks);
+            launch_next(adjoint_terms_kernel, n * (chunks + echunks), ADJ_NT, 0, st, v, a, c0, chunks, echunks);
+            launch_next(adjoint_add_kernel, (unsigned)((3LL * n * v.max_nv + 255) / 256), 256, 0, st, v, a, c0, n);
+        }
     } else {  // meshes whose gather records do not fit
         const size_t smem = cell_adjoint_smem_bytes<R>(v.max_nv, v.max_nt);
         const int slices = std::max(1, std::min(32, v.nsm / v.ncell));
