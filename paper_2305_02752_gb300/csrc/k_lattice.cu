@@ -456,12 +456,13 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) collide_tiles_kernel(View<R> 
 
     // Consumers: the pairs of nodes of a tile (row j, columns x and x + 1; rows have
     // an even number of nodes) spread over all consumer threads, each tile
-    // starting where the one before ended, so that the warps get the same number;
-    // the step from one pair of a thread to its next one (dj, dx) is taken once
+    // starting where the one before ended (a thread's position is carried from
+    // tile to tile), so that the warps get the same number; the step from one pair
+    // of a thread to its next one (dj, dx) is taken once
     static_assert(sizeof(T) == 2, "two values per word");
     constexpr int CT = 32 * TILE_CONSUMER_WARPS;
     const int ct = threadIdx.x - 32, np = nx / 2, dx = 2 * (CT % np), dj = CT / np;
-    int first = ct;  // this thread's first pair of the tile
+    int x = 2 * (ct % np), j = ct / np;  // this thread's pair
     // the tile table entry is read one tile ahead, and the references of
     // the thread's first row before the wait for the stage's data, so that
     // their latency overlaps the wait
@@ -470,18 +471,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) collide_tiles_kernel(View<R> 
         const int s = it % S;
         const int4 tl_next = tile_of(it + 1) < ntiles ? v.rtiles[tile_of(it + 1)] : tl;
         const int y0 = tl.z, z0 = tl.w;  // a tile's rows lie in one z-plane
-        int x0 = first, j0 = 0;
-        while (x0 >= np) {
-            x0 -= np;
-            ++j0;
-        }
-        x0 *= 2;
-        first -= tl.y * np % CT;
-        if (first < 0) first += CT;
         // the node's row and its neighbours' references (direction i arrives
         // from the row shifted by -c_i and leaves to the row shifted by
         // +c_i), reloaded when the row changes
-        int rj = j0 < tl.y ? j0 : tl.y - 1;
+        int rj = j < tl.y ? j : tl.y - 1;
         RowRefs rr = row_refs<T>(v, y0 + rj, z0, PARITY == 1);
         const bool ok = mbar_wait(full + s, (unsigned)((it / S) & 1));
         if (!__all_sync(0xffffffffu, ok)) {  // the producer's copies did not land in time
@@ -490,7 +483,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) collide_tiles_kernel(View<R> 
         }
         T *P = (T *)(ring + s * stage_bytes);
         const R *Fs = (const R *)(ring + s * stage_bytes + Q * pop_bytes);
-        for (int j = j0, x = x0; j < tl.y;) {
+        while (j < tl.y) {
             if (j != rj) {
                 rj = j;
                 rr = row_refs<T>(v, y0 + j, z0, PARITY == 1);
@@ -551,6 +544,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) collide_tiles_kernel(View<R> 
                 ++j;
             }
         }
+        j -= tl.y;
         tl = tl_next;
         fence_async_smem();  // this thread's writes, before the producer's bulk stores read them
         __syncwarp();
