@@ -318,6 +318,11 @@ int hemo_get_sizes(const hemo_sim *sim, long long *n_nodes, long long *n_vertice
  * ints, caller-owned. */
 int hemo_get_lattice_plan(const hemo_sim *sim, int *plan);
 
+/* CTAs per cell of the membrane kernel: more than one (a cluster) where cells
+ * are few.  Set with the mesh tables, at the first step or read-out; 0 before.
+ * ctas: host, caller-owned. */
+int hemo_get_membrane_plan(const hemo_sim *sim, int *ctas);
+
 /* The library's D3Q19 velocity order: c (host, 19*3 int), w (host, 19). */
 int hemo_velocity_set(int32_t *c, double *w);
 

@@ -1614,6 +1614,12 @@ int hemo_get_lattice_plan(const hemo_sim *s, int *plan) {
     return HEMO_OK;
 }
 
+int hemo_get_membrane_plan(const hemo_sim *s, int *ctas) {
+    if (!s || !ctas) return fail(HEMO_ERR_ARG, "null pointer");
+    *ctas = s->finalized ? s->slices : 0;
+    return HEMO_OK;
+}
+
 int hemo_get_fields(hemo_sim *s, unsigned what, void *rho, void *u, double *verts, double *forces,
                     double *cellstats) {
     NvtxRange nvtx_("hemo_get_fields");

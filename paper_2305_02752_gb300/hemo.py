@@ -86,6 +86,7 @@ def lib():
         'hemo_get_fields': ([vp, C.c_uint, vp, vp, vp, vp, vp], i),
         'hemo_get_sizes': ([vp, C.POINTER(ll), C.POINTER(ll), C.POINTER(i), C.POINTER(i)], i),
         'hemo_get_lattice_plan': ([vp, vp], i),
+        'hemo_get_membrane_plan': ([vp, vp], i),
         'hemo_velocity_set': ([vp, vp], i),
         'hemo_get_populations': ([vp, vp], i),
         'hemo_get_links': ([vp, vp], i),
@@ -117,7 +118,7 @@ def exported_symbols():
     return ['hemo_create_lattice', 'hemo_set_velocity', 'hemo_add_cells', 'hemo_step', 'hemo_set_time_scales',
             'hemo_set_force_tolerance', 'hemo_get_force_evaluations',
             'hemo_set_viscosity_ratio', 'hemo_get_inside', 'hemo_set_lees_edwards', 'hemo_sync',
-            'hemo_get_fields', 'hemo_get_sizes', 'hemo_get_lattice_plan', 'hemo_velocity_set', 'hemo_get_populations',
+            'hemo_get_fields', 'hemo_get_sizes', 'hemo_get_lattice_plan', 'hemo_get_membrane_plan', 'hemo_velocity_set', 'hemo_get_populations',
             'hemo_get_links', 'hemo_get_edges', 'hemo_set_vertices', 'hemo_get_bins',
             'hemo_set_phase_timing', 'hemo_get_phase_times', 'hemo_bin_vertices_noalloc', 'hemo_state_bytes',
             'hemo_save_state', 'hemo_load_state', 'hemo_record',
@@ -336,6 +337,13 @@ class Simulation:
         plan = (C.c_int * 4)()
         check(lib().hemo_get_lattice_plan(self.handle, plan))
         return tuple(plan)
+
+    def membrane_plan(self):
+        """CTAs per cell of the membrane kernel (0 before the first step or
+        read-out)."""
+        n = C.c_int(0)
+        check(lib().hemo_get_membrane_plan(self.handle, C.byref(n)))
+        return n.value
 
     # -- read-out ----------------------------------------------------------
     def get_fields(self, what=HEMO_RHO | HEMO_U | HEMO_VERTS | HEMO_FORCES | HEMO_CELLSTATS, out=None):
