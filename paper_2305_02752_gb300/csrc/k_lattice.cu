@@ -290,8 +290,8 @@ template <typename T> __device__ __forceinline__ unsigned enc2(F2 q, float ref) 
 // neighbouring nodes in packed arithmetic, whole words in and out where the
 // populations allow.  A pair needs up to 128 registers, which 16 warps have:
 // 15 consumer warps.  Pipe, 31.4 M nodes: 656 and 691 us (a node per thread, 18
-// consumer warps) -> 520 and 564 us even and odd (0.75 and 0.69 of the measured
-// copy bandwidth).
+// consumer warps) -> 513 and 562 us even and odd (with the rows next to walls 0.75
+// and 0.68 of the measured copy bandwidth).
 constexpr int TILE_NODES = 1024;           // stride of a direction's range in a stage (nodes)
 constexpr int TILE_CONSUMER_WARPS = 15;
 constexpr int TILE_THREADS = 32 * (1 + TILE_CONSUMER_WARPS);  // warp 0: the producer
