@@ -91,7 +91,8 @@ typedef struct {
  * two: rows of at least 512 nodes, or of at least 64 in large lattices (13
  * tiles of up to 1024 nodes per multiprocessor) unless one of the two options
  * below asks for an unstaged kernel.  HEMO_OPT_STAGED_COLLISION: for all
- * others too; HEMO_OPT_UNSTAGED_COLLISION: never (it wins over the former).  The results are the same bits in every case. */
+ * others too; HEMO_OPT_UNSTAGED_COLLISION: never (it wins over the former).
+ * The results are the same bits in every case. */
 enum { HEMO_OPT_STAGED_COLLISION = 1u, HEMO_OPT_UNSTAGED_COLLISION = 64u };
 
 /* 16-bit storage with nx even computes the post-streaming velocity two

@@ -20,6 +20,7 @@ SOURCES = ['hemo_api.cu', 'k_lattice.cu', 'k_ibm.cu', 'k_membrane.cu', 'k_adjoin
 HEADERS = [os.path.join(CSRC, 'hemo_internal.cuh'), os.path.join(CSRC, 'lattice_core.cuh'),
            os.path.join(os.path.dirname(HERE), 'include', 'hemo.h')]
 ARCH = ['-gencode', 'arch=compute_103a,code=sm_103a']
+# (no -ftz=true or -use_fast_math: the FP32 spreading rounds on the denormal grid)
 FLAGS = ['-O3', '-lineinfo', '-std=c++17', '-Xcompiler', '-fPIC', '-Xcompiler', '-fno-strict-aliasing']
 
 

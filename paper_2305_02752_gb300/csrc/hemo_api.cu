@@ -501,9 +501,10 @@ int finalize_impl(hemo_sim *s) {
         // gather, consecutive items in the triangle and edge passes) load
         // nearby shared-memory records (measured: membrane kernel 1163 ->
         // 976 us on the pipe against the earlier order that spread a warp
-        // over far-apart mesh parts, made for scattering atomics).  The FP64
-        // adjoint, which still scatters with atomics, walks the same tables
-        // with a coprime stride (MeshDev::tstride, estride).
+        // over far-apart mesh parts, made for scattering atomics).  The FP32
+        // adjoint of meshes too large for its gather, which scatters with
+        // shared-memory atomics, walks the same tables with a coprime stride
+        // (MeshDev::tstride, estride).
         std::vector<int> edge_p(4 * (size_t)m.ne), tri_p(3 * (size_t)m.nt), etri_p(2 * (size_t)m.ne);
         std::vector<R> invL0(m.ne), th0(m.ne);
         std::vector<R> At0_p(m.nt);
@@ -694,9 +695,9 @@ int finalize_impl(hemo_sim *s) {
     }
     const size_t smem = cell_smem_bytes<R>(s->max_nv, s->max_nt, s->max_ne);
     if (smem > 48 * 1024) HEMO_CU(set_cell_smem_limit<R>(smem));
-    const size_t smem_adj = cell_adjoint_smem_bytes<R>(s->max_nv, s->max_nt);
-    if (smem_adj > 48 * 1024) HEMO_CU(set_cell_adjoint_smem_limit<R>(smem_adj));
     if (std::is_same<R, float>::value) {
+        const size_t smem_adj = cell_adjoint_smem_bytes(s->max_nv, s->max_nt);
+        if (smem_adj > 48 * 1024) HEMO_CU(set_cell_adjoint_smem_limit(smem_adj));
         const size_t gs = cell_adjoint_gather_bytes(s->max_nv, s->max_nt, s->max_ne);
         if (gs > 48 * 1024 && gs <= CELL_ADJ_GATHER_MAX_SMEM) HEMO_CU(set_cell_adjoint_gather_smem_limit(gs));
     }
@@ -1136,7 +1137,7 @@ int hemo_velocity_set(int32_t *c, double *w) {
 // needs 16-byte aligned rows (bulk copies), rows of at most 1024 nodes (a
 // stage's range) and at least two stages of the ring in shared memory (one
 // CTA per SM takes up to four), and is for 2-byte storage only.  By default
-// it is used for rows of at least 512 nodes (pipe: 523 and 568 us against 754
+// it is used for rows of at least 512 nodes (pipe: 513 and 562 us against 754
 // and 860 per node), and for rows of at least 64 where the tiles are at least
 // 13 per SM, so that the ring's start and end are small against the rest: 128 x
 // 128 x 512 channel 141 and 153 us against 171 and 198 per node, 128^3 47.4 and

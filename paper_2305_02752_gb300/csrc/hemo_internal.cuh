@@ -307,13 +307,15 @@ template <typename R> void launch_restore_natural(const View<R> &v, int precisio
 template <typename R> void launch_adj_moments(const View<R> &v, const AdjView<R> &a, cudaStream_t st);
 template <typename R> void launch_adj_collide(const View<R> &v, const AdjView<R> &a, cudaStream_t st);
 template <typename R> void launch_cell_adjoint(const View<R> &v, const AdjView<R> &a, cudaStream_t st);
-template <typename R> cudaError_t set_cell_adjoint_smem_limit(size_t bytes);
-inline int adjoint_chunks(int items) { return (items + 63) / 64; }  // CTAs of 64 items (FP64)
+cudaError_t set_cell_adjoint_smem_limit(size_t bytes);  // (FP32; the FP64 kernels use none)
+// FP64 membrane adjoint: items (triangles, edges) per CTA, and CTAs for a mesh's
+constexpr int ADJ_ITEMS = 64;
+inline int adjoint_chunks(int items) { return (items + ADJ_ITEMS - 1) / ADJ_ITEMS; }
 // cells whose triangle records (64 bytes each) fill 64 MB: 819 red cells, 16,000 CTAs
 inline int adjoint_batch(int ncell, int max_nt) {
     return std::max(1, std::min(ncell, (64 << 20) / (64 * std::max(max_nt, 1))));
 }
-template <typename R> size_t cell_adjoint_smem_bytes(int max_nv, int max_nt) { return (9 * (size_t)max_nv + 8 * (size_t)max_nt) * sizeof(R); }
+inline size_t cell_adjoint_smem_bytes(int max_nv, int max_nt) { return (9 * (size_t)max_nv + 8 * (size_t)max_nt) * sizeof(float); }
 // FP32 gather form of the membrane adjoint: positions, direction, triangle
 // and edge records with their derivatives, 16 bytes each; used while it fits
 // the largest shared-memory allocation of a CTA

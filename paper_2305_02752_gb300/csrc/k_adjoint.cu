@@ -118,9 +118,9 @@ __device__ __forceinline__ void pull_adjoint(const View<R> &v, const AdjView<R> 
 
 // transpose of streaming (pull, with the moments term of the pulled
 // population) and of the collision at fluid node n
-constexpr int ADJ_NT = 128;  // (FP64, 32^3 box: 25.7 us against 27.0 with 256; FP32 the same)
+constexpr int ADJ_COLLIDE_NT = 128;  // (FP64, 32^3 box: 25.7 us against 27.0 with 256; FP32 the same)
 template <typename R>
-__global__ void __launch_bounds__(ADJ_NT) adj_collide_kernel(View<R> v, AdjView<R> a) {
+__global__ void __launch_bounds__(ADJ_COLLIDE_NT) adj_collide_kernel(View<R> v, AdjView<R> a) {
     wait_previous();
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     R acc[4] = {R(0), R(0), R(0), R(0)};  // wall-velocity scale, g_x, g_y, g_z
@@ -239,7 +239,7 @@ void launch_adj_moments(const View<R> &v, const AdjView<R> &a, cudaStream_t st) 
 
 template <typename R>
 void launch_adj_collide(const View<R> &v, const AdjView<R> &a, cudaStream_t st) {
-    launch_next(adj_collide_kernel<R>, nblocks(v.N, ADJ_NT), ADJ_NT, 0, st, v, a);
+    launch_next(adj_collide_kernel<R>, nblocks(v.N, ADJ_COLLIDE_NT), ADJ_COLLIDE_NT, 0, st, v, a);
 }
 
 #define HEMO_INST(R)                                                                  \

@@ -478,24 +478,18 @@ __device__ __forceinline__ void stage_tile(const View<R> &v, const R *A, const i
 // contribution, is below the FP32 rounding of sums of that size.  FP64:
 // 64-bit integers with 2^62 in place of 2^30 (quantum max|F| n 2^-65, below
 // FP64 rounding).
-template <typename R> struct TileAcc {
-    static constexpr int E = 61;  // log2 of the bound minus one
-};
-template <> struct TileAcc<float> {
-    static constexpr int E = 29;
-};
+constexpr int ACC_F32 = 29, ACC_F64 = 61;  // log2 of the bound on a sum, minus one
 constexpr int SPREAD_CAP = 352, SP64_THREADS = 512;  // vertices staged at a time, threads (FP64)
 
-// the scale of a component from its largest force; 0 (and the numeric
+// FP64: the scale of a component from its largest force; 0 (and the numeric
 // status) for forces that are not finite
-template <typename R>
-__device__ __forceinline__ R tile_scale(R fmax_abs, int n, unsigned *status) {
-    const R bound = fmax_abs * R(n) * R(0.125);
-    if (!(bound <= R(3.0e38))) {
+__device__ __forceinline__ double tile_scale(double fmax_abs, int n, unsigned *status) {
+    const double bound = fmax_abs * n * 0.125;
+    if (!(bound <= 3.0e38)) {
         atomicOr(status, ST_NUMERIC);
-        return R(0);
+        return 0.0;
     }
-    return bound > R(0) ? ldexp(R(1), min(TileAcc<R>::E - ilogb(bound), 120)) : R(0);
+    return bound > 0.0 ? ldexp(1.0, min(ACC_F64 - ilogb(bound), 120)) : 0.0;
 }
 
 // FP32.  Two lanes per vertex, lane h adding the stencil's x nodes 2h and
@@ -644,7 +638,7 @@ __global__ void __launch_bounds__(SP_CHUNK, 6) spread_tile_f32_kernel(View<float
 #pragma unroll
         for (int o = 1; o < NW; o <<= 1) mm = max(mm, __shfl_xor_sync(0xffffffffu, mm, o));
         const float bound = __uint_as_float(mm) * (float)n * 0.125f;
-        int x = min(TileAcc<float>::E + 127 - (int)(__float_as_uint(bound) >> 23), 120);
+        int x = min(ACC_F32 + 127 - (int)(__float_as_uint(bound) >> 23), 120);
         if (!(bound <= 3.0e38f)) {
             if (tid < 3 * NW) atomicOr(v.status, ST_NUMERIC);
             x = NO_SCALE;
@@ -743,7 +737,7 @@ __global__ void __launch_bounds__(SP_CHUNK, 6) spread_tile_f32_kernel(View<float
 // Bound by the FP64 pipe (19 cycles per warp instruction), then by the shared
 // atomics: the four weights along x are w0, 1/2 - w3, 1/2 - w0, w3, so a row
 // takes three conversions and two products, the other two nodes a subtraction
-// of integers; the 64-bit sums are kept as two words with the carry taken from
+// of integers (one quantum of rounding instead of a half); the 64-bit sums are kept as two words with the carry taken from
 // the first atomic (4 cycles per warp instruction; a 64-bit shared atomic takes
 // 12).  48 x 39 x 64 channel with 30 cells: 65 ->
 // 50 us; 32^3 box with one cell: 16.7 -> 11.7 us.  Threads for a whole SM's
@@ -1105,12 +1099,12 @@ __global__ void __launch_bounds__(256) hold_bins_kernel(View<R> v) {
 // the weights are computed, a thread per vertex and axis) and by the FP64 pipe:
 // 32^3 box with one cell 20.5 -> 16.4 us, 48 x 39 x 64 channel with 30 cells
 // 45 -> 35 us.
-constexpr int InterpCap = 32;  // vertices per chunk
+constexpr int INTERP_CAP = 32;  // vertices per chunk
 template <typename R, int INTEG>
 __global__ void __launch_bounds__(256) interpolate_kernel(View<R> v, int parts) {
     wait_previous();
     drop_dead_lines(v);
-    constexpr int CAP = InterpCap;
+    constexpr int CAP = INTERP_CAP;
     const int k = bin_of(v, blockIdx.x % v.nbins), part = blockIdx.x / v.nbins;  // CTA part takes chunks part, part + parts, ...
     const int s = v.start[k], e = v.start[k + 1];
     if (s + part * CAP >= e) return;
@@ -1176,9 +1170,10 @@ __global__ void __launch_bounds__(256) interpolate_kernel(View<R> v, int parts) 
 // 8: four cycles per load instead of about ten.  The fullest class sets the
 // number of lanes (1.39 times the vertices on the pipe).
 //
-// Bound by shared-memory wavefronts (75 M -> 46 M on the 128 x 128 x 512 vessel,
-// 81 % of the kernel's cycles).  Vessel 238 -> 194 us, 1000 x 208 x 208 pipe 953
-// -> 776 us; five CTAs per SM 785, seven 806 (spills).
+// Bound by shared-memory wavefronts (62.5 M -> 47.3 M on the 128 x 128 x 512
+// vessel, 77 % of the kernel's cycles; conflicts 29.8 M -> 8.9 M).  Vessel 238 ->
+// 194 us, 1000 x 208 x 208 pipe 953 -> 776 us; five CTAs per SM 785, seven 806
+// (spills).
 //
 // Staging.  With a tensor map of u (4-D: x, y, z, component) one thread
 // copies the box x in [ox - 4, ox + 12), y in [oy - 1, oy + 10), z in
@@ -1438,12 +1433,12 @@ __device__ __forceinline__ void peskin4_d(R t, R *w, R *dw) {
 // grad_X w = (w'_x w_y w_z, w_x w'_y w_z, w_x w_y w'_z).  Either output may
 // be null (B is then unused).  out_grad may alias B: a vertex reads B[v]
 // before its own write.
-template <typename R> struct VfStage { static constexpr int CAP = sizeof(R) == 8 ? 16 : 128; };
+constexpr int VF_CAP = 16;  // vertices per chunk
 template <typename R>
 __global__ void __launch_bounds__(256) vertex_field_kernel(View<R> v, const R *A, const R *B, R *out_grad,
                                                            R *out_interp, int parts) {
     wait_previous();
-    constexpr int CAP = VfStage<R>::CAP;
+    constexpr int CAP = VF_CAP;
     const int k = bin_of(v, blockIdx.x % v.nbins), part = blockIdx.x / v.nbins;  // CTA part takes chunks part, part + parts, ...
     const int s = v.start[k], e = v.start[k + 1];
     if (s + part * CAP >= e) return;
@@ -1676,7 +1671,11 @@ template <typename R>
 void launch_spread(const View<R> &v, cudaStream_t st) {
     if constexpr (std::is_same<R, float>::value) launch_next(spread_tile_f32_kernel, v.nbins, SP_CHUNK, 0, st, v);
     else launch_next(spread_tile_kernel, 3 * v.nbins, SP64_THREADS, 0, st, v);
-    // (across a periodic edge the tiles' positions are those of whole blocks only)
+    // (across a periodic edge the tiles' positions are those of whole blocks only;
+    // the general gather for every block of such a lattice: FP32 channel 128 x 64 x
+    // 253 288 us a step, 128 x 64 x 256 269.  For the edge layers alone, with
+    // spread_gather3_kernel for the rest, 284, but the second launch costs small
+    // lattices more: 61 x 64 x 253 151 -> 155, 45 x 39 x 61 in FP64 186 -> 196 us)
     const int dims[3] = {v.nx, v.ny, v.nz};
     bool regular = true;
     for (int d = 0; d < 3; ++d) regular &= v.nb[d] >= 3 && (!v.per[d] || dims[d] % BLK == 0);

@@ -259,7 +259,9 @@ __global__ void __launch_bounds__(256) le_interp_kernel(View<R> v) {
 }
 
 __global__ void le_advance_kernel(long long *n) {
-    wait_previous(); *n += 1; }
+    wait_previous();
+    *n += 1;
+}
 
 }  // namespace
 

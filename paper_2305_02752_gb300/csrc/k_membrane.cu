@@ -1,6 +1,6 @@
-// Membrane mechanics, one CTA per cell or, with few cells, a cluster (Sec. 2.3: F_total = F_link + F_bend
-// + F_area + F_volume; vertices are Lagrangian points of a triangulated
-// membrane).
+// Membrane mechanics, one CTA per cell or, with few cells, a cluster (Sec. 2.3:
+// F_total = F_link + F_bend + F_area + F_volume; vertices are Lagrangian points
+// of a triangulated membrane).
 //
 // A CTA stages its cell's vertex offsets in shared memory, re-bases the cell
 // (centroid += mean offset, offsets -= mean, so the FP32 offsets stay small
@@ -8,11 +8,10 @@
 // the triangles in FP64, and accumulates the four force terms per vertex in
 // shared memory before one coalesced write.  The edge and triangle tables
 // arrive in a processing order sorted on the host by smallest vertex id, so
-// that the lanes of a warp load nearby shared-memory records; the FP32 adjoint of
-// meshes too large for the gather, which scatters with shared-memory atomics,
-// walks them with a coprime stride instead (lanes on far-apart mesh parts).
-// Energies (forms documented in
-// hemo.h):
+// that the lanes of a warp load nearby shared-memory records; the FP32 adjoint
+// of meshes too large for the gather, which scatters with shared-memory
+// atomics, walks them with a coprime stride instead (lanes on far-apart mesh
+// parts).  Energies (forms documented in hemo.h):
 //   link   K L0 [eps^2/2 - 1/2 ln(1 - eps^2/m^2)],   eps = (L - L0)/L0
 //   bend   1/2 kb (theta - theta0)^2, theta = signed angle between the
 //          outward normals of the two triangles of an edge
@@ -930,11 +929,10 @@ __global__ void __launch_bounds__(NT, CellMinBlocks<R, NT>::B) cell_adjoint_kern
 // with the records for 96 us.  32^3 box, one cell: 109 -> 8.4 + 17.7 + 2.3 us.
 // Many cells go through the three kernels adjoint_batch() at a time, from cell
 // c0: their records would take 1.6 GB for the 19,600 cells of the pipe.
-constexpr int ADJ_NT = 64;  // items per CTA
 __device__ __forceinline__ V3<Dual<double>> vertex_dual(const View<double> &v, const AdjView<double> &a, size_t i) {
     return dld3(v.off + 3 * i, a.lamFv + 3 * i);
 }
-__global__ void __launch_bounds__(ADJ_NT) adjoint_records_kernel(View<double> v, AdjView<double> a, int c0, int chunks) {
+__global__ void __launch_bounds__(ADJ_ITEMS) adjoint_records_kernel(View<double> v, AdjView<double> a, int c0, int chunks) {
     wait_previous();
     using D = Dual<double>;
     const int lc = blockIdx.x / chunks, c = c0 + lc, chunk = blockIdx.x % chunks;
@@ -942,7 +940,7 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_records_kernel(View<double> v,
     const size_t first = v.cell_first[c];
     __shared__ double scratch[4][32];
     Acc<double> av[4];  // A, dA, V, dV
-    const int t = chunk * ADJ_NT + threadIdx.x;
+    const int t = chunk * ADJ_ITEMS + threadIdx.x;
     if (t < m.nt) {
         const int4 T = __ldg(m.tri4 + t);
         const V3<D> p0 = vertex_dual(v, a, first + T.x), p1 = vertex_dual(v, a, first + T.y), p2 = vertex_dual(v, a, first + T.z);
@@ -964,7 +962,7 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_records_kernel(View<double> v,
     if (threadIdx.x < 4) a.tri_part[4 * ((size_t)lc * chunks + chunk) + threadIdx.x] = scratch[threadIdx.x][31];
 }
 
-__global__ void __launch_bounds__(ADJ_NT) adjoint_terms_kernel(View<double> v, AdjView<double> a, int c0, int chunks, int echunks) {
+__global__ void __launch_bounds__(ADJ_ITEMS) adjoint_terms_kernel(View<double> v, AdjView<double> a, int c0, int chunks, int echunks) {
     wait_previous();
     using D = Dual<double>;
     using R = double;
@@ -979,7 +977,7 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_terms_kernel(View<double> v, A
     Acc<R> th[2];  // lamFv . unit-modulus forces: link and bend, or area and volume
     const bool edges = chunk < echunks;
     if (edges) {
-        const int e = chunk * ADJ_NT + threadIdx.x;
+        const int e = chunk * ADJ_ITEMS + threadIdx.x;
         if (e < m.ne) {
             const int4 E = __ldg(reinterpret_cast<const int4 *>(m.edge) + e);
             const int2 T = __ldg(reinterpret_cast<const int2 *>(m.etri) + e);
@@ -1021,7 +1019,7 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_terms_kernel(View<double> v, A
         }
         __syncthreads();
         const D ua = {cuv[0], cuv[1]}, uv = {cuv[2], cuv[3]};
-        const int t = (chunk - echunks) * ADJ_NT + threadIdx.x;
+        const int t = (chunk - echunks) * ADJ_ITEMS + threadIdx.x;
         if (t < m.nt) {
             const int4 T = __ldg(m.tri4 + t);
             const int j[3] = {T.x, T.y, T.z};
@@ -1378,27 +1376,23 @@ void launch_cell_adjoint(const View<R> &v, const AdjView<R> &a, cudaStream_t st)
         const int batch = adjoint_batch(v.ncell, v.max_nt);
         for (int c0 = 0; c0 < v.ncell; c0 += batch) {
             const int n = std::min(batch, v.ncell - c0);
-            launch_next(adjoint_records_kernel, n * chunks, ADJ_NT, 0, st, v, a, c0, chunks);
-            launch_next(adjoint_terms_kernel, n * (chunks + echunks), ADJ_NT, 0, st, v, a, c0, chunks, echunks);
+            launch_next(adjoint_records_kernel, n * chunks, ADJ_ITEMS, 0, st, v, a, c0, chunks);
+            launch_next(adjoint_terms_kernel, n * (chunks + echunks), ADJ_ITEMS, 0, st, v, a, c0, chunks, echunks);
             launch_next(adjoint_add_kernel, (unsigned)((3LL * n * v.max_nv + 255) / 256), 256, 0, st, v, a, c0, n);
         }
     } else {  // meshes whose gather records do not fit
-        const size_t smem = cell_adjoint_smem_bytes<R>(v.max_nv, v.max_nt);
+        const size_t smem = cell_adjoint_smem_bytes(v.max_nv, v.max_nt);
         const int slices = std::max(1, std::min(32, v.nsm / v.ncell));
         if (slices == 1 && cell_wide(v)) launch_next(cell_adjoint_kernel<R, CellMax<R>::T>, v.ncell, CellMax<R>::T, smem, st, v, a, 1);
         else launch_next(cell_adjoint_kernel<R, 256>, v.ncell * slices, 256, smem, st, v, a, slices);
     }
 }
 
-template <typename R>
 cudaError_t set_cell_adjoint_smem_limit(size_t bytes) {
-    if constexpr (std::is_same<R, double>::value) return cudaSuccess;  // (its kernels use none)
-    else {
-    cudaError_t e = cudaFuncSetAttribute(cell_adjoint_kernel<R, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess && CellMax<R>::T != 256)
-        e = cudaFuncSetAttribute(cell_adjoint_kernel<R, CellMax<R>::T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = cudaFuncSetAttribute(cell_adjoint_kernel<float, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(cell_adjoint_kernel<float, CellMax<float>::T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     return e;
-    }
 }
 
 cudaError_t set_cell_adjoint_gather_smem_limit(size_t bytes) {
@@ -1416,8 +1410,6 @@ void launch_deformation_loss(const View<R> &v, const double *c0, double *cell_lo
 
 template void launch_cell_adjoint<double>(const View<double> &, const AdjView<double> &, cudaStream_t);
 template void launch_cell_adjoint<float>(const View<float> &, const AdjView<float> &, cudaStream_t);
-template cudaError_t set_cell_adjoint_smem_limit<double>(size_t);
-template cudaError_t set_cell_adjoint_smem_limit<float>(size_t);
 template void launch_deformation_loss<double>(const View<double> &, const double *, double *, double *, cudaStream_t);
 template void launch_deformation_loss<float>(const View<float> &, const double *, double *, float *, cudaStream_t);
 template void launch_cell_forces<double>(const View<double> &, int, double *, cudaStream_t);
