@@ -28,7 +28,7 @@ constexpr unsigned ST_BOUNDS = 8u;   // an index failed its check (bounds-checke
 
 // The bounds-checked build (HEMO_BOUNDS_CHECK=1, libhemo_checked.so) tests
 // the data-driven indices of the vertex, bin and membrane kernels (vertex
-// ids read from the bin order, cell ids, mesh-table entries, bin slots)
+// ids and bins read from their lists, cell ids, mesh-table entries, bin slots)
 // before use: a failed test sets ST_BOUNDS in the status word and the
 // access is skipped.  In the default build index_ok is the constant true
 // and the tests compile away.

@@ -404,7 +404,8 @@ __device__ __forceinline__ int neighbour_blocks(int b, int nb, int n, int period
     return cnt;
 }
 
-// The b-th bin of a vertex kernel's grid: by size where the list is kept.
+// The b-th bin of a vertex kernel's grid: by size where the list is kept (-1 in
+// the bounds-checked build for an entry that fails its check).
 // Bins hold from none to several times the mean, and a grid of a few CTAs per
 // SM ends when its largest does: with the largest first, 48 x 39 x 64 channel,
 // FP64 interpolation 33 -> 30 us; 64 x 64 x 256 channel, FP32 spreading 27.4 ->
@@ -413,7 +414,8 @@ __device__ __forceinline__ int neighbour_blocks(int b, int nb, int n, int period
 // less.
 template <typename R>
 __device__ __forceinline__ int bin_of(const View<R> &v, int b) {
-    return v.order ? v.order[b] : b;
+    const int k = v.order ? v.order[b] : b;
+    return index_ok(k >= 0 && k < v.nbins, v.status) ? k : -1;
 }
 
 // FP64 vertex kernels: anchors and weights of one chunk of a bin, staged in
@@ -581,6 +583,7 @@ __device__ __forceinline__ void spread_item(int *first, int s, const float (&F)[
 __global__ void __launch_bounds__(SP_CHUNK, 6) spread_tile_f32_kernel(View<float> v) {
     wait_previous();
     const int k = bin_of(v, blockIdx.x);
+    if (HEMO_BOUNDS_CHECK && k < 0) return;
     const int s = v.start[k], e = v.start[k + 1], n = e - s;
     if (n == 0) return;
     __shared__ __align__(16) int tile[3 * SP_N];
@@ -752,6 +755,7 @@ __global__ void __cluster_dims__(3, 1, 1) __launch_bounds__(SP64_THREADS) spread
     constexpr int CAP = SPREAD_CAP, W = 10;  // 2 w0 and 2 w3 along x, four weights along y and z
     const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     const int k = bin_of(v, blockIdx.x / 3), d = (int)cluster.block_rank();
+    if (HEMO_BOUNDS_CHECK && k < 0) return;
     const int s = v.start[k], e = v.start[k + 1];
     if (s == e) return;  // (the whole cluster)
     __shared__ unsigned lo[TILE_SMEM], hi[TILE_SMEM];
@@ -1106,6 +1110,7 @@ __global__ void __launch_bounds__(256) interpolate_kernel(View<R> v, int parts) 
     drop_dead_lines(v);
     constexpr int CAP = INTERP_CAP;
     const int k = bin_of(v, blockIdx.x % v.nbins), part = blockIdx.x / v.nbins;  // CTA part takes chunks part, part + parts, ...
+    if (HEMO_BOUNDS_CHECK && k < 0) return;
     const int s = v.start[k], e = v.start[k + 1];
     if (s + part * CAP >= e) return;
     __shared__ R tile[3][TILE_SMEM];
@@ -1204,6 +1209,7 @@ __global__ void __launch_bounds__(IT_CHUNK, 6) interpolate_v4_kernel(View<float>
     wait_previous();
     drop_dead_lines(v);
     const int k = bin_of(v, blockIdx.x);
+    if (HEMO_BOUNDS_CHECK && k < 0) return;
     const int s = v.start[k], e = v.start[k + 1];
     if (s == e) return;
     __shared__ __align__(128) unsigned char tile_raw[INTERP_SMEM];
@@ -1440,6 +1446,7 @@ __global__ void __launch_bounds__(256) vertex_field_kernel(View<R> v, const R *A
     wait_previous();
     constexpr int CAP = VF_CAP;
     const int k = bin_of(v, blockIdx.x % v.nbins), part = blockIdx.x / v.nbins;  // CTA part takes chunks part, part + parts, ...
+    if (HEMO_BOUNDS_CHECK && k < 0) return;
     const int s = v.start[k], e = v.start[k + 1];
     if (s + part * CAP >= e) return;
     __shared__ R tile[3][TILE_SMEM];
@@ -1513,6 +1520,7 @@ __global__ void __launch_bounds__(256) vertex_field_v4_kernel(View<float> v, con
                                                               float *out_grad, float *out_interp) {
     wait_previous();
     const int k = bin_of(v, blockIdx.x);
+    if (HEMO_BOUNDS_CHECK && k < 0) return;
     const int s = v.start[k], e = v.start[k + 1];
     if (s == e) return;
     __shared__ float4 tile[TILE_SMEM];

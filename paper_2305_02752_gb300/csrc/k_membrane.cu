@@ -569,6 +569,7 @@ __global__ void __launch_bounds__(SliceThreads<R>::T, 1) cell_slices_kernel(View
     // latency)
     const int tf = t0 + (int)threadIdx.x, ef = e0 + (int)threadIdx.x;
     const int ti = tf < t1 ? __ldg(m.sl_items + tf) : -1, ei = mode == 0 && ef < e1 ? __ldg(m.sl_items + ef) : -1;
+    auto item_ok = [&](int k, int n) { return index_ok(k >= 0 && k < n, v.status); };
 
     // mean offset and re-base, as in cell_kernel
     constexpr int KC = 4;
@@ -591,8 +592,8 @@ __global__ void __launch_bounds__(SliceThreads<R>::T, 1) cell_slices_kernel(View
     int4 Tf = make_int4(0, 0, 0, 0), Ef = Tf;
     int2 Uf = make_int2(0, 0);
     R lf = R(0), hf = R(0);
-    if (ti >= 0) Tf = __ldg(m.tri4 + (ti >> 1));
-    if (ei >= 0) {
+    if (ti >= 0 && item_ok(ti >> 1, m.nt)) Tf = __ldg(m.tri4 + (ti >> 1));
+    if (ei >= 0 && item_ok(ei, m.ne)) {
         Ef = __ldg(reinterpret_cast<const int4 *>(m.edge) + ei);
         Uf = __ldg(reinterpret_cast<const int2 *>(m.etri) + ei);
         lf = __ldg(m.invL0 + ei);
@@ -650,6 +651,7 @@ __global__ void __launch_bounds__(SliceThreads<R>::T, 1) cell_slices_kernel(View
     Acc<R> sum[2];
     for (int q = tf; q < t1; q += NT) {
         const int id = q == tf ? ti : __ldg(m.sl_items + q), t = id >> 1;
+        if (!item_ok(t, m.nt)) continue;
         const int4 T = q == tf ? Tf : __ldg(m.tri4 + t);
         if (!tri_ok(m, T, v.status)) continue;
         R area, vol;
@@ -692,8 +694,9 @@ __global__ void __launch_bounds__(SliceThreads<R>::T, 1) cell_slices_kernel(View
     if (mode == 0) {
         for (int q = ef; q < e1; q += NT) {
             int e = ei;
+            if (q != ef) e = __ldg(m.sl_items + q);
+            if (!item_ok(e, m.ne)) continue;
             if (q != ef) {
-                e = __ldg(m.sl_items + q);
                 Ef = __ldg(reinterpret_cast<const int4 *>(m.edge) + e);
                 Uf = __ldg(reinterpret_cast<const int2 *>(m.etri) + e);
                 lf = __ldg(m.invL0 + e);
