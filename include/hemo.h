@@ -43,7 +43,8 @@ enum hemo_status {
     HEMO_ERR_ARG = -1,      /* invalid argument (null, size, range)           */
     HEMO_ERR_OOM = -2,      /* device allocation failed                        */
     HEMO_ERR_CUDA = -3,     /* a CUDA call or kernel launch failed             */
-    HEMO_ERR_NUMERIC = -4,  /* non-finite or |u| > 0.3 velocity seen on device */
+    HEMO_ERR_NUMERIC = -4,  /* non-finite or |u| > 0.3 velocity, or a force that
+                               is not finite, seen on the device              */
     HEMO_ERR_DOMAIN = -5,   /* a vertex left the domain across a wall axis     */
     HEMO_ERR_STATE = -6     /* call not valid in the simulation's state        */
 };
