@@ -159,24 +159,17 @@ __global__ void __launch_bounds__(NODE_BX * NODE_BY) le_stream_kernel(View<R> v)
 }
 
 // the layer c (-1..2 around the anchor) of a vertex's stencil: node z, x
-// anchor and fraction, velocity offset of the image
+// anchor and fraction, velocity offset of the image.  The layer lies in the
+// k-th box above (below for k < 0): 0 or +-1 for cells at the plane, any
+// number for a lattice lower than the stencil and for vertices thrown far out
+// by a run that blows up, whose layers have to be nodes of the lattice too
 template <typename R>
 __device__ __forceinline__ void le_layer(const View<R> &v, double D, double X, int jz0, int c, int &zn, int &jx, R &tx,
                                         R &du) {
-    int jz = jz0 + c;
-    double xp = X;
-    du = R(0);
-    if (jz >= v.nz) {
-        jz -= v.nz;
-        xp = X - D;
-        du = R(v.le_U);
-    } else if (jz < 0) {
-        jz += v.nz;
-        xp = X + D;
-        du = R(-v.le_U);
-    }
-    const double fl = floor(xp);
-    zn = jz;
+    const int jz = jz0 + c, k = jz >= 0 ? jz / v.nz : -1 - (-1 - jz) / v.nz;
+    const double xp = X - k * D, fl = floor(xp);
+    du = R(k * v.le_U);
+    zn = jz - k * v.nz;
     jx = (int)fl;
     tx = R(xp - fl);
 }
