@@ -661,6 +661,7 @@ int finalize_impl(hemo_sim *s) {
         d.V0 = m.V0;
         d.K = R(m.k_link * m.kbt / m.persistence);
         d.m2 = R(m.max_strain * m.max_strain);
+        d.lmax = R(std::min(4096.0, (1.0 + m.max_strain) * *std::max_element(m.L0.begin(), m.L0.end())));
         d.kb = R(m.k_bend * m.kbt);
         d.k_area = m.k_area;
         d.k_volume = m.k_volume;

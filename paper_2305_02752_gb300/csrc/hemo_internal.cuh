@@ -125,6 +125,7 @@ template <typename R> struct MeshDev {
     double A0, V0;
     R K;                // k_link * kbt / persistence
     R m2;               // max_strain^2
+    R lmax;             // longest edge at the maximum strain (at most 4096 nodes)
     R kb;               // k_bend * kbt
     double k_area, k_volume;
     double c_area, c_volume;  // 1/2 k_area / A0^2, k_volume / (6 V0^2)

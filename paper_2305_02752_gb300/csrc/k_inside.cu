@@ -67,6 +67,13 @@ __global__ void __launch_bounds__(256) inside_toggle_kernel(View<R> v) {
         for (int d = 0; d < 2; ++d) {
             lo[d] = fmin(P[0][d], fmin(P[1][d], P[2][d]));
             hi[d] = fmax(P[0][d], fmax(P[1][d], P[2][d]));
+            // a triangle wider than the box whose links are past their maximum
+            // strain belongs to a run that blew up: reported instead of walking its
+            // columns, which may be any number (and beyond an int's range endless)
+            if (!(lo[d] > R(-1e9) && hi[d] < R(1e9) && hi[d] - lo[d] <= fmax(R(dims[d]), m.lmax))) {
+                atomicOr(v.status, ST_NUMERIC);
+                return;
+            }
         }
         const int jx0 = (int)ceil(lo[0]), jx1 = (int)floor(hi[0]);
         const int jy0 = (int)ceil(lo[1]), jy1 = (int)floor(hi[1]);
