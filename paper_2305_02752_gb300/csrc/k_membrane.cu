@@ -1352,11 +1352,23 @@ void launch_cell_forces(const View<R> &v, int mode, double *stats, cudaStream_t 
     else launch_next(cell_kernel<R, 256>, v.ncell, 256, smem, st, v, mode, stats);
 }
 
+// Allows a kernel `bytes` of dynamic shared memory: the largest amount beside its
+// own, the same for every simulation, as the attribute is the process's and a
+// simulation with a smaller mesh must not lower it for another.  More than that
+// is refused by the runtime.
+template <typename K>
+cudaError_t allow_smem(K *kernel, size_t bytes) {
+    cudaFuncAttributes fa;
+    const cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)std::max(bytes, (size_t)227 * 1024 - fa.sharedSizeBytes));
+}
+
 template <typename R>
 cudaError_t set_cell_smem_limit(size_t bytes) {
-    cudaError_t e = cudaFuncSetAttribute(cell_kernel<R, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess && CellMax<R>::T != 256)
-        e = cudaFuncSetAttribute(cell_kernel<R, CellMax<R>::T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_smem(cell_kernel<R, 256>, bytes);
+    if (e == cudaSuccess && CellMax<R>::T != 256) e = allow_smem(cell_kernel<R, CellMax<R>::T>, bytes);
     return e;
 }
 
@@ -1392,16 +1404,14 @@ void launch_cell_adjoint(const View<R> &v, const AdjView<R> &a, cudaStream_t st)
 }
 
 cudaError_t set_cell_adjoint_smem_limit(size_t bytes) {
-    cudaError_t e = cudaFuncSetAttribute(cell_adjoint_kernel<float, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(cell_adjoint_kernel<float, CellMax<float>::T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_smem(cell_adjoint_kernel<float, 256>, bytes);
+    if (e == cudaSuccess) e = allow_smem(cell_adjoint_kernel<float, CellMax<float>::T>, bytes);
     return e;
 }
 
 cudaError_t set_cell_adjoint_gather_smem_limit(size_t bytes) {
-    cudaError_t e = cudaFuncSetAttribute(cell_adjoint_gather_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(cell_adjoint_gather_kernel<CellMax<float>::T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_smem(cell_adjoint_gather_kernel<256>, bytes);
+    if (e == cudaSuccess) e = allow_smem(cell_adjoint_gather_kernel<CellMax<float>::T>, bytes);
     return e;
 }
 
